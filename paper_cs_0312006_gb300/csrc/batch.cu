@@ -189,9 +189,8 @@ __device__ __forceinline__ void job_pass(const BatchJob& j, int c, uint32_t t, u
         // words share it and take the five-call draws together
         const uint32_t items = j.rows * (((uint32_t)j.W + 31u) >> 5);
         const uint32_t rgroups = packed_row_groups((uint32_t)j.W);
-        for (uint32_t it = rank; it < items; it += nthr)
-            packed_word<DIMS, MEASURE, NC, RULE, RULE != kRuleMultiHit>(a, it, e_acc, m_acc,
-                                                                        rgroups);
+            for (uint32_t it = rank; it < items; it += nthr)
+            packed_word<DIMS, MEASURE, NC, RULE>(a, it, e_acc, m_acc, rgroups);
     }
 }
 

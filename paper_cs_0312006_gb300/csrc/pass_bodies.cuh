@@ -20,9 +20,22 @@
 
 #include <cstdint>
 
+#include <type_traits>
+#include <utility>
+
 #include "ising_device.cuh"
 
 namespace ising {
+
+// f(std::integral_constant<int, I>) for I = 0..N-1, unrolled.
+template <int N, typename F, int... I>
+__device__ __forceinline__ void static_for(F&& f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, typename F>
+__device__ __forceinline__ void static_for(F&& f) {
+    static_for<N>(f, std::make_integer_sequence<int, N>{});
+}
 
 constexpr uint32_t kByteBit1 = 0x02020202u;
 constexpr uint32_t kByteBit7 = 0x80808080u;
@@ -573,111 +586,131 @@ __device__ __forceinline__ uint32_t site_threshold(const Digits& k, int b, const
     return d2 ? hi : lo;
 }
 
+// Thresholds of a rule: the Metropolis dims, or the heat bath's 2 dims + 1.
+template <int DIMS, int RULE>
+constexpr int kThresholds = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
+
+// What bounds the drawing passes is instructions issued.  Measured on the
+// generator and these tests alone (cycles per scheduler and Philox call, any
+// occupancy from two to eight CTAs per SM): a 32x32 -> 64-bit product holds the
+// issue port ~3.6 cycles, a 32-bit multiply-add 2 and everything else 1,
+// whichever pipe it runs on.  Ten rounds cost 82.5.  Selecting each site's
+// threshold and comparing took 33 more (as compiled); every draw against every
+// threshold with mark_below takes 15 (2D), and choose_answer picks for 32 sites
+// at once.  2D L = 8192: 29.1 -> 24.6 us per pass (1.36e12 site updates/s).
+// Tests as saturating fp32 multiply-adds, off the integer pipes, took 26: a
+// multiply-add costs an issue slot like a compare.
+//
+// The draws of 16 sites (one half of a packed word) against all N thresholds:
+// bit 16 HALF + b of A[n] is set iff site b's draw lies below threshold n.
+// The word's first bit is half index 4 g0 + M (M = 0..3: where the row starts
+// inside a Philox group), so site b takes draw (M + b) & 3 of group
+// g0 + 4 HALF + ((M + b) >> 2): four calls, or five when M != 0, made together.
+template <int N, int M, int HALF>
+__device__ __forceinline__ void half_tests(uint32_t g0, const PassArgs& a, uint32_t c2,
+                                           uint32_t (&A)[N]) {
+    PhiloxRuns<1, M == 0 ? 4 : 5> ps;
+    const uint32_t base[1] = {g0 + (uint32_t)(4 * HALF)};
+    ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
+#pragma unroll
+    for (int r = 1; r < 10; ++r) ps.next_round();
+    static_for<16>([&](auto bit) {
+        constexpr int b = decltype(bit)::value, j = (M + b) & 3;
+        const Philox4 u = ps.result((M + b) >> 2);
+        const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
+#pragma unroll
+        for (int n = 0; n < N; ++n) mark_below<(1u << (16 * HALF + b))>(A[n], w, a.thr[n]);
+    });
+}
+
+// Accept mask of the `need` bits, one Philox call at a time: where the lanes
+// of a warp start at different offsets m inside their groups.
 template <int DIMS, typename K>
-__device__ __forceinline__ uint32_t group_accept(const K& k, const Philox4& u, int i,
-                                                 const PassArgs& a) {
-    const uint32_t w[4] = {u.w0, u.w1, u.w2, u.w3};
+__device__ __forceinline__ uint32_t packed_accept_mixed(const K& k, uint32_t need, uint32_t m,
+                                                        uint32_t g0, const PassArgs& a,
+                                                        uint32_t c2) {
     uint32_t acc = 0u;
+#pragma unroll 1
+    for (int g = 0; g < 9; ++g) {
+        const int lo = 4 * g - (int)m;  // bit of the group's word 0 (may be < 0)
+        if (lo > 31) break;
+        const uint32_t gmask = lo >= 0 ? (0xFu << lo) : (0xFu >> (-lo));
+        if (!(need & gmask)) continue;
+        const Philox4 u = philox4x32_10(g0 + (uint32_t)g, a.t, c2, kTagSweep, a.key0, a.key1);
+        const uint32_t w[4] = {u.w0, u.w1, u.w2, u.w3};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int b = 4 * i + j;
-        acc |= (w[j] < site_threshold<DIMS>(k, b, a) ? 1u : 0u) << b;
+        for (int j = 0; j < 4; ++j) {
+            const int b = lo + j;
+            if (b < 0 || b > 31) continue;
+            acc |= (w[j] < site_threshold<DIMS>(k, b, a) ? 1u : 0u) << b;
+        }
     }
     return acc;
 }
 
-// Accept mask of a 16-site half of a packed word whose first bit is half
-// index g0 * 4 + M + 16 * HALF (M = 1..3: the row starts inside a Philox
-// group).  Its sites draw from the five groups g0 + 4 HALF .. g0 + 4 HALF + 4
-// (bit b takes word (M + b) & 3 of group g0 + ((M + b) >> 2)); the five calls
-// are made together, and every index is a compile-time constant.
-template <int DIMS, int M, int HALF, typename K>
-__device__ __forceinline__ uint32_t packed_accept_half_shifted(const K& k, uint32_t g0,
-                                                               const PassArgs& a, uint32_t c2) {
-    Philox4 u[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-        u[i] = philox4x32_10(g0 + (uint32_t)(4 * HALF + i), a.t, c2, kTagSweep, a.key0, a.key1);
-    uint32_t acc = 0u;
-#pragma unroll
-    for (int b = 16 * HALF; b < 16 * HALF + 16; ++b) {
-        const int q = M + b - 16 * HALF;  // draw index within the five calls
-        const Philox4& g = u[q >> 2];
-        const uint32_t w = (q & 3) == 0 ? g.w0 : (q & 3) == 1 ? g.w1 : (q & 3) == 2 ? g.w2 : g.w3;
-        acc |= (w < site_threshold<DIMS>(k, b, a) ? 1u : 0u) << b;
+// Each site's answer for the threshold of its own number of disagreeing
+// neighbours, from the answers A[n] for every threshold (site_threshold's
+// choice, 32 sites at once).
+template <int DIMS>
+__device__ __forceinline__ uint32_t choose_answer(const Counts& k, const uint32_t (&A)[DIMS]) {
+    if constexpr (DIMS == 2) return (k.eq0 & A[1]) | (k.eq1 & A[0]);
+    else return (k.eq0 & A[2]) | (k.eq1 & A[1]) | (k.eq2 & A[0]);
+}
+template <int DIMS>
+__device__ __forceinline__ uint32_t choose_answer(const Digits& k,
+                                                  const uint32_t (&A)[2 * DIMS + 1]) {
+    const uint32_t a01 = (k.d0 & A[1]) | (~k.d0 & A[0]), a23 = (k.d0 & A[3]) | (~k.d0 & A[2]);
+    const uint32_t lo = (k.d1 & a23) | (~k.d1 & a01);
+    uint32_t hi = A[4];
+    if constexpr (DIMS == 3) {
+        const uint32_t a45 = (k.d0 & A[5]) | (~k.d0 & A[4]);
+        hi = (k.d1 & A[6]) | (~k.d1 & a45);
     }
-    return acc;
+    return (k.d2 & hi) | (~k.d2 & lo);
 }
 
-template <int DIMS, int M, typename K>
-__device__ __forceinline__ uint32_t packed_accept_shifted(const K& k, uint32_t need, uint32_t g0,
-                                                          const PassArgs& a, uint32_t c2) {
-    uint32_t acc = 0u;
-    if (need & 0xFFFFu) acc |= packed_accept_half_shifted<DIMS, M, 0>(k, g0, a, c2);
-    if (need >> 16) acc |= packed_accept_half_shifted<DIMS, M, 1>(k, g0, a, c2);
-    return acc;
+// ALL: draw for both halves in one straight line (a full word of a lattice
+// where nearly every half holds a site that draws); else a half without a
+// site that draws, such as the one past a short row's end, is passed over.
+template <int DIMS, int RULE, int M, bool ALL, typename K>
+__device__ __forceinline__ uint32_t packed_accept_at(const K& k, uint32_t need, uint32_t g0,
+                                                     const PassArgs& a, uint32_t c2) {
+    constexpr int N = kThresholds<DIMS, RULE>;
+    uint32_t A[N];
+#pragma unroll
+    for (int n = 0; n < N; ++n) A[n] = 0u;
+    if (ALL || (need & 0xFFFFu)) half_tests<N, M, 0>(g0, a, c2, A);
+    if (ALL || (need >> 16)) half_tests<N, M, 1>(g0, a, c2, A);
+    return choose_answer<DIMS>(k, A);
 }
 
 // Accept mask of the `need` bits of a packed word (Metropolis: the sites with
 // dE > 0; heat bath: every valid site) whose 32 bits are the half indices
-// hb = hbase + b (b = 0..31).  Bit b's draw
-// is word (hb & 3) of Philox group hb >> 2.  When hbase is a multiple of 4 the
-// eight groups are the word's nibbles and are computed four at a time; when a
-// row starts inside a group (W not a multiple of 4) the word spans nine
-// groups.  With ILP9 (the per-lattice pass), when the lanes of the warp share
-// the row offset, each half takes its five groups together
-// (packed_accept_shifted); otherwise, and in the batched kernel (which runs at
-// a fixed register budget), the nine are taken one at a time.
+// hb = hbase + b (b = 0..31).  Bit b's draw is word (hb & 3) of Philox group
+// hb >> 2: eight groups when hbase is a multiple of 4, nine when a row starts
+// inside a group (W not a multiple of 4).  The offset is a compile-time
+// constant in each path, taken when the lanes of the warp share it.
 // ALIGNED: the caller knows hbase % 4 == 0 (rows of a multiple of 32 sites),
 // so only the eight-group path is compiled.
-template <int DIMS, typename K, bool ILP9 = false, bool ALIGNED = false>
-__device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t need, uint32_t hbase,
-                                                  const PassArgs& a, uint32_t c2) {
-    uint32_t acc = 0u;
-    const uint32_t m = ALIGNED ? 0u : hbase & 3u, g0 = hbase >> 2;
-    if (!ALIGNED && ILP9 && m != 0u) {
-        // the compile-time offset paths only when the warp agrees on it
+template <int DIMS, int RULE, bool ALIGNED, typename K>
+__device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t need,
+                                                  uint32_t hbase, const PassArgs& a,
+                                                  uint32_t c2) {
+    const uint32_t g0 = hbase >> 2;
+    if constexpr (ALIGNED) {
+        return packed_accept_at<DIMS, RULE, 0, true>(k, need, g0, a, c2);
+    } else {
+        const uint32_t m = hbase & 3u;
+        if (m == 0u) return packed_accept_at<DIMS, RULE, 0, false>(k, need, g0, a, c2);
         const uint32_t lanes = __activemask();
         const uint32_t m0 = __shfl_sync(lanes, m, __ffs(lanes) - 1);
         if (__all_sync(lanes, m == m0)) {
-            if (m == 1u) return packed_accept_shifted<DIMS, 1>(k, need, g0, a, c2);
-            if (m == 2u) return packed_accept_shifted<DIMS, 2>(k, need, g0, a, c2);
-            return packed_accept_shifted<DIMS, 3>(k, need, g0, a, c2);
+            if (m == 1u) return packed_accept_at<DIMS, RULE, 1, false>(k, need, g0, a, c2);
+            if (m == 2u) return packed_accept_at<DIMS, RULE, 2, false>(k, need, g0, a, c2);
+            return packed_accept_at<DIMS, RULE, 3, false>(k, need, g0, a, c2);
         }
+        return packed_accept_mixed<DIMS>(k, need, m, g0, a, c2);
     }
-    if (m == 0u) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            if (!((need >> (16 * half)) & 0xFFFFu)) continue;
-            // four consecutive groups: one first-round product for the four
-            PhiloxRuns<1> ps;
-            const uint32_t base[1] = {g0 + (uint32_t)(4 * half)};
-            ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
-#pragma unroll
-            for (int r = 1; r < 10; ++r) ps.next_round();
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc |= group_accept<DIMS>(k, ps.result(i), 4 * half + i, a);
-        }
-        return acc;
-    }
-    if constexpr (!ALIGNED) {
-#pragma unroll 1
-        for (int g = 0; g < 9; ++g) {
-            const int lo = 4 * g - (int)m;  // bit of the group's word 0 (may be < 0)
-            const uint32_t gmask = lo >= 0 ? (0xFu << lo) : (0xFu >> (-lo));
-            if (!(need & gmask)) continue;
-            const Philox4 u = philox4x32_10(g0 + (uint32_t)g, a.t, c2, kTagSweep, a.key0,
-                                            a.key1);
-            const uint32_t w[4] = {u.w0, u.w1, u.w2, u.w3};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int b = lo + j;
-                if (b < 0 || b > 31) continue;
-                acc |= (w[j] < site_threshold<DIMS>(k, b, a) ? 1u : 0u) << b;
-            }
-        }
-    }
-    return acc;
 }
 
 // Update word (r, q) of the packed colour array.  A half row of W sites takes
@@ -717,7 +750,7 @@ __device__ __forceinline__ uint32_t grouped_row(uint32_t j, uint32_t rows, uint3
 // store and the word's share of E and M.  valid: the word's sites (nb bits);
 // hbase: the half index of bit 0 (its Philox draw is word hbase & 3 of group
 // hbase >> 2).  ALIGNED: hbase % 4 == 0 is known (packed_accept).
-template <int DIMS, bool MEASURE, int RULE, bool ILP9, bool ALIGNED>
+template <int DIMS, bool MEASURE, int RULE, bool ALIGNED>
 __device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_word, uint32_t s,
                                               uint32_t o, uint32_t sh, uint32_t oym,
                                               uint32_t oyp, uint32_t ozm, uint32_t ozp,
@@ -727,7 +760,7 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_w
     if constexpr (RULE == kRuleHeatBath) {  // every valid site draws
         const Digits k = DIMS == 2 ? digits2(s ^ o, s ^ sh, s ^ oym, s ^ oyp)
                                    : digits3(s ^ o, s ^ sh, s ^ oym, s ^ oyp, s ^ ozm, s ^ ozp);
-        flip = packed_accept<DIMS, Digits, ILP9, ALIGNED>(k, valid, hbase, a, (uint32_t)a.c);
+        flip = packed_accept<DIMS, RULE, ALIGNED>(k, valid, hbase, a, (uint32_t)a.c);
     } else if constexpr (RULE == kRuleMultiHit) {  // a.hits trials, neighbours fixed
         uint32_t cur = s;
 #pragma unroll 1
@@ -741,8 +774,8 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_w
             uint32_t f = k.always;
             const uint32_t need = ~k.always & valid;
             if (need)
-                f |= packed_accept<DIMS, Counts, ILP9, ALIGNED>(k, need, hbase, a,
-                                                               (uint32_t)a.c + 2u * (uint32_t)m);
+                f |= packed_accept<DIMS, RULE, ALIGNED>(k, need, hbase, a,
+                                                        (uint32_t)a.c + 2u * (uint32_t)m);
             cur ^= f & valid;
         }
         flip = cur ^ s;
@@ -755,7 +788,8 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_w
         }
         flip = k.always;
         const uint32_t need = ~k.always & valid;
-        if (need) flip |= packed_accept<DIMS, Counts, ILP9, ALIGNED>(k, need, hbase, a, (uint32_t)a.c);
+        if (ALIGNED || need)
+            flip |= packed_accept<DIMS, RULE, ALIGNED>(k, need, hbase, a, (uint32_t)a.c);
     }
     const uint32_t snew = s ^ (flip & valid);
     *own_word = snew;
@@ -770,9 +804,9 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_w
     }
 }
 
-template <int DIMS, bool MEASURE, int NC, int RULE = kRuleMetropolis, bool ILP9 = false>
+template <int DIMS, bool MEASURE, int NC, int RULE>
 __device__ __forceinline__ void packed_word(const PassArgs& a, uint32_t item, int& e_acc,
-                                            int& m_acc, uint32_t rgroups = 1u) {
+                                            int& m_acc, uint32_t rgroups) {
     const uint32_t W = (uint32_t)a.W;
     const uint32_t nq = (W + 31u) >> 5;
     const uint32_t L = (uint32_t)a.L;
@@ -818,9 +852,8 @@ __device__ __forceinline__ void packed_word(const PassArgs& a, uint32_t item, in
             sh = __funnelshift_r(o, load_other<NC>(other + row + q + 1u), 1);
         }
     }
-    packed_update<DIMS, MEASURE, RULE, ILP9, false>(a, own + row + q, s, o, sh, oym, oyp, ozm,
-                                                     ozp, valid, nb, r * W + 32u * q, e_acc,
-                                                     m_acc);
+    packed_update<DIMS, MEASURE, RULE, false>(a, own + row + q, s, o, sh, oym, oyp, ozm, ozp,
+                                              valid, nb, r * W + 32u * q, e_acc, m_acc);
 }
 
 }  // namespace ising

@@ -48,8 +48,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, uint32_t rgrou
     launch_dependents();
     if constexpr (!FULL) {
         for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < items; g += stride)
-            packed_word<DIMS, MEASURE, 1, RULE, RULE != kRuleMultiHit>(a, g, e_acc, m_acc,
-                                                                       rgroups);
+            packed_word<DIMS, MEASURE, 1, RULE>(a, g, e_acc, m_acc, rgroups);
     } else {
         const uint32_t nq = 1u << nq_shift, L = (uint32_t)a.L, W = (uint32_t)a.W;
         uint32_t* own = static_cast<uint32_t*>(a.own);
@@ -92,7 +91,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, uint32_t rgrou
                 // bit b <- neighbour xh - 1 (p = 0) or xh + 1 (p = 1)
                 const uint32_t sh = p == 0 ? __funnelshift_l(cur.x, cur.o, 1)
                                            : __funnelshift_r(cur.o, cur.x, 1);
-                packed_update<DIMS, MEASURE, RULE, RULE != kRuleMultiHit, true>(
+                packed_update<DIMS, MEASURE, RULE, true>(
                     a, own + r * nq + q, cur.s, cur.o, sh, cur.ym, cur.yp, cur.zm, cur.zp,
                     0xFFFFFFFFu, 32u, r * W + 32u * q, e_acc, m_acc);
                 if (!more) break;
