@@ -71,7 +71,9 @@ int perc_get_pores(perc_medium *m, uint8_t *host_out);
 int perc_get_cluster(perc_medium *m, uint8_t *host_out);
 
 /* How perc_invade runs its passes (same results either way):
- *   PERC_PASSES_AUTO (default): PERC_PASSES_GRAPH (measured the faster);
+ *   PERC_PASSES_AUTO (default): 2D media in tiles held in registers, many
+ *       passes per launch; 3D media as PERC_PASSES_GRAPH (both measured the
+ *       fastest);
  *   PERC_PASSES_GRAPH: a CUDA graph of 64 chained pass launches (each placed
  *       on the SMs while the previous one drains) replayed until a pass adds
  *       nothing;

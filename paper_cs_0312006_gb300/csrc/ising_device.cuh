@@ -15,6 +15,8 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <type_traits>
+#include <utility>
 
 namespace ising {
 
@@ -139,6 +141,28 @@ __device__ __forceinline__ void mark_below(uint32_t& mask, uint32_t u, uint32_t 
         "}"
         : "+r"(mask)
         : "r"(u), "r"(thr), "n"(BITS));
+}
+
+// mask |= bits where u <= thr.
+template <uint32_t BITS>
+__device__ __forceinline__ void mark_upto(uint32_t& mask, uint32_t u, uint32_t thr) {
+    asm("{\n"
+        ".reg .pred p;\n"
+        "setp.le.u32 p, %1, %2;\n"
+        "@p or.b32 %0, %0, %3;\n"
+        "}"
+        : "+r"(mask)
+        : "r"(u), "r"(thr), "n"(BITS));
+}
+
+// f(std::integral_constant<int, I>) for I = 0..N-1, unrolled.
+template <int N, typename F, int... I>
+__device__ __forceinline__ void static_for(F&& f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, typename F>
+__device__ __forceinline__ void static_for(F&& f) {
+    static_for<N>(f, std::make_integer_sequence<int, N>{});
 }
 
 // Programmatic dependent launch (griddepcontrol, sm_90 and later).  The

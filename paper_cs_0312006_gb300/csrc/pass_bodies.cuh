@@ -20,22 +20,9 @@
 
 #include <cstdint>
 
-#include <type_traits>
-#include <utility>
-
 #include "ising_device.cuh"
 
 namespace ising {
-
-// f(std::integral_constant<int, I>) for I = 0..N-1, unrolled.
-template <int N, typename F, int... I>
-__device__ __forceinline__ void static_for(F&& f, std::integer_sequence<int, I...>) {
-    (f(std::integral_constant<int, I>{}), ...);
-}
-template <int N, typename F>
-__device__ __forceinline__ void static_for(F&& f) {
-    static_for<N>(f, std::make_integer_sequence<int, N>{});
-}
 
 constexpr uint32_t kByteBit1 = 0x02020202u;
 constexpr uint32_t kByteBit7 = 0x80808080u;

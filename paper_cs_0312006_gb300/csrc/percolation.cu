@@ -19,11 +19,16 @@
 // Draws: site i is a pore iff word (i & 3) of Philox4x32-10(seed; i >> 2, 0,
 // 0, 3) is <= floor(P 2^32) (capped at 2^32 - 1).
 //
-// A single medium's passes touch only a band of rows: each pass records the
-// lowest and highest row of the front it writes (Band), and the next pass
-// visits the rows next to that front plus the rows of the front before it
-// (which it must clear from the buffer it overwrites).  Two ways to run the
-// passes, with the same results (the graph is the default: measured faster):
+// A single 2D medium grows in registers, many passes per launch (grow_block,
+// perc_blocked_kernel): a pass at a time, each launch cost 2 - 4 us whatever the
+// pass held.  2D L = 4096, P = 0.6, from a face, 8951 passes: 28.0 -> 3.2 ms.
+//
+// 3D media, and 2D ones on request (perc_set_passes), run pass by pass.  Those
+// passes touch only a band of rows: each records the lowest and highest row of
+// the front it writes (Band), and the next visits the rows next to that front
+// plus the rows of the front before it (which it must clear from the buffer it
+// overwrites).  Two ways to run them, with the same results (the graph is the
+// 3D default: measured faster):
 //   - one cooperative persistent launch: every CTA resident, the passes
 //     separated by a grid barrier (an arrival counter and a generation word;
 //     every wait on it bounded by %globaltimer, a CTA that gives up raises
@@ -59,44 +64,40 @@ struct PercGeom {
 __device__ __forceinline__ uint32_t pore_word(uint64_t i0, uint32_t nb, uint32_t key0,
                                               uint32_t key1, uint32_t thr) {
     uint32_t w = 0u;
+    const uint32_t valid = nb == 32u ? 0xFFFFFFFFu : (1u << nb) - 1u;
     const uint32_t g0 = (uint32_t)(i0 >> 2);
     const int m = (int)(i0 & 3u);
     if (m == 0) {  // the bits are whole Philox groups: eight at most, four at a time
-        const uint32_t groups = (nb + 3u) >> 2;
+        static_for<2>([&](auto half) {
+            constexpr int h = decltype(half)::value;
+            if (nb <= 16u * h) return;
+            PhiloxRuns<1> ps;
+            const uint32_t base[1] = {g0 + 4u * h};
+            ps.first_round(base, 0u, 0u, kTagPore, key0, key1);
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            Philox4 u[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t gi = 4u * half + k;
-                u[k] = gi < groups ? philox4x32_10(g0 + gi, 0u, 0u, kTagPore, key0, key1)
-                                   : Philox4{0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t v[4] = {u[k].w0, u[k].w1, u[k].w2, u[k].w3};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t b = 16u * half + 4u * k + j;
-                    w |= (v[j] <= thr && b < nb ? 1u : 0u) << b;
-                }
-            }
-        }
-        return w;
+            for (int r = 1; r < 10; ++r) ps.next_round();
+            static_for<16>([&](auto bit) {
+                constexpr int b = decltype(bit)::value, j = b & 3;
+                const Philox4 u = ps.result(b >> 2);
+                mark_upto<(1u << (16 * h + b))>(
+                    w, j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3, thr);
+            });
+        });
+        return w & valid;
     }
 #pragma unroll 1
     for (int g = 0; g < 9; ++g) {  // a row that starts inside a group spans nine
         const int lo = 4 * g - m;
         if (lo >= (int)nb) break;
         const Philox4 u = philox4x32_10(g0 + (uint32_t)g, 0u, 0u, kTagPore, key0, key1);
-        const uint32_t v[4] = {u.w0, u.w1, u.w2, u.w3};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int b = lo + j;
-            if (b >= 0 && b < (int)nb && v[j] <= thr) w |= 1u << b;
-        }
+        uint32_t four = 0u;
+        mark_upto<1u>(four, u.w0, thr);
+        mark_upto<2u>(four, u.w1, thr);
+        mark_upto<4u>(four, u.w2, thr);
+        mark_upto<8u>(four, u.w3, thr);
+        w |= lo >= 0 ? four << lo : four >> -lo;
     }
-    return w;
+    return w & valid;
 }
 
 __device__ __forceinline__ uint32_t valid_bits(uint32_t L, uint32_t q) {
@@ -272,6 +273,211 @@ __global__ void __launch_bounds__(256) perc_band_kernel(const uint32_t* pore, ui
     block_sum_u64(cnt, added);
 }
 
+// Growth with a block of the medium in registers.  A thread holds a block of
+// kBlockRows rows by kBlockCols words (32 sites each) of the pores P and the
+// cluster C; LANES lanes in a row hold neighbouring columns, and the CTA's
+// block rows follow one another.  In a pass the bits that cross between columns
+// are gathered from the thread's rows into one word per side (a byte per row)
+// and exchanged with one shuffle each; every block's first and last row goes
+// through shared memory, double buffered, so a pass has one barrier.  Growing
+// from the whole cluster instead of the last front gives the same passes (every
+// pore next to an older cluster site joined already), so no front is kept.
+// Passes go in groups of kGroup.  A warp's block rows are consecutive, at least
+// kGroup rows of them, so nothing can change in a warp during a group when
+// neither it nor the warps above and below changed in the group before; it then
+// only meets the barriers.  An active warp's pass is about 70 instructions, all
+// on the ALU pipe (2 cycles each: 88 % busy with many CTAs per SM, when every
+// warp took every pass).  2048 media of L = 256 at the threshold (504 passes on
+// average): 6.4 -> 1.1 ms with the host's work, against fronts and clusters in
+// shared memory; 1.5 ms before idle warps were passed over.
+constexpr int kBlockRows = 4, kBlockCols = 2;
+constexpr int kGroup = 4;         // passes between looks at which warps still grow
+constexpr int kAllPasses = 0x7FFFFFFF / kGroup * kGroup;
+// Up to here one CTA of at most 256 threads holds a whole 2D medium and runs to
+// the steady state in one launch: ~0.2 us a pass (L = 256, 631 passes: 125 us;
+// in tiles 219 us; the graph's 64 launches a replay 1350 us).  At L = 300 the
+// tiles' 0.35 us a pass (223 us) is less than one CTA of twice the warps needs.
+constexpr int kWholeL = 256;
+// A tiled medium: CTAs of 32 block rows by 8 lanes, 64 rows by 12 words inside
+// the halo, 32 passes a launch.  L = 4096 / 1000, 8951 / 2457 passes from a face:
+// 3.25 / 0.73 ms; with 512 threads (192 rows inside) 3.69 / 0.96, 16 passes a
+// launch 3.64 / 0.99, 64 passes and 512 threads 3.56 / 0.79.
+constexpr int kTilePasses = 32;
+constexpr int kTileLanes = 8;
+constexpr int kTileThreads = 256;
+constexpr int kHaloWords = 2;     // columns of halo on a side: whole threads, at least kTilePasses sites
+
+// Words of shared memory that grow_block exchanges rows and the warps' growth
+// through (1024 threads at most).
+constexpr int kWarpFlags = 32 + 2;
+__host__ __device__ constexpr int edge_words(int blocks, int lanes) {
+    return 4 * (blocks + 2) * lanes * kBlockCols + 2 * kWarpFlags;
+}
+
+// Runs up to max_passes passes (a multiple of kGroup), fewer once nothing in
+// the whole block changes; returns the last pass (counted from 1) in which this
+// thread's words grew, 0 for none.  Every thread of the CTA calls it.
+template <int LANES>
+__device__ __forceinline__ int grow_block(const uint32_t (&P)[kBlockRows][kBlockCols],
+                                          uint32_t (&C)[kBlockRows][kBlockCols], int max_passes,
+                                          uint32_t* edges, int blocks, int block, int lane) {
+    static_assert(32 / LANES * kBlockRows >= kGroup, "growth must not cross a warp in a group");
+    uint2* rows = reinterpret_cast<uint2*>(edges);
+    const int plane = (blocks + 2) * LANES;  // one buffer's first (or last) rows, with guards
+    for (int i = threadIdx.x; i < 4 * plane; i += blockDim.x) {
+        const int b = (i % plane) / LANES;
+        if (b == 0 || b == blocks + 1) rows[i] = make_uint2(0u, 0u);
+    }
+    int* warp_grew = reinterpret_cast<int*>(rows + 4 * plane);
+    for (int i = threadIdx.x; i < 2 * kWarpFlags; i += blockDim.x) warp_grew[i] = 0;
+    __syncthreads();
+    const int warp = (int)(threadIdx.x >> 5);
+    const uint32_t left_ok = lane > 0 ? 0xFFFFFFFFu : 0u;
+    const uint32_t right_ok = lane < LANES - 1 ? 0xFFFFFFFFu : 0u;
+    const int at = (block + 1) * LANES + lane;
+    auto give_rows = [&](int buffer) {
+        uint2* r = rows + buffer * 2 * plane + at;
+        r[0] = make_uint2(C[0][0], C[0][1]);
+        r[plane] = make_uint2(C[kBlockRows - 1][0], C[kBlockRows - 1][1]);
+    };
+    // one pass, the neighbouring rows taken from `buffer`; the bits that grew
+    auto pass = [&](int buffer) {
+        const uint2* r = rows + buffer * 2 * plane + at;
+        const uint2 before = r[plane - LANES], after = r[LANES];
+        // byte i: the outer byte of row i's last word (its top bit crosses to
+        // the right) and of its first word (its low bit crosses to the left)
+        uint32_t from_left = 0u, from_right = 0u;
+        if constexpr (LANES > 1) {
+            const uint32_t to_right = __byte_perm(__byte_perm(C[0][1], C[1][1], 0x0073),
+                                                  __byte_perm(C[2][1], C[3][1], 0x0073), 0x5410);
+            const uint32_t to_left = __byte_perm(__byte_perm(C[0][0], C[1][0], 0x0040),
+                                                 __byte_perm(C[2][0], C[3][0], 0x0040), 0x5410);
+            from_left = __shfl_up_sync(0xffffffffu, to_right, 1, LANES) & left_ok;
+            from_right = __shfl_down_sync(0xffffffffu, to_left, 1, LANES) & right_ok;
+        }
+        uint32_t above0 = before.x, above1 = before.y, grew = 0u;
+#pragma unroll
+        for (int i = 0; i < kBlockRows; ++i) {
+            const uint32_t c0 = C[i][0], c1 = C[i][1];
+            const uint32_t down0 = i + 1 < kBlockRows ? C[i + 1][0] : after.x;
+            const uint32_t down1 = i + 1 < kBlockRows ? C[i + 1][1] : after.y;
+            const uint32_t side0 = __funnelshift_l(from_left << (24 - 8 * i), c0, 1) |
+                                   __funnelshift_r(c0, c1, 1);
+            const uint32_t side1 = __funnelshift_l(c0, c1, 1) |
+                                   __funnelshift_r(c1, from_right >> (8 * i), 1);
+            const uint32_t n0 = c0 | ((side0 | above0 | down0) & P[i][0]);
+            const uint32_t n1 = c1 | ((side1 | above1 | down1) & P[i][1]);
+            grew |= n0 ^ c0;
+            grew |= n1 ^ c1;
+            C[i][0] = n0;
+            C[i][1] = n1;
+            above0 = c0;
+            above1 = c1;
+        }
+        return grew;
+    };
+    int last = 0;
+    uint32_t grew_group = 1u;
+    for (int k = 0; k < max_passes; k += kGroup) {
+        int* flags = warp_grew + (k / kGroup & 1) * kWarpFlags + warp;
+        give_rows(0);
+        const int warp_any = __any_sync(0xffffffffu, grew_group != 0u);
+        if ((threadIdx.x & 31u) == 0u) flags[1] = warp_any;
+        if (!__syncthreads_or(grew_group != 0u)) break;  // nothing changed in the last group
+        grew_group = 0u;
+        if ((flags[0] | flags[1] | flags[2]) == 0) {
+            give_rows(1);
+#pragma unroll
+            for (int j = 1; j < kGroup; ++j) __syncthreads();
+            continue;
+        }
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j) {
+            if (j > 0) {
+                give_rows(j & 1);
+                __syncthreads();
+            }
+            const uint32_t grew = pass(j & 1);
+            grew_group |= grew;
+            if (grew != 0u) last = k + j + 1;
+        }
+    }
+    return last;
+}
+
+// One launch of blocked growth over a 2D medium: each CTA takes a tile with a
+// halo of `passes` rows above and below and kHaloWords words on each side, and
+// grows it `passes` times; the halo's outer ring is stale by one more site after
+// every pass, so the tile itself stays exact.  A single tile (no halo) runs
+// until nothing grows.  Tiles are read from Ci and written to Co: a tile is
+// skipped unless it or a neighbour grew in the launch before (then nothing can
+// reach it, and both buffers hold it alike).  stamps: per parity of the launch,
+// the launch (from 1) in which each tile last grew.  *steps becomes the last
+// pass that added a site anywhere.
+struct TileGrid {
+    int nx, ny;        // tiles
+    int words, rows;   // interior of a tile
+    int halo;          // rows above and below; with it, kHaloWords on each side if nx > 1
+};
+
+template <int LANES>
+__global__ void __launch_bounds__(512) perc_blocked_kernel(const uint32_t* pore,
+                                                           const uint32_t* Ci, uint32_t* Co,
+                                                           PercGeom g, TileGrid tg, int passes,
+                                                           int launch, int* stamps,
+                                                           unsigned long long* steps) {
+    extern __shared__ __align__(8) uint32_t edges[];
+    __shared__ int s_last;
+    const int tile = (int)blockIdx.x, ty = tile / tg.nx, tx = tile - ty * tg.nx;
+    const int tiles = tg.nx * tg.ny;
+    const int block = (int)threadIdx.x / LANES, lane = (int)threadIdx.x % LANES;
+    const int blocks = (int)blockDim.x / LANES;
+    const int side = tg.nx > 1 ? kHaloWords : 0;
+    const int r0 = ty * tg.rows - tg.halo + block * kBlockRows;
+    const int q0 = tx * tg.words - side + lane * kBlockCols;
+    uint32_t P[kBlockRows][kBlockCols], C[kBlockRows][kBlockCols];
+    auto inside = [&](int i, int j) {
+        return r0 + i >= 0 && r0 + i < (int)g.rows && q0 + j >= 0 && q0 + j < (int)g.nq;
+    };
+    auto word = [&](int i, int j) { return (uint32_t)(r0 + i) * g.nq + (uint32_t)(q0 + j); };
+    grid_dependency_wait();
+    launch_dependents();
+    if (launch > 0) {
+        int active = 0;
+        if (threadIdx.x < 9) {
+            const int nx = tx + (int)threadIdx.x % 3 - 1, ny = ty + (int)threadIdx.x / 3 - 1;
+            if (nx >= 0 && nx < tg.nx && ny >= 0 && ny < tg.ny)
+                active = stamps[((launch - 1) & 1) * tiles + ny * tg.nx + nx] == launch;
+        }
+        if (!__syncthreads_or(active)) return;
+    }
+    if (threadIdx.x == 0) s_last = 0;
+#pragma unroll
+    for (int i = 0; i < kBlockRows; ++i)
+#pragma unroll
+        for (int j = 0; j < kBlockCols; ++j) {
+            P[i][j] = inside(i, j) ? __ldg(pore + word(i, j)) : 0u;
+            C[i][j] = inside(i, j) ? Ci[word(i, j)] : 0u;
+        }
+    const int last = grow_block<LANES>(P, C, passes, edges, blocks, block, lane);
+    const int row = block * kBlockRows, col = lane * kBlockCols;
+    const bool mine = row >= tg.halo && row < tg.halo + tg.rows && col >= side &&
+                      col < side + tg.words;
+    if (mine) {
+        if (last > 0) atomicMax(&s_last, last);
+#pragma unroll
+        for (int i = 0; i < kBlockRows; ++i)
+#pragma unroll
+            for (int j = 0; j < kBlockCols; ++j)
+                if (inside(i, j)) Co[word(i, j)] = C[i][j];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_last > 0) {
+        stamps[(launch & 1) * tiles + tile] = launch + 1;
+        atomicMax(steps, (unsigned long long)launch * (unsigned)passes + (unsigned)s_last);
+    }
+}
+
 struct GridBar {
     unsigned int count;  // CTAs arrived at the current barrier
     unsigned int gen;    // barriers completed
@@ -393,7 +599,12 @@ __global__ void perc_export_kernel(const uint32_t* bits, PercGeom g, uint8_t* ou
     }
 }
 
-// One CTA per medium, everything in shared memory: pores, cluster, fronts.
+// The low four bits of h as four bytes 0 / 1.
+__device__ __forceinline__ uint32_t spread4(uint32_t h) {
+    return ((h & 0xFu) * 0x00204081u) & 0x01010101u;
+}
+
+// One CTA per 3D medium, everything in shared memory: pores, cluster, fronts.
 __global__ void __launch_bounds__(512) perc_batch_kernel(PercGeom g, uint32_t thr,
                                                          const uint64_t* seeds, int source,
                                                          uint64_t site, perc_result* res,
@@ -473,6 +684,95 @@ __global__ void __launch_bounds__(512) perc_batch_kernel(PercGeom g, uint32_t th
     }
 }
 
+// 2D media with a cluster held in registers (grow_block): one CTA per medium,
+// ceil(L / 4) block rows of LANES >= ceil(L / 64) lanes.
+template <int LANES>
+__global__ void __launch_bounds__(LANES == 8 ? 1024 : 256)
+    perc_batch_blocked_kernel(PercGeom g, uint32_t thr, const uint64_t* seeds, int source,
+                              uint64_t site, perc_result* res, uint8_t* clusters, bool vec) {
+    extern __shared__ uint32_t sm[];
+    __shared__ unsigned long long s_size;
+    __shared__ int s_last;
+    const uint32_t words = g.rows * g.nq;
+    uint32_t* bits = sm;           // pores, then the cluster
+    uint32_t* edges = sm + ((words + 1u) & ~1u);
+    const int block = (int)threadIdx.x / LANES, lane = (int)threadIdx.x % LANES;
+    const int blocks = (int)blockDim.x / LANES;
+    const uint64_t seed = seeds[blockIdx.x];
+    const uint32_t key0 = (uint32_t)(seed & 0xFFFFFFFFu), key1 = (uint32_t)(seed >> 32);
+    if (threadIdx.x == 0) {
+        s_size = 0ull;
+        s_last = 0;
+    }
+    for (uint32_t w = threadIdx.x; w < words; w += blockDim.x) {
+        const uint32_t r = w / g.nq, q = w - r * g.nq;
+        bits[w] = pore_word((uint64_t)g.L * r + 32u * q, valid_bits(g.L, q), key0, key1, thr);
+    }
+    __syncthreads();
+    const int r0 = block * kBlockRows, q0 = lane * kBlockCols;
+    const int site_r = (int)(site / g.L);
+    const uint32_t site_x = (uint32_t)(site - (uint64_t)site_r * g.L);
+    uint32_t P[kBlockRows][kBlockCols], C[kBlockRows][kBlockCols];
+    auto inside = [&](int i, int j) { return r0 + i < (int)g.rows && q0 + j < (int)g.nq; };
+#pragma unroll
+    for (int i = 0; i < kBlockRows; ++i)
+#pragma unroll
+        for (int j = 0; j < kBlockCols; ++j) {
+            const uint32_t p = inside(i, j) ? bits[(r0 + i) * (int)g.nq + q0 + j] : 0u;
+            P[i][j] = p;
+            if (source == PERC_FACE)
+                C[i][j] = r0 + i == 0 ? p : 0u;
+            else
+                C[i][j] = r0 + i == site_r && q0 + j == (int)(site_x >> 5)
+                              ? p & (1u << (site_x & 31u)) : 0u;
+        }
+    // ends: every pass that continues adds at least one of the medium's sites
+    const int last = grow_block<LANES>(P, C, kAllPasses, edges, blocks, block, lane);
+    int size = 0, first_face = 0, last_face = 0;
+#pragma unroll
+    for (int i = 0; i < kBlockRows; ++i)
+#pragma unroll
+        for (int j = 0; j < kBlockCols; ++j) {
+            size += __popc(C[i][j]);
+            if (C[i][j] != 0u && r0 + i == 0) first_face = 1;
+            if (C[i][j] != 0u && r0 + i == (int)g.L - 1) last_face = 1;
+            if (inside(i, j)) bits[(r0 + i) * (int)g.nq + q0 + j] = C[i][j];
+        }
+    size = __reduce_add_sync(0xffffffffu, size);
+    const int warp_last = __reduce_max_sync(0xffffffffu, last);
+    if ((threadIdx.x & 31u) == 0u) {
+        if (size) atomicAdd(&s_size, (unsigned long long)size);
+        if (warp_last) atomicMax(&s_last, warp_last);
+    }
+    first_face = __syncthreads_or(first_face);
+    last_face = __syncthreads_or(last_face);
+    if (threadIdx.x == 0) {
+        perc_result o;
+        o.size = (int64_t)s_size;
+        o.spans = first_face && last_face ? 1 : 0;
+        o.reserved = 0;
+        o.steps = s_last;
+        res[blockIdx.x] = o;
+    }
+    if (!clusters) return;
+    const uint32_t sites = g.rows * g.L;
+    uint8_t* out = clusters + (uint64_t)blockIdx.x * sites;
+    if (vec) {  // L % 16 == 0 and a 16-byte aligned buffer: half a word at a time
+        const uint32_t per_row = g.L >> 4;
+        for (uint32_t i = threadIdx.x; i < g.rows * per_row; i += blockDim.x) {
+            const uint32_t r = i / per_row, x = i - r * per_row;
+            const uint32_t h = bits[r * g.nq + (x >> 1)] >> (16u * (x & 1u));
+            reinterpret_cast<uint4*>(out)[i] =
+                make_uint4(spread4(h), spread4(h >> 4), spread4(h >> 8), spread4(h >> 12));
+        }
+    } else {
+        for (uint32_t i = threadIdx.x; i < sites; i += blockDim.x) {
+            const uint32_t r = i / g.L, x = i - r * g.L;
+            out[i] = (uint8_t)((bits[r * g.nq + (x >> 5)] >> (x & 31u)) & 1u);
+        }
+    }
+}
+
 unsigned grid_for(uint64_t n, int sm_count) {
     uint64_t b = (n + 255) / 256;
     const uint64_t cap = (uint64_t)sm_count * 16;
@@ -506,6 +806,8 @@ struct perc_medium {
     Band* bands = nullptr;
     cudaGraphExec_t passes = nullptr;      // kPassesPerGraph banded passes
     int mode = PERC_PASSES_AUTO;
+    int* stamps = nullptr;                 // blocked growth: tiles' last launch with growth
+    size_t stamp_bytes = 0;
     int coop_grid = 0;                     // resident CTAs of the persistent kernel (0: none)
     void* coop = nullptr;                  // counters, barrier, steps, error flag
     cudaStream_t stream = nullptr;
@@ -521,6 +823,7 @@ void free_medium(perc_medium* m) {
     if (m->meas) cudaFree(m->meas);
     if (m->bands) cudaFree(m->bands);
     if (m->coop) cudaFree(m->coop);
+    if (m->stamps) cudaFree(m->stamps);
     if (m->passes) cudaGraphExecDestroy(m->passes);
     delete m;
 }
@@ -545,6 +848,101 @@ bool geometry(int dims, int L, PercGeom* g, uint64_t* sites) {
         cudaError_t e_ = (call);                            \
         if (e_ != cudaSuccess) return ising::cuda_fail(e_); \
     } while (0)
+
+namespace {
+
+// Lanes of a block row that holds a whole row of nq words.
+int whole_lanes(int nq) {
+    int lanes = 1;
+    while (lanes * kBlockCols < nq) lanes *= 2;
+    return lanes;
+}
+
+// The tiles of a 2D medium's blocked growth and the CTA that takes one.
+struct BlockedPlan {
+    TileGrid tg;
+    int lanes, threads, passes;
+};
+
+BlockedPlan blocked_plan(const PercGeom& g) {
+    BlockedPlan p{};
+    const int L = (int)g.L, nq = (int)g.nq;
+    if (L <= kWholeL) {  // one CTA holds it all
+        p.lanes = whole_lanes(nq);
+        const int blocks = (L + kBlockRows - 1) / kBlockRows;
+        p.threads = (blocks * p.lanes + 31) / 32 * 32;
+        p.tg = TileGrid{1, 1, p.lanes * kBlockCols, p.threads / p.lanes * kBlockRows, 0};
+        p.passes = kAllPasses;
+    } else {
+        p.lanes = kTileLanes;
+        p.threads = kTileThreads;
+        p.passes = kTilePasses;
+        const int words = kTileLanes * kBlockCols;
+        const int rows = p.threads / p.lanes * kBlockRows - 2 * p.passes;
+        int nx = 1, inner = words;  // whole rows in a tile where they fit
+        if (nq > words) {
+            inner = words - 2 * kHaloWords;
+            nx = (nq + inner - 1) / inner;
+            inner = ((nq + nx - 1) / nx + kBlockCols - 1) / kBlockCols * kBlockCols;
+        }
+        p.tg = TileGrid{nx, (L + rows - 1) / rows, inner, rows, p.passes};
+    }
+    return p;
+}
+
+cudaError_t launch_blocked(const perc_medium* m, const BlockedPlan& p, int launch,
+                           unsigned long long* steps) {
+    const uint32_t* Ci = (launch & 1) ? m->F[0] : m->C;
+    // (a single tile is read whole before it is written: in place)
+    uint32_t* Co = (launch & 1) || p.tg.halo == 0 ? m->C : m->F[0];
+    const unsigned grid = (unsigned)(p.tg.nx * p.tg.ny);
+    const size_t smem = sizeof(uint32_t) * (size_t)edge_words(p.threads / p.lanes, p.lanes);
+    auto go = [&](auto kernel) {
+        return launch_chained(kernel, grid, (unsigned)p.threads, smem, m->stream,
+                              static_cast<const uint32_t*>(m->pore), Ci, Co, m->g, p.tg, p.passes,
+                              launch, m->stamps, steps);
+    };
+    switch (p.lanes) {
+        case 1: return go(perc_blocked_kernel<1>);
+        case 2: return go(perc_blocked_kernel<2>);
+        case 4: return go(perc_blocked_kernel<4>);
+        default: return go(perc_blocked_kernel<8>);
+    }
+}
+
+// Blocked growth from the seeded C and F[0] (which hold the same) to the
+// steady state; the cluster ends in both.  The host looks at the pass count
+// after a few launches at a time: passes run beyond the last that added a site
+// mean the steady state is reached.
+int invade_blocked(perc_medium* m, int64_t* steps_out) {
+    const BlockedPlan p = blocked_plan(m->g);
+    const size_t stamp_bytes = sizeof(int) * 2 * (size_t)p.tg.nx * p.tg.ny;
+    if (!m->stamps) {
+        PERC_CHECK(cudaMalloc(reinterpret_cast<void**>(&m->stamps), stamp_bytes));
+        m->stamp_bytes = stamp_bytes;
+    }
+    unsigned long long* steps = m->meas;
+    PERC_CHECK(cudaMemsetAsync(m->stamps, 0, m->stamp_bytes, m->stream));
+    PERC_CHECK(cudaMemsetAsync(steps, 0, 8, m->stream));
+    unsigned long long seen = 0;
+    if (p.tg.halo == 0) {  // one tile, one launch: to the steady state
+        PERC_CHECK(launch_blocked(m, p, 0, steps));
+        PERC_CHECK(cudaMemcpyAsync(&seen, steps, 8, cudaMemcpyDeviceToHost, m->stream));
+        PERC_CHECK(cudaStreamSynchronize(m->stream));
+    } else {
+        int launch = 0;
+        for (int batch = 4;; batch = batch < 16 ? batch * 2 : 16) {
+            for (int k = 0; k < batch; ++k) PERC_CHECK(launch_blocked(m, p, launch++, steps));
+            PERC_CHECK(cudaMemcpyAsync(&seen, steps, 8, cudaMemcpyDeviceToHost, m->stream));
+            PERC_CHECK(cudaStreamSynchronize(m->stream));
+            if (seen < (unsigned long long)launch * (unsigned)p.passes) break;
+        }
+    }
+    *steps_out = (int64_t)seen;
+    return ISING_OK;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -629,7 +1027,11 @@ int perc_invade(perc_medium* m, int source, int64_t site, perc_result* out) {
                                                   m->bands);
     PERC_CHECK(cudaGetLastError());
     int64_t steps = 0;
-    // AUTO takes the graph: on GB300 it measured 4.6 us per pass at L = 16384
+    if (m->mode == PERC_PASSES_AUTO && m->g.dims == 2) {
+        const int rc = invade_blocked(m, &steps);
+        if (rc != ISING_OK) return rc;
+    } else
+    // the graph: on GB300 it measured 4.6 us per pass at L = 16384
     // (chained launches, eight CTAs per SM) against 8.5 us for the persistent
     // launch (2 - 4 CTAs per SM; 12 us with one, 14 us with all that fit): the
     // pass's own work needs the wide grid, and the grid barrier costs more than
@@ -766,25 +1168,47 @@ int perc_batch(int dims, int L, double porosity, const uint64_t* seeds, int n, i
     uint32_t thr = 0;
     int rc = porosity_threshold(porosity, &thr);
     if (rc != ISING_OK) return rc;
-    const size_t smem = (size_t)4 * g.rows * g.nq * sizeof(uint32_t);
-    cudaError_t e = cudaFuncSetAttribute(perc_batch_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(smem > 48 * 1024 ? smem : 48 * 1024));
+    const int lanes = dims == 2 ? whole_lanes((int)g.nq) : 1;
+    // 2D: a thread per block of a word column; 3D: the words in shared memory
+    const int blocked = ((int)g.rows + kBlockRows - 1) / kBlockRows * lanes;
+    const int threads = dims == 2 ? (blocked + 31) / 32 * 32 : g.rows * g.nq >= 2048 ? 512 : 256;
+    const size_t words = (size_t)g.rows * g.nq;
+    const size_t smem =
+        sizeof(uint32_t) * (dims == 2 ? ((words + 1) & ~(size_t)1) +
+                                            (size_t)edge_words(threads / lanes, lanes)
+                                      : 4 * words);
+    cudaError_t e = cudaSuccess;
+    if (smem > 46 * 1024)  // near or over the default limit (with the static part)
+        e = cudaFuncSetAttribute(dims == 2 ? (const void*)perc_batch_blocked_kernel<8>
+                                           : (const void*)perc_batch_kernel,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint64_t* d_seeds = nullptr;
     perc_result* d_res = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&d_seeds), sizeof(uint64_t) * (size_t)n, st);
+    const DeviceProps* dp = nullptr;
+    rc = device_props(&dp);
+    if (rc != ISING_OK) return rc;
+    e = pool_alloc(reinterpret_cast<void**>(&d_seeds), sizeof(uint64_t) * (size_t)n, *dp, st);
     if (e == cudaSuccess)
-        e = cudaMallocAsync(reinterpret_cast<void**>(&d_res), sizeof(perc_result) * (size_t)n, st);
+        e = pool_alloc(reinterpret_cast<void**>(&d_res), sizeof(perc_result) * (size_t)n, *dp, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_seeds, seeds, sizeof(uint64_t) * (size_t)n, cudaMemcpyHostToDevice,
                             st);
     if (e == cudaSuccess) {
-        const int threads = g.rows * g.nq >= 2048 ? 512 : 256;
-        perc_batch_kernel<<<(unsigned)n, threads, smem, st>>>(
-            g, thr, d_seeds, source, source == PERC_POINT ? (uint64_t)site : 0ull, d_res,
-            clusters_dev);
+        const uint64_t at = source == PERC_POINT ? (uint64_t)site : 0ull;
+        const bool vec = L % 16 == 0 && ((uintptr_t)clusters_dev & 15u) == 0;
+        auto blocks2d = [&](auto kernel) {
+            kernel<<<(unsigned)n, threads, smem, st>>>(g, thr, d_seeds, source, at, d_res,
+                                                       clusters_dev, vec);
+        };
+        if (dims == 3)
+            perc_batch_kernel<<<(unsigned)n, threads, smem, st>>>(g, thr, d_seeds, source, at,
+                                                                  d_res, clusters_dev);
+        else if (lanes == 1) blocks2d(perc_batch_blocked_kernel<1>);
+        else if (lanes == 2) blocks2d(perc_batch_blocked_kernel<2>);
+        else if (lanes == 4) blocks2d(perc_batch_blocked_kernel<4>);
+        else blocks2d(perc_batch_blocked_kernel<8>);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
