@@ -409,9 +409,12 @@ typedef struct ising_batch ising_batch; /* opaque */
 
 typedef struct ising_batch_opts {
     int block_threads;  /* threads per CTA: 128 or 256 (0: 256) */
-    int cluster_size;   /* CTAs per cluster for large lattices, 1..8 (0: 4);
-                           1 runs every lattice on a single CTA */
-    int64_t big_sites;  /* size threshold of the cluster queue (0: 2^18) */
+    int cluster_size;   /* CTAs per cluster for large lattices, 1..8; 1 runs every
+                           lattice on a single CTA.  0: large lattices advance
+                           together, one launch per colour pass of all of them
+                           (clusters of 4 in ising_batch_run_static) */
+    int64_t big_sites;  /* from how many sites a lattice counts as large (0: 2^18
+                           with clusters, 2^12 with joint passes) */
     int use_graph;      /* >= 0: capture the persistent launch in a CUDA graph and
                            replay it; < 0: plain launches */
     int64_t huge_sites; /* lattices this large use the per-lattice kernels

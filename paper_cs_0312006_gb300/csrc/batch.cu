@@ -4,10 +4,12 @@
 //
 // Lattices of at least huge_sites sites are advanced with the per-lattice
 // pass kernels (each pass spread over the whole GPU), issued on the batch's
-// stream ahead of the persistent launch; everything smaller goes through the
-// persistent kernel.
+// stream ahead of the rest.  When the caller leaves the cluster size open, the
+// large ones of the rest take joint passes (joint_pass_kernel: one launch per
+// colour pass of all of them) and the small ones the persistent kernel, a CTA
+// each; with a cluster size given, all go through the persistent kernel.
 //
-// Work queue: one job per lattice, holding everything its sweeps need (spin
+// Work queue of the persistent kernel: one job per lattice, holding everything its sweeps need (spin
 // arrays, thresholds, key, first sweep index, sweep count, measurement
 // interval, record slots).  Jobs are ordered by work (sites x sweeps),
 // largest first, and split in two queues at a size threshold:
@@ -69,6 +71,18 @@ static void fill_job(BatchJob& j, const ising_lattice* h, int64_t nsweeps, int e
     j.nsweeps = (int32_t)nsweeps;
     j.measure_every = every;
 }
+
+// From this many sites a lattice of a batch takes part in the joint passes; the
+// others run a CTA each, all their sweeps at once (256 mixed lattices: 4.0 ms
+// here, 4.2 from 2^14 sites on and 5.3 from 2^16, a CTA's slowest lattice then
+// outlasting the rest; 2^10 the same as here).
+constexpr int64_t kJointSites = 1 << 12;
+
+// A warp's share of a joint pass: the items of a job from `first` on.
+struct JointChunk {
+    int32_t job;
+    uint32_t first;
+};
 
 namespace {
 
@@ -146,9 +160,7 @@ __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom
     }
 }
 
-template <int DIMS, int LAYOUT, bool MEASURE, int NC, int RULE>
-__device__ __forceinline__ void job_pass(const BatchJob& j, int c, uint32_t t, uint32_t rank,
-                                         uint32_t nthr, int& e_acc, int& m_acc) {
+__device__ __forceinline__ PassArgs job_args(const BatchJob& j, int c, uint32_t t) {
     PassArgs a;
     a.own = c == 0 ? j.col0 : j.col1;
     a.other = c == 0 ? j.col1 : j.col0;
@@ -162,6 +174,14 @@ __device__ __forceinline__ void job_pass(const BatchJob& j, int c, uint32_t t, u
     a.key1 = j.key1;
     a.t = t;
     a.c = c;
+    return a;
+}
+
+template <int DIMS, int LAYOUT, bool MEASURE, int NC, int RULE>
+__device__ __forceinline__ void job_pass(const BatchJob& j, const PackedGeom& geom, int c,
+                                         uint32_t t, uint32_t rank, uint32_t nthr, int& e_acc,
+                                         int& m_acc) {
+    const PassArgs a = job_args(j, c, t);
     if (LAYOUT == ISING_INT8) {
         WordGeom g;
         g.W = (uint32_t)j.W;
@@ -185,12 +205,31 @@ __device__ __forceinline__ void job_pass(const BatchJob& j, int c, uint32_t t, u
         }
         if (MEASURE) m_acc += n_sites - 2 * m_neg;
     } else {
-        // rows grouped by their offset in a Philox group, so that a warp's
-        // words share it and take the five-call draws together
-        const uint32_t items = j.rows * (((uint32_t)j.W + 31u) >> 5);
-        const uint32_t rgroups = packed_row_groups((uint32_t)j.W);
-            for (uint32_t it = rank; it < items; it += nthr)
-            packed_word<DIMS, MEASURE, NC, RULE>(a, it, e_acc, m_acc, rgroups);
+        // (one body for aligned and ragged rows: at half the code the kernels
+        // spill less and stay in the instruction cache)
+        constexpr uint32_t step = kWarpWords<kDrawRagged>;
+        for (uint32_t first = (rank >> 5) * step; first < geom.items; first += (nthr >> 5) * step)
+            packed_words<DIMS, MEASURE, NC, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
+    }
+}
+
+// A warp's chunk of a joint pass (see joint_pass_kernel).
+template <int DIMS, int LAYOUT, bool MEASURE, int RULE>
+__device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom& geom, int c,
+                                            uint32_t t, uint32_t first, int& e_acc, int& m_acc) {
+    const PassArgs a = job_args(j, c, t);
+    if constexpr (LAYOUT == ISING_INT8) {
+        WordGeom g;
+        g.W = (uint32_t)j.W;
+        g.L = (uint32_t)j.L;
+        g.rows = j.rows;
+        g.half = j.half;
+        int m_neg = 0, n_sites = 0;
+        const uint32_t v = first + (threadIdx.x & 31u);
+        if (16u * v < j.half) int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_neg, n_sites);
+        if (MEASURE) m_acc += n_sites - 2 * m_neg;
+    } else {
+        packed_words<DIMS, MEASURE, 1, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
     }
 }
 
@@ -202,6 +241,12 @@ __device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader)
     // the 2048-lattice mix than reading through L2 only)
     constexpr int NC = 0;
     const BatchJob j = *jp;
+    // in shared memory: the kernel runs at its register cap
+    __shared__ PackedGeom geom;
+    if (LAYOUT == ISING_BITPACK) {
+        if (threadIdx.x == 0) geom = PackedGeom((uint32_t)j.W, (uint32_t)j.L, j.rows);
+        __syncthreads();
+    }
     int rec = 0;
     for (int s = 0; s < j.nsweeps; ++s) {
         const uint32_t t = j.t0 + (uint32_t)s;
@@ -209,9 +254,9 @@ __device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader)
         int e = 0, m = 0;
         for (int c = 0; c < 2; ++c) {
             if (measure)
-                job_pass<DIMS, LAYOUT, true, NC, RULE>(j, c, t, rank, nthr, e, m);
+                job_pass<DIMS, LAYOUT, true, NC, RULE>(j, geom, c, t, rank, nthr, e, m);
             else
-                job_pass<DIMS, LAYOUT, false, NC, RULE>(j, c, t, rank, nthr, e, m);
+                job_pass<DIMS, LAYOUT, false, NC, RULE>(j, geom, c, t, rank, nthr, e, m);
             group_sync<MODE>();  // this pass's writes before the next pass reads them
         }
         if (measure) {
@@ -278,6 +323,77 @@ __global__ void __launch_bounds__(256, RULE == kRuleHeatBath ? 2 : 3) batch_kern
     }
 }
 
+// One colour pass of many lattices in one launch (the large lattices of a
+// batch whose cluster size is left open).  A chunk is a warp's step of one job:
+// 31 or 32 words of a packed lattice, 32 16-site vectors of an int8 one.  Every
+// pass spreads over the whole GPU, so lattices of any mix finish together; a
+// cluster per lattice left the largest lattice on a few SMs long after the rest
+// were done.  50 sweeps of 256 mixed lattices: 11.5 ms with clusters of four,
+// 5.9 of eight, 4.0 in joint passes; of 64: 5.3, 2.4, 0.9; of 16: 4.1, 1.9, 0.7;
+// 100 sweeps of 2048, where clusters balance: 45.8, 43.0, 43.7.
+template <int RULE>
+__global__ void __launch_bounds__(256, RULE == kRuleHeatBath ? 2 : 3)
+    joint_pass_kernel(const BatchJob* __restrict__ jobs, const PackedGeom* __restrict__ geoms,
+                      const JointChunk* __restrict__ chunks, int n_chunks, uint32_t s, int c) {
+    const int lane = threadIdx.x & 31;
+    const int warps = (int)(gridDim.x * blockDim.x) >> 5;
+    int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    grid_dependency_wait();
+    launch_dependents();
+    for (; k < n_chunks; k += warps) {
+        const JointChunk ch = chunks[k];
+        const BatchJob& j = jobs[ch.job];
+        const uint32_t t = j.t0 + s;
+        // sweep t is recorded iff t + 1 is a multiple (t + 1 = 2^32 needs 64 bits)
+        const uint32_t every = (uint32_t)j.measure_every;
+        const bool measure = t + 1u != 0u ? (t + 1u) % every == 0u
+                                          : ((uint64_t)t + 1u) % (uint64_t)every == 0u;
+        int e = 0, m = 0;
+        auto run = [&](auto dims, auto layout) {
+            constexpr int D = decltype(dims)::value, Y = decltype(layout)::value;
+            if (measure)
+                joint_chunk<D, Y, true, RULE>(j, geoms[ch.job], c, t, ch.first, e, m);
+            else
+                joint_chunk<D, Y, false, RULE>(j, geoms[ch.job], c, t, ch.first, e, m);
+        };
+        using I8 = std::integral_constant<int, ISING_INT8>;
+        using BP = std::integral_constant<int, ISING_BITPACK>;
+        using D2 = std::integral_constant<int, 2>;
+        using D3 = std::integral_constant<int, 3>;
+        if (j.layout == ISING_BITPACK) {
+            if (j.dims == 2) run(D2{}, BP{});
+            else run(D3{}, BP{});
+        } else {
+            if (j.dims == 2) run(D2{}, I8{});
+            else run(D3{}, I8{});
+        }
+        if (measure) {
+            __syncwarp();
+            e = __reduce_add_sync(0xffffffffu, e);
+            m = __reduce_add_sync(0xffffffffu, m);
+            if (lane == 0) {
+                // the record's index among this launch's
+                const uint64_t rec = ((uint64_t)t + 1u) / every - (uint64_t)j.t0 / every - 1u;
+                unsigned long long* slot = j.obs + 2 * rec;
+                if (c == 1 && e != 0) atomicAdd(&slot[0], (unsigned long long)(long long)e);
+                if (m != 0) atomicAdd(&slot[1], (unsigned long long)(long long)m);
+            }
+        }
+    }
+}
+
+// After a launch's last joint pass: the jobs go on from here at the next.
+__global__ void joint_advance_kernel(BatchJob* jobs, const int* joint, int n) {
+    const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    grid_dependency_wait();
+    launch_dependents();
+    if (i >= n) return;
+    BatchJob& j = jobs[joint[i]];
+    const uint64_t every = (uint64_t)j.measure_every, t0 = j.t0;
+    j.obs += 2 * ((t0 + (uint64_t)j.nsweeps) / every - t0 / every);
+    j.t0 = (uint32_t)(t0 + (uint64_t)j.nsweeps);
+}
+
 using BatchKernel = void (*)(BatchJob*, const int*, int, const int*, int, int*);
 
 BatchKernel batch_kernel_for(int rule) {
@@ -334,6 +450,14 @@ struct RuleQueues {
     int grid = 0;  // resident CTAs of that rule's kernel
 };
 
+// The jointly passed lattices of one update rule: their chunks, longest sweep
+// counts first, and how many of the chunks take part in each sweep.
+struct JointQueue {
+    int offset = 0, n_chunks = 0;
+    int64_t max_sweeps = 0;
+    std::vector<std::pair<int64_t, int>> active;  // (sweeps, chunks of jobs with as many)
+};
+
 #define ISING_BCHECK(call)                                  \
     do {                                                    \
         cudaError_t e_ = (call);                            \
@@ -358,6 +482,17 @@ struct ising_batch {
     int* d_counters = nullptr;   // two per rule
     RuleQueues q[2];             // [ISING_RULE_METROPOLIS], [ISING_RULE_HEATBATH]
     int grid[2] = {0, 0};        // resident CTAs of each rule's kernel (0: not yet known)
+    bool joint = false;          // large lattices in joint passes (opts.cluster_size was 0)
+    std::vector<int> joint_jobs[2];  // [rule]
+    JointQueue jq[2];
+    JointChunk* d_chunks = nullptr;
+    JointChunk* h_chunks = nullptr;  // pinned mirror
+    int* d_joint = nullptr;      // the joint jobs, both rules
+    int* h_joint = nullptr;
+    PackedGeom* d_geoms = nullptr;
+    PackedGeom* h_geoms = nullptr;
+    int chunk_cap = 0, joint_cap = 0;
+    int n_chunks = 0, n_joint = 0;
     std::vector<int> rule;       // each lattice's rule when the batch was made
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t uploaded = nullptr;
@@ -387,7 +522,21 @@ int queued_jobs(const ising_batch* b) {
     return b->q[0].n_big + b->q[0].n_small + b->q[1].n_big + b->q[1].n_small;
 }
 
+void free_joint(ising_batch* b) {
+    if (b->d_chunks) cudaFreeAsync(b->d_chunks, b->stream);
+    if (b->d_joint) cudaFreeAsync(b->d_joint, b->stream);
+    if (b->d_geoms) cudaFreeAsync(b->d_geoms, b->stream);
+    if (b->h_chunks) cudaFreeHost(b->h_chunks);
+    if (b->h_joint) cudaFreeHost(b->h_joint);
+    if (b->h_geoms) cudaFreeHost(b->h_geoms);
+    b->d_chunks = b->h_chunks = nullptr;
+    b->d_joint = b->h_joint = nullptr;
+    b->d_geoms = b->h_geoms = nullptr;
+    b->chunk_cap = b->joint_cap = 0;
+}
+
 void free_batch(ising_batch* b) {
+    free_joint(b);
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->uploaded) cudaEventDestroy(b->uploaded);
     if (b->d_jobs) cudaFreeAsync(b->d_jobs, b->stream);
@@ -396,6 +545,107 @@ void free_batch(ising_batch* b) {
     if (b->h_jobs) cudaFreeHost(b->h_jobs);
     if (b->h_order) cudaFreeHost(b->h_order);
     delete b;
+}
+
+// Items of a lattice in a joint pass, and how many a warp takes at a time.
+uint32_t joint_items(const ising_lattice* h, uint32_t* step) {
+    if (h->layout == ISING_BITPACK) {
+        const PackedGeom g((uint32_t)h->W, (uint32_t)h->L, (uint32_t)h->rows);
+        *step = kWarpWords<kDrawRagged>;
+        return g.items;
+    }
+    *step = 32u;
+    return (uint32_t)((h->half_sites + 15) >> 4);
+}
+
+// The chunk and geometry tables of the joint jobs, in the pinned mirrors,
+// longest sweep counts first.
+int joint_tables(ising_batch* b) {
+    b->n_chunks = b->n_joint = 0;
+    size_t chunks = 0, joint = 0;
+    for (int r = 0; r < 2; ++r) {
+        std::stable_sort(b->joint_jobs[r].begin(), b->joint_jobs[r].end(),
+                         [&](int x, int y) { return b->sweeps[x] > b->sweeps[y]; });
+        joint += b->joint_jobs[r].size();
+        for (int i : b->joint_jobs[r]) {
+            uint32_t step = 0;
+            const uint32_t items = joint_items(b->lats[i], &step);
+            chunks += (items + step - 1u) / step;
+        }
+    }
+    if (joint == 0) return ISING_OK;
+    if (chunks > 0x7FFFFFFF) return ISING_EINVAL;
+    // the mirrors may still be the source of a queued upload
+    if (b->uploaded) ISING_BCHECK(cudaEventSynchronize(b->uploaded));
+    if ((int)chunks > b->chunk_cap || (int)b->lats.size() > b->joint_cap) {
+        free_joint(b);
+        const size_t n = b->lats.size();
+        ISING_BCHECK(pool_alloc(reinterpret_cast<void**>(&b->d_chunks),
+                                sizeof(JointChunk) * chunks, *b->dp, b->stream));
+        ISING_BCHECK(pool_alloc(reinterpret_cast<void**>(&b->d_joint), sizeof(int) * n, *b->dp,
+                                b->stream));
+        ISING_BCHECK(pool_alloc(reinterpret_cast<void**>(&b->d_geoms), sizeof(PackedGeom) * n,
+                                *b->dp, b->stream));
+        ISING_BCHECK(cudaMallocHost(reinterpret_cast<void**>(&b->h_chunks),
+                                    sizeof(JointChunk) * chunks));
+        ISING_BCHECK(cudaMallocHost(reinterpret_cast<void**>(&b->h_joint), sizeof(int) * n));
+        ISING_BCHECK(cudaMallocHost(reinterpret_cast<void**>(&b->h_geoms),
+                                    sizeof(PackedGeom) * n));
+        b->chunk_cap = (int)chunks;
+        b->joint_cap = (int)n;
+    }
+    for (int r = 0; r < 2; ++r) {
+        JointQueue& q = b->jq[r];
+        q.offset = b->n_chunks;
+        q.n_chunks = 0;
+        q.max_sweeps = 0;
+        q.active.clear();
+        for (int i : b->joint_jobs[r]) {
+            const ising_lattice* h = b->lats[i];
+            b->h_joint[b->n_joint++] = i;
+            b->h_geoms[i] = PackedGeom((uint32_t)h->W, (uint32_t)h->L, (uint32_t)h->rows);
+            uint32_t step = 0;
+            const uint32_t items = joint_items(h, &step);
+            for (uint32_t first = 0; first < items; first += step) {
+                b->h_chunks[q.offset + q.n_chunks] = JointChunk{i, first};
+                ++q.n_chunks;
+            }
+            if (b->sweeps[i] > q.max_sweeps) q.max_sweeps = b->sweeps[i];
+            if (!q.active.empty() && q.active.back().first == b->sweeps[i])
+                q.active.back().second = q.n_chunks;
+            else
+                q.active.emplace_back(b->sweeps[i], q.n_chunks);
+        }
+        b->n_chunks += q.n_chunks;
+    }
+    return ISING_OK;
+}
+
+// The joint passes of one launch: sweep s of every job with more than s sweeps.
+cudaError_t launch_joint(ising_batch* b) {
+    for (int r = 0; r < 2; ++r) {
+        const JointQueue& q = b->jq[r];
+        if (b->joint_jobs[r].empty()) continue;
+        const int cap = b->dp->sm_count * (r == ISING_RULE_HEATBATH ? 2 : 3);
+        size_t last = q.active.size();  // the entries before it have sweeps > s
+        for (int64_t s = 0; s < q.max_sweeps; ++s) {
+            while (last > 0 && q.active[last - 1].first <= s) --last;
+            const int n = q.active[last - 1].second;
+            const int grid = (n + 7) / 8 < cap ? (n + 7) / 8 : cap;
+            for (int c = 0; c < 2; ++c) {
+                const cudaError_t e = launch_chained(
+                    r == ISING_RULE_HEATBATH ? joint_pass_kernel<kRuleHeatBath>
+                                             : joint_pass_kernel<kRuleMetropolis>,
+                    (unsigned)grid, 256u, 0, b->stream, static_cast<const BatchJob*>(b->d_jobs),
+                    static_cast<const PackedGeom*>(b->d_geoms),
+                    static_cast<const JointChunk*>(b->d_chunks + q.offset), n, (uint32_t)s, c);
+                if (e != cudaSuccess) return e;
+            }
+        }
+    }
+    if (b->n_joint == 0) return cudaSuccess;
+    return launch_chained(joint_advance_kernel, (unsigned)((b->n_joint + 255) / 256), 256u, 0,
+                          b->stream, b->d_jobs, static_cast<const int*>(b->d_joint), b->n_joint);
 }
 
 // Arguments of a batch's lattice list: valid handles, each at most once.
@@ -429,6 +679,7 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
     b->every.resize(n);
     for (int i = 0; i < n; ++i) b->every[i] = measure_every ? measure_every[i] : 1;
     std::vector<int> big[2], small[2];
+    for (auto& v : b->joint_jobs) v.clear();
     b->huge.clear();
     b->in_table.assign(n, 1);
     b->rule.resize(n);
@@ -442,7 +693,10 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
             b->huge.push_back(i);
             b->in_table[i] = 0;
         } else {
-            (o.cluster_size > 1 && b->lats[i]->sites >= o.big_sites ? big[r] : small[r])
+            const bool large = b->lats[i]->sites >= o.big_sites;
+            (b->joint && large                 ? b->joint_jobs[r]
+             : o.cluster_size > 1 && large ? big[r]
+                                           : small[r])
                 .push_back(i);
         }
     }
@@ -491,6 +745,8 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
         b->grid[r] = clusters * o.cluster_size;
         b->q[r].grid = b->grid[r];
     }
+    const int rc = joint_tables(b);
+    if (rc != ISING_OK) return rc;
     if (b->exec) {  // the captured launch holds the old queue sizes
         cudaGraphExecDestroy(b->exec);
         b->exec = nullptr;
@@ -511,13 +767,19 @@ int ising_batch_create(ising_batch** out, ising_lattice* const* lats, int n,
     *out = nullptr;
     ising_batch_opts o = {};
     if (opts) o = *opts;
+    const bool joint = o.cluster_size == 0;
     if (o.block_threads == 0) o.block_threads = 256;
-    if (o.cluster_size == 0) o.cluster_size = 4;
-    if (o.big_sites == 0) o.big_sites = 1 << 18;
+    if (joint) o.cluster_size = 1;  // what is left runs a CTA each
+    if (o.big_sites == 0) o.big_sites = joint ? kJointSites : 1 << 18;
     if (o.huge_sites == 0) o.huge_sites = (int64_t)1 << 22;
     if (o.block_threads != 128 && o.block_threads != 256) return ISING_EINVAL;
     if (o.cluster_size < 1 || o.cluster_size > 8) return ISING_EINVAL;
-    int rc = check_members(lats, n, sweeps, measure_every);
+    int rc = ISING_OK;
+    try {
+        rc = check_members(lats, n, sweeps, measure_every);
+    } catch (const std::bad_alloc&) {
+        return ISING_ENOMEM;
+    }
     if (rc != ISING_OK) return rc;
     const DeviceProps* dp = nullptr;
     rc = device_props(&dp);
@@ -525,6 +787,7 @@ int ising_batch_create(ising_batch** out, ising_lattice* const* lats, int n,
     ising_batch* b = new (std::nothrow) ising_batch();
     if (!b) return ISING_ENOMEM;
     b->opts = o;
+    b->joint = joint;
     b->dp = dp;
     b->stream = static_cast<cudaStream_t>(stream);
     cudaError_t e = pool_alloc(reinterpret_cast<void**>(&b->d_counters), 4 * sizeof(int), *dp,
@@ -534,7 +797,11 @@ int ising_batch_create(ising_batch** out, ising_lattice* const* lats, int n,
         free_batch(b);
         return cuda_fail(e);
     }
-    rc = assign_members(b, lats, n, sweeps, measure_every);
+    try {
+        rc = assign_members(b, lats, n, sweeps, measure_every);
+    } catch (const std::bad_alloc&) {
+        rc = ISING_ENOMEM;
+    }
     if (rc != ISING_OK) {
         free_batch(b);
         return rc;
@@ -546,9 +813,13 @@ int ising_batch_create(ising_batch** out, ising_lattice* const* lats, int n,
 int ising_batch_update(ising_batch* b, ising_lattice* const* lats, int n, const int64_t* sweeps,
                        const int* measure_every) {
     if (!b) return ISING_EINVAL;
-    const int rc = check_members(lats, n, sweeps, measure_every);
-    if (rc != ISING_OK) return rc;
-    return assign_members(b, lats, n, sweeps, measure_every);
+    try {
+        const int rc = check_members(lats, n, sweeps, measure_every);
+        if (rc != ISING_OK) return rc;
+        return assign_members(b, lats, n, sweeps, measure_every);
+    } catch (const std::bad_alloc&) {
+        return ISING_ENOMEM;
+    }
 }
 
 int ising_batch_launch(ising_batch* b) {
@@ -583,6 +854,15 @@ int ising_batch_launch(ising_batch* b) {
     if (moved || b->order_dirty) {
         ISING_BCHECK(cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(BatchJob) * (size_t)n,
                                      cudaMemcpyHostToDevice, b->stream));
+        if (b->order_dirty && b->n_joint > 0) {
+            ISING_BCHECK(cudaMemcpyAsync(b->d_chunks, b->h_chunks,
+                                         sizeof(JointChunk) * (size_t)b->n_chunks,
+                                         cudaMemcpyHostToDevice, b->stream));
+            ISING_BCHECK(cudaMemcpyAsync(b->d_joint, b->h_joint, sizeof(int) * (size_t)b->n_joint,
+                                         cudaMemcpyHostToDevice, b->stream));
+            ISING_BCHECK(cudaMemcpyAsync(b->d_geoms, b->h_geoms, sizeof(PackedGeom) * (size_t)n,
+                                         cudaMemcpyHostToDevice, b->stream));
+        }
         if (b->order_dirty && !b->order.empty()) {  // empty when every lattice is huge
             std::memcpy(b->h_order, b->order.data(), sizeof(int) * b->order.size());
             ISING_BCHECK(cudaMemcpyAsync(b->d_order, b->h_order, sizeof(int) * b->order.size(),
@@ -608,6 +888,7 @@ int ising_batch_launch(ising_batch* b) {
         cudaStreamDestroy(cap);
         if (e != cudaSuccess) return cuda_fail(e);
     }
+    ISING_BCHECK(launch_joint(b));
     if (queued_jobs(b) > 0) {
         if (b->exec)
             ISING_BCHECK(cudaGraphLaunch(b->exec, b->stream));
@@ -662,8 +943,11 @@ int ising_batch_run(ising_lattice* const* lats, int n, const int64_t* sweeps, in
 
 int ising_batch_info(const ising_batch* b, int* grid, int* n_big, int* n_small, int* n_huge) {
     if (!b) return ISING_EINVAL;
-    if (grid) *grid = b->q[0].grid > b->q[1].grid ? b->q[0].grid : b->q[1].grid;
-    if (n_big) *n_big = b->q[0].n_big + b->q[1].n_big;
+    if (grid) {
+        *grid = b->q[0].grid > b->q[1].grid ? b->q[0].grid : b->q[1].grid;
+        if (b->n_joint > 0) *grid = std::max(*grid, b->dp->sm_count * 3);
+    }
+    if (n_big) *n_big = b->q[0].n_big + b->q[1].n_big + b->n_joint;
     if (n_small) *n_small = b->q[0].n_small + b->q[1].n_small;
     if (n_huge) *n_huge = (int)b->huge.size();
     return ISING_OK;

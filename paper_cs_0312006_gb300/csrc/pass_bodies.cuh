@@ -557,22 +557,6 @@ __device__ __forceinline__ Digits digits3(uint32_t a, uint32_t b, uint32_t c, ui
     return Digits{s1 ^ s2, k1 ^ k2 ^ k0, (k1 & k2) | (k0 & (k1 ^ k2))};
 }
 
-// Threshold of bit b: Metropolis, for a site with dE > 0 (d < dims) ...
-template <int DIMS>
-__device__ __forceinline__ uint32_t site_threshold(const Counts& k, int b, const PassArgs& a) {
-    if (DIMS == 2) return (k.eq0 >> b) & 1u ? a.thr[1] : a.thr[0];
-    return (k.eq0 >> b) & 1u ? a.thr[2] : ((k.eq1 >> b) & 1u ? a.thr[1] : a.thr[0]);
-}
-
-// ... and heat bath, thr[d] for any d.
-template <int DIMS>
-__device__ __forceinline__ uint32_t site_threshold(const Digits& k, int b, const PassArgs& a) {
-    const bool d0 = (k.d0 >> b) & 1u, d1 = (k.d1 >> b) & 1u, d2 = (k.d2 >> b) & 1u;
-    const uint32_t lo = d1 ? (d0 ? a.thr[3] : a.thr[2]) : (d0 ? a.thr[1] : a.thr[0]);
-    const uint32_t hi = DIMS == 2 ? a.thr[4] : (d1 ? a.thr[6] : (d0 ? a.thr[5] : a.thr[4]));
-    return d2 ? hi : lo;
-}
-
 // Thresholds of a rule: the Metropolis dims, or the heat bath's 2 dims + 1.
 template <int DIMS, int RULE>
 constexpr int kThresholds = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
@@ -588,51 +572,30 @@ constexpr int kThresholds = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
 // Tests as saturating fp32 multiply-adds, off the integer pipes, took 26: a
 // multiply-add costs an issue slot like a compare.
 //
-// The draws of 16 sites (one half of a packed word) against all N thresholds:
-// bit 16 HALF + b of A[n] is set iff site b's draw lies below threshold n.
-// The word's first bit is half index 4 g0 + M (M = 0..3: where the row starts
-// inside a Philox group), so site b takes draw (M + b) & 3 of group
-// g0 + 4 HALF + ((M + b) >> 2): four calls, or five when M != 0, made together.
-template <int N, int M, int HALF>
-__device__ __forceinline__ void half_tests(uint32_t g0, const PassArgs& a, uint32_t c2,
+// The draws of the Philox groups g0 .. g0 + 7 against all N thresholds: bit b of
+// A[n] is set iff draw b (word b & 3 of group g0 + (b >> 2)) lies below
+// threshold n.  Four calls at a time; without `both`, bits 16..31 stay clear.
+template <int N>
+__device__ __forceinline__ void word_tests(uint32_t g0, const PassArgs& a, uint32_t c2, bool both,
                                            uint32_t (&A)[N]) {
-    PhiloxRuns<1, M == 0 ? 4 : 5> ps;
-    const uint32_t base[1] = {g0 + (uint32_t)(4 * HALF)};
-    ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
 #pragma unroll
-    for (int r = 1; r < 10; ++r) ps.next_round();
-    static_for<16>([&](auto bit) {
-        constexpr int b = decltype(bit)::value, j = (M + b) & 3;
-        const Philox4 u = ps.result((M + b) >> 2);
-        const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
+    for (int n = 0; n < N; ++n) A[n] = 0u;
+    static_for<2>([&](auto half) {
+        constexpr int h = decltype(half)::value;
+        if (h == 1 && !both) return;
+        PhiloxRuns<1> ps;
+        const uint32_t base[1] = {g0 + 4u * h};
+        ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
 #pragma unroll
-        for (int n = 0; n < N; ++n) mark_below<(1u << (16 * HALF + b))>(A[n], w, a.thr[n]);
+        for (int r = 1; r < 10; ++r) ps.next_round();
+        static_for<16>([&](auto bit) {
+            constexpr int b = decltype(bit)::value, j = b & 3;
+            const Philox4 u = ps.result(b >> 2);
+            const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
+#pragma unroll
+            for (int n = 0; n < N; ++n) mark_below<(1u << (16 * h + b))>(A[n], w, a.thr[n]);
+        });
     });
-}
-
-// Accept mask of the `need` bits, one Philox call at a time: where the lanes
-// of a warp start at different offsets m inside their groups.
-template <int DIMS, typename K>
-__device__ __forceinline__ uint32_t packed_accept_mixed(const K& k, uint32_t need, uint32_t m,
-                                                        uint32_t g0, const PassArgs& a,
-                                                        uint32_t c2) {
-    uint32_t acc = 0u;
-#pragma unroll 1
-    for (int g = 0; g < 9; ++g) {
-        const int lo = 4 * g - (int)m;  // bit of the group's word 0 (may be < 0)
-        if (lo > 31) break;
-        const uint32_t gmask = lo >= 0 ? (0xFu << lo) : (0xFu >> (-lo));
-        if (!(need & gmask)) continue;
-        const Philox4 u = philox4x32_10(g0 + (uint32_t)g, a.t, c2, kTagSweep, a.key0, a.key1);
-        const uint32_t w[4] = {u.w0, u.w1, u.w2, u.w3};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int b = lo + j;
-            if (b < 0 || b > 31) continue;
-            acc |= (w[j] < site_threshold<DIMS>(k, b, a) ? 1u : 0u) << b;
-        }
-    }
-    return acc;
 }
 
 // Each site's answer for the threshold of its own number of disagreeing
@@ -656,48 +619,41 @@ __device__ __forceinline__ uint32_t choose_answer(const Digits& k,
     return (k.d2 & hi) | (~k.d2 & lo);
 }
 
-// ALL: draw for both halves in one straight line (a full word of a lattice
-// where nearly every half holds a site that draws); else a half without a
-// site that draws, such as the one past a short row's end, is passed over.
-template <int DIMS, int RULE, int M, bool ALL, typename K>
-__device__ __forceinline__ uint32_t packed_accept_at(const K& k, uint32_t need, uint32_t g0,
-                                                     const PassArgs& a, uint32_t c2) {
+// How the words of a lattice draw (the whole warp takes part in a word's
+// tests, each lane for its own word).
+constexpr int kDrawAligned = 0;  // every row starts on a Philox group
+constexpr int kDrawRagged = 1;   // rows start anywhere in a group
+// Words a warp takes at a time.
+template <int DRAW>
+constexpr uint32_t kWarpWords = DRAW == kDrawRagged ? 31u : 32u;
+
+// Accept mask of a packed word whose 32 bits are the half indices hbase + b:
+// bit b's draw is word (hb & 3) of Philox group hb >> 2.  A row that starts
+// inside a group (hbase & 3 = M != 0) needs nine groups' draws 0..35 and uses
+// draws M .. M + 31: the tests stay at draw positions, the same code for every
+// M, the last four positions are the next lane's first four (its word starts
+// with the ninth group: words follow one another in h, and where a row's last
+// word is shorter than 32 - M sites the ninth group is not needed), and one
+// funnel shift per threshold moves the answers to their sites.  So a ragged
+// word costs eight calls like an aligned one; the last lane of the warp only
+// lends its draws (packed_words).  Against five calls per half, with the code
+// compiled per M and the rows grouped by M, and with divisions for an item's
+// place: 3D L = 202 11.0 -> 8.6 us per pass; a joint pass of 256 mixed lattices
+// 47 -> 39 us.
+template <int DIMS, int RULE, int DRAW, typename K>
+__device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t hbase, bool both,
+                                                  const PassArgs& a, uint32_t c2) {
     constexpr int N = kThresholds<DIMS, RULE>;
     uint32_t A[N];
+    word_tests<N>(hbase >> 2, a, c2, both, A);
+    if constexpr (DRAW == kDrawRagged) {
 #pragma unroll
-    for (int n = 0; n < N; ++n) A[n] = 0u;
-    if (ALL || (need & 0xFFFFu)) half_tests<N, M, 0>(g0, a, c2, A);
-    if (ALL || (need >> 16)) half_tests<N, M, 1>(g0, a, c2, A);
-    return choose_answer<DIMS>(k, A);
-}
-
-// Accept mask of the `need` bits of a packed word (Metropolis: the sites with
-// dE > 0; heat bath: every valid site) whose 32 bits are the half indices
-// hb = hbase + b (b = 0..31).  Bit b's draw is word (hb & 3) of Philox group
-// hb >> 2: eight groups when hbase is a multiple of 4, nine when a row starts
-// inside a group (W not a multiple of 4).  The offset is a compile-time
-// constant in each path, taken when the lanes of the warp share it.
-// ALIGNED: the caller knows hbase % 4 == 0 (rows of a multiple of 32 sites),
-// so only the eight-group path is compiled.
-template <int DIMS, int RULE, bool ALIGNED, typename K>
-__device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t need,
-                                                  uint32_t hbase, const PassArgs& a,
-                                                  uint32_t c2) {
-    const uint32_t g0 = hbase >> 2;
-    if constexpr (ALIGNED) {
-        return packed_accept_at<DIMS, RULE, 0, true>(k, need, g0, a, c2);
-    } else {
-        const uint32_t m = hbase & 3u;
-        if (m == 0u) return packed_accept_at<DIMS, RULE, 0, false>(k, need, g0, a, c2);
-        const uint32_t lanes = __activemask();
-        const uint32_t m0 = __shfl_sync(lanes, m, __ffs(lanes) - 1);
-        if (__all_sync(lanes, m == m0)) {
-            if (m == 1u) return packed_accept_at<DIMS, RULE, 1, false>(k, need, g0, a, c2);
-            if (m == 2u) return packed_accept_at<DIMS, RULE, 2, false>(k, need, g0, a, c2);
-            return packed_accept_at<DIMS, RULE, 3, false>(k, need, g0, a, c2);
+        for (int n = 0; n < N; ++n) {
+            const uint32_t next = __shfl_down_sync(0xffffffffu, A[n], 1);
+            A[n] = __funnelshift_r(A[n], next, hbase & 3u);
         }
-        return packed_accept_mixed<DIMS>(k, need, m, g0, a, c2);
     }
+    return choose_answer<DIMS>(k, A);
 }
 
 // Update word (r, q) of the packed colour array.  A half row of W sites takes
@@ -705,80 +661,79 @@ __device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t need,
 // when xh < W; the other bits of a row's last word stay 0 and never flip).
 // The x-neighbour wrap at the row ends comes from the row's last valid bit
 // (p = 0, first word) or first bit (p = 1, last word).
-//
-// With rgroups > 1 the items visit the rows grouped by r mod rgroups: every
-// row of a group starts at the same offset inside a Philox group (r W mod 4
-// depends only on r mod 4 for odd W, on r mod 2 for W = 2 mod 4), so the lanes
-// of a warp share it and take the five-call path together instead of
-// diverging over all four offsets.  Group c holds rows c, c + rgroups, ...
-// (the first rows mod rgroups groups one row more).
-__host__ __device__ __forceinline__ uint32_t packed_row_groups(uint32_t W) {
-    return (W & 1u) ? 4u : ((W & 3u) == 2u ? 2u : 1u);
-}
 
-__device__ __forceinline__ uint32_t grouped_row(uint32_t j, uint32_t rows, uint32_t rgroups) {
-    const uint32_t G = rows / rgroups, rem = rows - G * rgroups;
-    const uint32_t head = rem * (G + 1u);  // rows in the longer groups
-    uint32_t c, k;
-    if (j < head) {
-        c = j / (G + 1u);
-        k = j - c * (G + 1u);
-    } else {
-        const uint32_t jj = j - head;
-        c = G ? jj / G : 0u;
-        k = jj - c * G;
-        c += rem;
+// Quotients by a fixed divisor d >= 1 of n < 2^31: with 2^s <= d < 2^(s+1) and
+// m = ceil(2^(32+s) / d), n m / 2^(32+s) exceeds n / d by less than
+// n / 2^31 / d, too little to reach the next integer.  Powers of two take
+// half of both, and d = 1 the last term.  Six issue slots instead of the twenty
+// or so of a division, of which a packed word of ragged rows needs four.
+struct FastDiv {
+    uint32_t d, m, s, one;
+    FastDiv() = default;
+    __host__ __device__ __forceinline__ explicit FastDiv(uint32_t div) : d(div), s(0), one(0) {
+        while ((2u << s) <= d && s < 31u) ++s;
+        if (d == 1u) {
+            m = 0u;
+            one = 0xFFFFFFFFu;
+        } else if ((d & (d - 1u)) == 0u) {
+            m = 0x80000000u;
+            --s;
+        } else {
+            m = (uint32_t)(((1ull << (32u + s)) + d - 1u) / d);
+        }
     }
-    return k * rgroups + c;
-}
+    __device__ __forceinline__ uint32_t quot(uint32_t n) const {
+        return (__umulhi(n, m) >> s) + (n & one);
+    }
+};
+
+// The geometry of a packed lattice's words.
+struct PackedGeom {
+    uint32_t items;    // words per colour
+    FastDiv words, L;  // words per half row, L
+    PackedGeom() = default;
+    __host__ __device__ __forceinline__ PackedGeom(uint32_t W, uint32_t L_, uint32_t rows)
+        : words((W + 31u) >> 5), L(L_) {
+        items = rows * words.d;
+    }
+};
 
 // The rule applied to one packed word, given the word s and its neighbour
 // words (sh: the x-neighbour across the colour, shifted into place), then the
 // store and the word's share of E and M.  valid: the word's sites (nb bits);
-// hbase: the half index of bit 0 (its Philox draw is word hbase & 3 of group
-// hbase >> 2).  ALIGNED: hbase % 4 == 0 is known (packed_accept).
-template <int DIMS, bool MEASURE, int RULE, bool ALIGNED>
-__device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_word, uint32_t s,
+// hbase: the half index of bit 0.  The whole warp takes part; a lane without
+// `mine` stores and counts nothing.
+template <int DIMS, bool MEASURE, int RULE, int DRAW>
+__device__ __forceinline__ void packed_update(const PassArgs& a, bool mine, bool both,
+                                              uint32_t* own_word, uint32_t s,
                                               uint32_t o, uint32_t sh, uint32_t oym,
                                               uint32_t oyp, uint32_t ozm, uint32_t ozp,
                                               uint32_t valid, uint32_t nb, uint32_t hbase,
                                               int& e_acc, int& m_acc) {
     uint32_t flip;
-    if constexpr (RULE == kRuleHeatBath) {  // every valid site draws
+    if constexpr (RULE == kRuleHeatBath) {
         const Digits k = DIMS == 2 ? digits2(s ^ o, s ^ sh, s ^ oym, s ^ oyp)
                                    : digits3(s ^ o, s ^ sh, s ^ oym, s ^ oyp, s ^ ozm, s ^ ozp);
-        flip = packed_accept<DIMS, RULE, ALIGNED>(k, valid, hbase, a, (uint32_t)a.c);
-    } else if constexpr (RULE == kRuleMultiHit) {  // a.hits trials, neighbours fixed
+        flip = packed_accept<DIMS, RULE, DRAW>(k, hbase, both, a, (uint32_t)a.c);
+    } else {
+        // one Metropolis trial, or a.hits in a row with the neighbours fixed
+        const int hits = RULE == kRuleMultiHit ? a.hits : 1;
         uint32_t cur = s;
 #pragma unroll 1
-        for (int m = 0; m < a.hits; ++m) {
+        for (int m = 0; m < hits; ++m) {
             Counts k;
             if (DIMS == 2) {
                 k = count2(cur ^ o, cur ^ sh, cur ^ oym, cur ^ oyp);
             } else {
                 k = count3(cur ^ o, cur ^ sh, cur ^ oym, cur ^ oyp, cur ^ ozm, cur ^ ozp);
             }
-            uint32_t f = k.always;
-            const uint32_t need = ~k.always & valid;
-            if (need)
-                f |= packed_accept<DIMS, RULE, ALIGNED>(k, need, hbase, a,
-                                                        (uint32_t)a.c + 2u * (uint32_t)m);
-            cur ^= f & valid;
+            cur ^= k.always | packed_accept<DIMS, RULE, DRAW>(k, hbase, both, a,
+                                                              (uint32_t)a.c + 2u * (uint32_t)m);
         }
         flip = cur ^ s;
-    } else {
-        Counts k;
-        if (DIMS == 2) {
-            k = count2(s ^ o, s ^ sh, s ^ oym, s ^ oyp);
-        } else {
-            k = count3(s ^ o, s ^ sh, s ^ oym, s ^ oyp, s ^ ozm, s ^ ozp);
-        }
-        flip = k.always;
-        const uint32_t need = ~k.always & valid;
-        if (ALIGNED || need)
-            flip |= packed_accept<DIMS, RULE, ALIGNED>(k, need, hbase, a, (uint32_t)a.c);
     }
     const uint32_t snew = s ^ (flip & valid);
+    if (!mine) return;
     *own_word = snew;
     if (MEASURE) {
         m_acc += 2 * __popc(snew & valid) - (int)nb;
@@ -791,32 +746,50 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, uint32_t* own_w
     }
 }
 
-template <int DIMS, bool MEASURE, int NC, int RULE>
-__device__ __forceinline__ void packed_word(const PassArgs& a, uint32_t item, int& e_acc,
-                                            int& m_acc, uint32_t rgroups) {
+// A warp's next words of the packed colour array: items first .. first + 31,
+// the lane's own at first + lane.  A half row of W sites takes nq = ceil(W / 32)
+// words; bit b of word q is half column xh = 32q + b (valid when xh < W; the
+// other bits of a row's last word stay 0 and never flip).  The x-neighbour wrap
+// at the row ends comes from the row's last valid bit (p = 0, first word) or
+// first bit (p = 1, last word).  With ragged draws lane 31 only lends its draws,
+// for lane 30's last sites, and its word is the first of the next step; a lane
+// past the end draws for the row after the last.
+template <int DIMS, bool MEASURE, int NC, int RULE, int DRAW>
+__device__ __forceinline__ void packed_words(const PassArgs& a, const PackedGeom& g,
+                                             uint32_t first, int& e_acc, int& m_acc) {
     const uint32_t W = (uint32_t)a.W;
-    const uint32_t nq = (W + 31u) >> 5;
+    const uint32_t nq = g.words.d;
     const uint32_t L = (uint32_t)a.L;
     uint32_t* own = static_cast<uint32_t*>(a.own);
     const uint32_t* other = static_cast<const uint32_t*>(a.other);
-    const uint32_t j = item / nq, q = item - j * nq;
-    const uint32_t r = rgroups > 1u ? grouped_row(j, (uint32_t)a.rows, rgroups) : j;
+    const uint32_t lane = threadIdx.x & 31u, item = first + lane;
+    const bool mine = item < g.items && lane < kWarpWords<DRAW>;
+    uint32_t r = g.words.quot(item), q = item - r * nq;
+    const uint32_t hbase = r * W + 32u * q;
+    if (item >= g.items) {  // loads something, keeps nothing
+        r = (uint32_t)a.rows - 1u;
+        q = 0u;
+    }
     uint32_t y = r, z = 0;
     if (DIMS == 3) {
-        z = r / L;
+        z = g.L.quot(r);
         y = r - z * L;
     }
     const uint32_t nb = W - 32u * q < 32u ? W - 32u * q : 32u;  // valid bits
     const uint32_t valid = nb == 32u ? 0xFFFFFFFFu : ((1u << nb) - 1u);
-    const uint32_t plane = z * L;
     const uint32_t row = r * nq;
-    const uint32_t o = load_other<NC>(other + row + q);
-    const uint32_t oym = load_other<NC>(other + (plane + (y == 0u ? L - 1u : y - 1u)) * nq + q);
-    const uint32_t oyp = load_other<NC>(other + (plane + (y + 1u == L ? 0u : y + 1u)) * nq + q);
+    // the rows (and planes) next to this one, as offsets from it
+    const uint32_t up = (y == 0u ? (L - 1u) * nq : 0u - nq);
+    const uint32_t down = (y + 1u == L ? 0u - (L - 1u) * nq : nq);
+    const uint32_t* at = other + row + q;
+    const uint32_t o = load_other<NC>(at);
+    const uint32_t oym = load_other<NC>(at + (int32_t)up);
+    const uint32_t oyp = load_other<NC>(at + (int32_t)down);
     uint32_t ozm = 0u, ozp = 0u;
     if (DIMS == 3) {
-        ozm = load_other<NC>(other + ((z == 0u ? L - 1u : z - 1u) * L + y) * nq + q);
-        ozp = load_other<NC>(other + ((z + 1u == L ? 0u : z + 1u) * L + y) * nq + q);
+        const uint32_t plane = L * nq;
+        ozm = load_other<NC>(at + (int32_t)(z == 0u ? (L - 1u) * plane : 0u - plane));
+        ozp = load_other<NC>(at + (int32_t)(z + 1u == L ? 0u - (L - 1u) * plane : plane));
     }
     const uint32_t s = own[row + q];
     const int p = (a.c + (int)y + (int)z) & 1;
@@ -824,23 +797,24 @@ __device__ __forceinline__ void packed_word(const PassArgs& a, uint32_t item, in
     if (p == 0) {  // bit b <- neighbour xh - 1
         uint32_t prev;
         if (q == 0u) {  // wrap: the row's last site, moved to bit 31
-            const uint32_t last = load_other<NC>(other + row + nq - 1u);
-            prev = last << (31u - ((W - 1u) & 31u));
+            prev = load_other<NC>(at + nq - 1u) << (31u - ((W - 1u) & 31u));
         } else {
-            prev = load_other<NC>(other + row + q - 1u);
+            prev = load_other<NC>(at - 1);
         }
         sh = __funnelshift_l(prev, o, 1);
     } else {       // bit b <- neighbour xh + 1
         if (q + 1u == nq) {  // wrap: bit nb - 1 takes the row's first site
-            const uint32_t first = q == 0u ? o : load_other<NC>(other + row);
+            const uint32_t first_word = q == 0u ? o : load_other<NC>(other + row);
             const uint32_t top = 1u << (nb - 1u);
-            sh = ((o >> 1) & ~top) | ((first & 1u) ? top : 0u);
+            sh = ((o >> 1) & ~top) | ((first_word & 1u) ? top : 0u);
         } else {
-            sh = __funnelshift_r(o, load_other<NC>(other + row + q + 1u), 1);
+            sh = __funnelshift_r(o, load_other<NC>(at + 1), 1);
         }
     }
-    packed_update<DIMS, MEASURE, RULE, false>(a, own + row + q, s, o, sh, oym, oyp, ozm, ozp,
-                                              valid, nb, r * W + 32u * q, e_acc, m_acc);
+    __syncwarp();
+    // rows of at most 13 sites need no draw past a word's first half
+    packed_update<DIMS, MEASURE, RULE, DRAW>(a, mine, W > 13u, own + row + q, s, o, sh, oym, oyp,
+                                             ozm, ozp, valid, nb, hbase, e_acc, m_acc);
 }
 
 }  // namespace ising

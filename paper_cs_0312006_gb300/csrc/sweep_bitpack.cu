@@ -27,28 +27,35 @@ namespace ising {
 
 namespace {
 
-// One item = one 32-site word of the colour array (see packed_word()).
-// Rows that start inside a Philox group are visited grouped by their offset
-// (rgroups, see packed_word).
-// FULL instances serve lattices whose words are all full (W % 32 == 0) and
-// whose word count per half row nq = 2^nq_shift is a power of two (then so is
-// L = 64 nq; in 3D l_shift = log2 L): an item's row, word and neighbours come
-// from shifts and masks, every row starts on a Philox group, and a thread
-// loads its next item's six words (eight in 3D) before it updates the current
-// one, so that their latency hides behind the current item's draws (at most
-// 64 registers for four CTAs per SM measured slower: 2D L = 8192 29.2 ->
-// 29.4 us per pass, 3D L = 256 9.0e11 -> 8.0e11 site updates/s).
-template <int DIMS, bool MEASURE, int RULE, bool FULL>
-__global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, uint32_t rgroups,
+// How a lattice's words are walked.
+//   kWordsFull: lattices whose words are all full (W % 32 == 0) and whose word
+//     count per half row nq = 2^nq_shift is a power of two (then so is
+//     L = 64 nq; in 3D l_shift = log2 L): an item's row, word and neighbours come
+//     from shifts and masks, every row starts on a Philox group, and a thread
+//     loads its next item's six words (eight in 3D) before it updates the current
+//     one, so that their latency hides behind the current item's draws (at most
+//     64 registers for four CTAs per SM measured slower: 2D L = 8192 29.2 ->
+//     29.4 us per pass, 3D L = 256 9.0e11 -> 8.0e11 site updates/s, both with the
+//     earlier, longer tests).
+//   kWordsAligned: rows that start on a Philox group (W % 4 == 0).
+//   kWordsRagged: any other even L.
+// In the last two a warp takes its words together (packed_words).
+constexpr int kWordsFull = 0, kWordsAligned = 1, kWordsRagged = 2;
+
+template <int DIMS, bool MEASURE, int RULE, int WORDS>
+__global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geom,
                                                       uint32_t nq_shift, uint32_t l_shift) {
-    const uint32_t items = (uint32_t)a.rows * (((uint32_t)a.W + 31u) >> 5);
+    const uint32_t items = geom.items;
     const uint32_t stride = gridDim.x * blockDim.x;
     int e_acc = 0, m_acc = 0;
     grid_dependency_wait();
     launch_dependents();
-    if constexpr (!FULL) {
-        for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < items; g += stride)
-            packed_word<DIMS, MEASURE, 1, RULE>(a, g, e_acc, m_acc, rgroups);
+    if constexpr (WORDS != kWordsFull) {
+        constexpr int draw = WORDS == kWordsAligned ? kDrawAligned : kDrawRagged;
+        constexpr uint32_t step = kWarpWords<draw>;
+        uint32_t first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * step;
+        for (; first < items; first += (stride >> 5) * step)
+            packed_words<DIMS, MEASURE, 1, RULE, draw>(a, geom, first, e_acc, m_acc);
     } else {
         const uint32_t nq = 1u << nq_shift, L = (uint32_t)a.L, W = (uint32_t)a.W;
         uint32_t* own = static_cast<uint32_t*>(a.own);
@@ -76,6 +83,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, uint32_t rgrou
             }
             w.s = own[row + q];
         };
+        // a warp's items are consecutive and items is a multiple of 32 here
         uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
         if (g < items) {
             Words cur;
@@ -91,8 +99,8 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, uint32_t rgrou
                 // bit b <- neighbour xh - 1 (p = 0) or xh + 1 (p = 1)
                 const uint32_t sh = p == 0 ? __funnelshift_l(cur.x, cur.o, 1)
                                            : __funnelshift_r(cur.o, cur.x, 1);
-                packed_update<DIMS, MEASURE, RULE, true>(
-                    a, own + r * nq + q, cur.s, cur.o, sh, cur.ym, cur.yp, cur.zm, cur.zp,
+                packed_update<DIMS, MEASURE, RULE, kDrawAligned>(
+                    a, true, true, own + r * nq + q, cur.s, cur.o, sh, cur.ym, cur.yp, cur.zm, cur.zp,
                     0xFFFFFFFFu, 32u, r * W + 32u * q, e_acc, m_acc);
                 if (!more) break;
                 cur = nxt;
@@ -183,26 +191,28 @@ template <int DIMS, bool MEASURE, int RULE>
 cudaError_t launch_packed_t(const PassArgs& a, const DeviceProps& dp, cudaStream_t st) {
     const int nq = (a.W + 31) >> 5;
     const int64_t items = a.rows * nq;
-    // (multi-hit keeps the general loop: its trials need the registers)
-    const bool full = RULE != kRuleMultiHit && a.W % 32 == 0 && is_pow2(nq);
-    int64_t blocks = (items + 255) / 256;
+    const int words = a.W % 32 == 0 && is_pow2(nq) ? kWordsFull
+                      : a.W % 4 == 0               ? kWordsAligned
+                                                   : kWordsRagged;
+    const int64_t per_block =
+        8 * (words == kWordsRagged ? kWarpWords<kDrawRagged> : kWarpWords<kDrawAligned>);
+    int64_t blocks = (items + per_block - 1) / per_block;
     const int64_t cap =
-        (int64_t)dp.sm_count * dp.blocks_per_sm_packed[RULE][DIMS - 2][MEASURE][full ? 1 : 0];
+        (int64_t)dp.sm_count * dp.blocks_per_sm_packed[RULE][DIMS - 2][MEASURE][words];
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    // odd W: a row's offset in its Philox group is r W mod 4, set by r mod 4;
-    // W = 2 mod 4: by r mod 2
-    const uint32_t rgroups = packed_row_groups((uint32_t)a.W);
-    if constexpr (RULE != kRuleMultiHit) {
-        if (full) {
-            const uint32_t nq_shift = (uint32_t)__builtin_ctz((unsigned)nq);
-            const uint32_t l_shift = DIMS == 3 ? (uint32_t)__builtin_ctz((unsigned)a.L) : 0u;
-            return launch_chained(pass_packed<DIMS, MEASURE, RULE, true>, (unsigned)blocks, 256u,
-                                  0, st, a, rgroups, nq_shift, l_shift);
-        }
+    const PackedGeom geom((uint32_t)a.W, (uint32_t)a.L, (uint32_t)a.rows);
+    if (words == kWordsFull) {
+        const uint32_t nq_shift = (uint32_t)__builtin_ctz((unsigned)nq);
+        const uint32_t l_shift = DIMS == 3 ? (uint32_t)__builtin_ctz((unsigned)a.L) : 0u;
+        return launch_chained(pass_packed<DIMS, MEASURE, RULE, kWordsFull>, (unsigned)blocks,
+                              256u, 0, st, a, geom, nq_shift, l_shift);
     }
-    return launch_chained(pass_packed<DIMS, MEASURE, RULE, false>, (unsigned)blocks, 256u, 0, st,
-                          a, rgroups, 0u, 0u);
+    if (words == kWordsAligned)
+        return launch_chained(pass_packed<DIMS, MEASURE, RULE, kWordsAligned>, (unsigned)blocks,
+                              256u, 0, st, a, geom, 0u, 0u);
+    return launch_chained(pass_packed<DIMS, MEASURE, RULE, kWordsRagged>, (unsigned)blocks, 256u,
+                          0, st, a, geom, 0u, 0u);
 }
 
 }  // namespace
@@ -213,8 +223,9 @@ cudaError_t packed_query_occupancy(DeviceProps& dp) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&dp.blocks_per_sm_packed[R][D - 2][M][F],\
                                                       pass_packed<D, M, R, F>, 256, 0);       \
     if (e != cudaSuccess) return e;
-#define ISING_OCC(R, D, M) ISING_OCC1(R, D, M, false) ISING_OCC1(R, D, M, true)
-#define ISING_OCC_MH(R, D, M) ISING_OCC1(R, D, M, false)
+#define ISING_OCC(R, D, M)                                                        \
+    ISING_OCC1(R, D, M, kWordsFull) ISING_OCC1(R, D, M, kWordsAligned)            \
+        ISING_OCC1(R, D, M, kWordsRagged)
     ISING_OCC(kRuleMetropolis, 2, false)
     ISING_OCC(kRuleMetropolis, 2, true)
     ISING_OCC(kRuleMetropolis, 3, false)
@@ -223,11 +234,10 @@ cudaError_t packed_query_occupancy(DeviceProps& dp) {
     ISING_OCC(kRuleHeatBath, 2, true)
     ISING_OCC(kRuleHeatBath, 3, false)
     ISING_OCC(kRuleHeatBath, 3, true)
-    ISING_OCC_MH(kRuleMultiHit, 2, false)
-    ISING_OCC_MH(kRuleMultiHit, 2, true)
-    ISING_OCC_MH(kRuleMultiHit, 3, false)
-    ISING_OCC_MH(kRuleMultiHit, 3, true)
-#undef ISING_OCC_MH
+    ISING_OCC(kRuleMultiHit, 2, false)
+    ISING_OCC(kRuleMultiHit, 2, true)
+    ISING_OCC(kRuleMultiHit, 3, false)
+    ISING_OCC(kRuleMultiHit, 3, true)
 #undef ISING_OCC
 #undef ISING_OCC1
     return cudaSuccess;
