@@ -105,7 +105,7 @@ __device__ __forceinline__ void group_sync() {
 // and draws of int8_word (word w's draw is Philox group w).
 template <int DIMS, bool MEASURE, int NC, int RULE>
 __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom& g, uint32_t w,
-                                               int& e_acc, int& m_neg, int& n_sites) {
+                                               int& e_acc, int& m_sum) {
     uint32_t* own = static_cast<uint32_t*>(a.own);
     const uint32_t* other = static_cast<const uint32_t*>(a.other);
     const uint32_t nq = g.W >> 2;  // words per half row
@@ -136,26 +136,16 @@ __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom
         nzp = load_other<NC>(other + ((z + 1u == g.L ? 0u : z + 1u) * g.L + y) * nq + q);
     }
     const uint32_t D = disagreements<DIMS>(s, nx, nxs, nym, nyp, nzm, nzp);
-    uint32_t X;
-    if (RULE == kRuleHeatBath) {
-        const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-        X = heatbath_count<DIMS>(D, u, a);
-    } else {
-        X = downhill_mask<DIMS>(D);
-        if (X != 0xFEFEFEFEu) {
-            const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-            X |= uphill_count<DIMS>(D, u, a);
-        }
-    }
-    const uint32_t snew = s ^ X;
+    const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
+    const uint32_t X = flip_mask<DIMS, RULE>(D, u, a);
+    const uint32_t snew = s ^ (X & kByteFlip);
     own[w] = snew;
     if (MEASURE) {
-        m_neg += __popc(snew & kByteBit7);
-        n_sites += 4;
+        m_sum = add_bytes(snew, m_sum);
         if (a.c == 1) {
             constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
             const uint32_t Dn = (D & ~X) | ((q2 - D) & X);
-            e_acc += __dp4a((int)Dn, (int)kByteOnes, 0) - 4 * 2 * DIMS;
+            e_acc = add_bytes(Dn, e_acc - 4 * 2 * DIMS);
         }
     }
 }
@@ -189,21 +179,19 @@ __device__ __forceinline__ void job_pass(const BatchJob& j, const PackedGeom& ge
         g.rows = j.rows;
         g.half = j.half;
         const uint32_t vecs = (j.half + 15u) >> 4;
-        int m_neg = 0, n_sites = 0;
         if (j.W >= 64 && vecs >= nthr) {
             for (uint32_t v = rank; v < vecs; v += nthr)
-                int8_vec<DIMS, MEASURE, NC, RULE>(a, g, v, e_acc, m_neg, n_sites);
+                int8_vec<DIMS, MEASURE, NC, RULE>(a, g, v, e_acc, m_acc);
         } else if (j.W % 4 == 0 && RULE != kRuleMultiHit) {
             // short rows of whole words: one uniform path for every word
             const uint32_t words = j.half >> 2;
             for (uint32_t w = rank; w < words; w += nthr)
-                int8_word_rows<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_neg, n_sites);
+                int8_word_rows<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
         } else {  // short rows or few vectors: four sites per item spread further
             const uint32_t words = (j.half + 3u) >> 2;
             for (uint32_t w = rank; w < words; w += nthr)
-                int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_neg, n_sites);
+                int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
         }
-        if (MEASURE) m_acc += n_sites - 2 * m_neg;
     } else {
         // (one body for aligned and ragged rows: at half the code the kernels
         // spill less and stay in the instruction cache)
@@ -224,10 +212,8 @@ __device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom&
         g.L = (uint32_t)j.L;
         g.rows = j.rows;
         g.half = j.half;
-        int m_neg = 0, n_sites = 0;
         const uint32_t v = first + (threadIdx.x & 31u);
-        if (16u * v < j.half) int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_neg, n_sites);
-        if (MEASURE) m_acc += n_sites - 2 * m_neg;
+        if (16u * v < j.half) int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_acc);
     } else {
         packed_words<DIMS, MEASURE, 1, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
     }

@@ -143,6 +143,25 @@ __device__ __forceinline__ void mark_below(uint32_t& mask, uint32_t u, uint32_t 
         : "r"(u), "r"(thr), "n"(BITS));
 }
 
+// sum += step where u < thr.
+template <uint32_t STEP>
+__device__ __forceinline__ void add_below(uint32_t& sum, uint32_t u, uint32_t thr) {
+    asm("{\n"
+        ".reg .pred p;\n"
+        "setp.lt.u32 p, %1, %2;\n"
+        "@p add.u32 %0, %0, %3;\n"
+        "}"
+        : "+r"(sum)
+        : "r"(u), "r"(thr), "n"(STEP));
+}
+
+// 0xFF in every byte of w whose top bit is set, else 0.
+__device__ __forceinline__ uint32_t byte_signs(uint32_t w) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(d) : "r"(w));
+    return d;
+}
+
 // mask |= bits where u <= thr.
 template <uint32_t BITS>
 __device__ __forceinline__ void mark_upto(uint32_t& mask, uint32_t u, uint32_t thr) {

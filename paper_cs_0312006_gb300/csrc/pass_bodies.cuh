@@ -39,71 +39,47 @@ __device__ __forceinline__ T load_other(const T* p) {
     return *p;
 }
 
-// Byte mask 0xFE of each site whose flip is decided without a draw: byte j of
-// D is 2*d_j, and bit 7 of D + bias is set iff d_j >= dims (dE <= 0).
+// 0xFF per site whose flip is decided without a draw: byte j of D is 2 d_j, and
+// bit 7 of D + bias is set iff d_j >= dims (dE <= 0).
 template <int DIMS>
 __device__ __forceinline__ uint32_t downhill_mask(uint32_t D) {
-    constexpr uint32_t bias = (0x80u - 2u * DIMS) * kByteOnes;
-    const uint32_t F = (D + bias) & kByteBit7;
-    return F | (F - (F >> 6));  // 0x80 -> 0xFE per byte, borrow-free
+    return byte_signs(D + (0x80u - 2u * DIMS) * kByteOnes);
 }
 
-// Metropolis test of site j (d_j < dims): u_j < thr[k], k = 2(dims - d_j).
-template <int DIMS>
-__device__ __forceinline__ uint32_t uphill_accept(uint32_t D, uint32_t u, int j,
-                                                  const PassArgs& a) {
-    const uint32_t dj = D & (0x0Eu << (8 * j));  // 2*d_j in place
-    uint32_t t;
-    if (DIMS == 2) {
-        t = dj == 0u ? a.thr[1] : a.thr[0];
-    } else {
-        t = dj == 0u ? a.thr[2] : (dj == (0x02u << (8 * j)) ? a.thr[1] : a.thr[0]);
-    }
-    return u < t ? (0xFEu << (8 * j)) : 0u;
-}
-
-// The same test for four sites by counting: byte j gains 2 for every threshold
-// u_j lies below; since the thresholds fall with k, site j (d_j < dims) flips
-// iff 2*(count_j + d_j) >= 2*dims, read off bit 7 after the bias.  A site with
-// d_j >= dims has bit 7 set by D + bias alone, and no byte carries (at most
-// 0x80 + 4 dims < 0x100), so the mask already holds every downhill
-// flip: where all four draws are made it is the whole flip mask.
-template <int DIMS>
-__device__ __forceinline__ uint32_t uphill_count(uint32_t D, const Philox4& u, const PassArgs& a) {
-    constexpr uint32_t bias = (0x80u - 2u * DIMS) * kByteOnes;
+// 0xFF per site (byte) of a word that flips, from D (byte j is 2 d_j) and the
+// draws of its four sites.  With cnt_j the number of the rule's thresholds that
+// u_j lies below (they are nested) -- Metropolis: the thresholds fall with k, so
+// a site with d < dims flips iff cnt + d >= dims, and one with d >= dims always
+// does: bit 7 of D + 2 cnt + bias (at most 0x80 + 4 dims: no carry).  Heat bath
+// (every site draws; it flips iff u < thr[d], the thresholds rising with d): iff
+// cnt + d >= 2 dims + 1 (at most 4 (2 dims) + 2 + bias < 256).
+//
+// A compare and a predicated add per threshold: with the generator, E and M in
+// registers 106 issue slots a word (2D; 83 the generator alone).  The sum of
+// selects took 119 as compiled, toggling the bits of the count 127: the ALU pipe
+// takes one instruction in two cycles, and adds (and the byte sums of E and M)
+// need not go there.
+template <int DIMS, int RULE>
+__device__ __forceinline__ uint32_t flip_mask(uint32_t D, const Philox4& u, const PassArgs& a) {
+    constexpr int N = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
+    constexpr uint32_t need = RULE == kRuleHeatBath ? 2u * DIMS + 1u : (uint32_t)DIMS;
+    constexpr uint32_t bias = (0x80u - 2u * need) * kByteOnes;
     uint32_t acc = D + bias;
-    acc += (u.w0 < a.thr[0] ? 0x00000002u : 0u) + (u.w0 < a.thr[1] ? 0x00000002u : 0u);
-    acc += (u.w1 < a.thr[0] ? 0x00000200u : 0u) + (u.w1 < a.thr[1] ? 0x00000200u : 0u);
-    acc += (u.w2 < a.thr[0] ? 0x00020000u : 0u) + (u.w2 < a.thr[1] ? 0x00020000u : 0u);
-    acc += (u.w3 < a.thr[0] ? 0x02000000u : 0u) + (u.w3 < a.thr[1] ? 0x02000000u : 0u);
-    if (DIMS == 3) {
-        acc += (u.w0 < a.thr[2] ? 0x00000002u : 0u) + (u.w1 < a.thr[2] ? 0x00000200u : 0u);
-        acc += (u.w2 < a.thr[2] ? 0x00020000u : 0u) + (u.w3 < a.thr[2] ? 0x02000000u : 0u);
-    }
-    const uint32_t F = acc & kByteBit7;
-    return F | (F - (F >> 6));
+    static_for<4>([&](auto site) {
+        constexpr int j = decltype(site)::value;
+        const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
+#pragma unroll
+        for (int n = 0; n < N; ++n) add_below<(2u << (8 * j))>(acc, w, a.thr[n]);
+    });
+    return byte_signs(acc);
 }
 
-// Heat-bath rule (every site draws; it flips iff u < thr[d], the thresholds
-// rising with d): with cnt = #{m = 0..2 dims : u < thr[m]}, u < thr[d] iff
-// cnt + d >= 2 dims + 1.  Byte j of D is 2 d_j, so byte j of D + bias + 2 cnt_j
-// reaches bit 7 exactly then (at most 4*(2 dims) + 2 + bias < 256: no carry).
-template <int DIMS>
-__device__ __forceinline__ uint32_t heatbath_count(uint32_t D, const Philox4& u,
-                                                   const PassArgs& a) {
-    constexpr uint32_t bias = (0x80u - 2u * (2u * DIMS + 1u)) * kByteOnes;
-    const uint32_t w[4] = {u.w0, u.w1, u.w2, u.w3};
-    uint32_t acc = D + bias;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        uint32_t cnt = 0u;
-#pragma unroll
-        for (int m = 0; m <= 2 * DIMS; ++m) cnt += w[j] < a.thr[m] ? 2u : 0u;
-        acc += cnt << (8 * j);
-    }
-    const uint32_t F = acc & kByteBit7;
-    return F | (F - (F >> 6));
+// Sum of a word's four spins (bytes +1 / -1) or counts, added to acc.
+__device__ __forceinline__ int add_bytes(uint32_t w, int acc) {
+    return __dp4a((int)w, (int)kByteOnes, acc);
 }
+
+constexpr uint32_t kByteFlip = 0xFEFEFEFEu;  // 0x01 <-> 0xFF
 
 // thr[d] by selects (d = 0..2*dims), for code that holds PassArgs in registers.
 template <int DIMS>
@@ -124,10 +100,10 @@ __device__ __forceinline__ uint32_t multihit_word(uint32_t D, uint32_t group, co
 #pragma unroll 1
     for (int m = 0; m < a.hits; ++m) {
         uint32_t X = downhill_mask<DIMS>(D);
-        if (X != 0xFEFEFEFEu) {
+        if (X != 0xFFFFFFFFu) {
             const Philox4 u = philox4x32_10(group, a.t, (uint32_t)a.c + 2u * (uint32_t)m,
                                             kTagSweep, a.key0, a.key1);
-            X |= uphill_count<DIMS>(D, u, a);
+            X = flip_mask<DIMS, kRuleMetropolis>(D, u, a);
         }
         D = (D & ~X) | ((q2 - D) & X);
         net ^= X;
@@ -163,11 +139,11 @@ struct WordGeom {
 };
 
 // Update word w of the int8 colour array `own` (colour a.c).  Accumulates the
-// number of -1 spins written (m_neg), the number of sites written (n_sites)
-// and, in the white pass, sum (2 d_new - 2 dims) over them (e_acc).
+// sum of the spins written (m_sum) and, in the white pass,
+// sum (2 d_new - 2 dims) over them (e_acc).
 template <int DIMS, bool MEASURE, int NC, int RULE = kRuleMetropolis>
 __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, uint32_t w,
-                                          int& e_acc, int& m_neg, int& n_sites) {
+                                          int& e_acc, int& m_sum) {
     uint32_t* own = static_cast<uint32_t*>(a.own);
     const uint32_t* other = static_cast<const uint32_t*>(a.other);
     const int8_t* other_b = static_cast<const int8_t*>(a.other);
@@ -196,28 +172,20 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
         }
         const uint32_t D = disagreements<DIMS>(s, nx, nxs, nym, nyp, nzm, nzp);
         uint32_t X;
-        if (RULE == kRuleHeatBath) {
-            const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-            X = heatbath_count<DIMS>(D, u, a);
-        } else if (RULE == kRuleMultiHit) {
+        if (RULE == kRuleMultiHit) {
             X = multihit_word<DIMS>(D, w, a);
         } else {
-            X = downhill_mask<DIMS>(D);
-            if (X != 0xFEFEFEFEu) {
-                const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-                X |= uphill_accept<DIMS>(D, u.w0, 0, a) | uphill_accept<DIMS>(D, u.w1, 1, a) |
-                     uphill_accept<DIMS>(D, u.w2, 2, a) | uphill_accept<DIMS>(D, u.w3, 3, a);
-            }
+            const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
+            X = flip_mask<DIMS, RULE>(D, u, a);
         }
-        const uint32_t snew = s ^ X;
+        const uint32_t snew = s ^ (X & kByteFlip);
         own[w] = snew;
         if (MEASURE) {
-            m_neg += __popc(snew & kByteBit7);
-            n_sites += 4;
+            m_sum = add_bytes(snew, m_sum);
             if (a.c == 1) {
                 constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
                 const uint32_t Dn = (D & ~X) | ((q2 - D) & X);
-                e_acc += __dp4a((int)Dn, (int)kByteOnes, 0) - 4 * 2 * DIMS;
+                e_acc = add_bytes(Dn, e_acc - 4 * 2 * DIMS);
             }
         }
         return;
@@ -300,8 +268,7 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
             const int sn = flips[j] ? -s_val[j] : s_val[j];
             if (flips[j]) own_b[h0 + j] = (int8_t)sn;
             if (MEASURE) {
-                m_neg += sn < 0;
-                n_sites += 1;
+                m_sum += sn;
                 if (a.c == 1) e_acc += 2 * d_cur[j] - 2 * DIMS;
             }
         }
@@ -332,8 +299,7 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
         const int sn = flip ? -s_val[j] : s_val[j];
         if (flip) own_b[h0 + j] = (int8_t)sn;
         if (MEASURE) {
-            m_neg += sn < 0;
-            n_sites += 1;
+            m_sum += sn;
             if (a.c == 1) {
                 const int dn = flip ? 2 * DIMS - d_val[j] : d_val[j];
                 e_acc += 2 * dn - 2 * DIMS;
@@ -343,87 +309,54 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
 }
 
 // Update the 16 sites of one 16-byte vector (four Philox groups g0..g0+3).
-// The four Philox calls are independent and computed together when any of
-// the 16 sites needs its draw (always, under the heat-bath rule).  Accumulates the number of -1 spins (m_neg)
-// and, in the white pass, sum_j 2*d_new_j (e_acc).
+// Accumulates the sum of the new spins (m_sum) and, in the white pass,
+// sum_j 2*d_new_j (e_acc).
 template <int DIMS, bool MEASURE, int RULE = kRuleMetropolis>
 __device__ __forceinline__ uint4 update_vec(const uint4& s, const uint4& x, const uint4& xs,
                                             const uint4& ym, const uint4& yp, const uint4& zm,
                                             const uint4& zp, uint32_t g0, const PassArgs& a,
-                                            int& e_acc, int& m_neg) {
+                                            int& e_acc, int& m_sum) {
     const uint32_t sv[4] = {s.x, s.y, s.z, s.w};
     uint32_t D[4], X[4];
     D[0] = disagreements<DIMS>(s.x, x.x, xs.x, ym.x, yp.x, zm.x, zp.x);
     D[1] = disagreements<DIMS>(s.y, x.y, xs.y, ym.y, yp.y, zm.y, zp.y);
     D[2] = disagreements<DIMS>(s.z, x.z, xs.z, ym.z, yp.z, zm.z, zp.z);
     D[3] = disagreements<DIMS>(s.w, x.w, xs.w, ym.w, yp.w, zm.w, zp.w);
-    if (RULE == kRuleMultiHit) {
-        constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
-        uint32_t Dc[4] = {D[0], D[1], D[2], D[3]};
+    // one trial, or a.hits in a row with the neighbours fixed; the four calls
+    // are consecutive groups and are made together, whether or not all four
+    // words hold a site that draws (nearly all do)
+    const int hits = RULE == kRuleMultiHit ? a.hits : 1;
+    uint32_t Dc[4] = {D[0], D[1], D[2], D[3]};
 #pragma unroll
-        for (int w = 0; w < 4; ++w) X[w] = 0u;
+    for (int w = 0; w < 4; ++w) X[w] = 0u;
 #pragma unroll 1
-        for (int m = 0; m < a.hits; ++m) {
-            uint32_t Y[4];
-            bool need = false;
+    for (int m = 0; m < hits; ++m) {
+        PhiloxRuns<1> ps;
+        const uint32_t base[1] = {g0};
+        ps.first_round(base, a.t, (uint32_t)a.c + 2u * (uint32_t)m, kTagSweep, a.key0, a.key1);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                Y[w] = downhill_mask<DIMS>(Dc[w]);
-                need |= Y[w] != 0xFEFEFEFEu;
-            }
-            if (need) {
-                Philox4 u[4];
-#pragma unroll
-                for (int w = 0; w < 4; ++w)
-                    u[w] = philox4x32_10(g0 + (uint32_t)w, a.t, (uint32_t)a.c + 2u * (uint32_t)m,
-                                         kTagSweep, a.key0, a.key1);
-#pragma unroll
-                for (int w = 0; w < 4; ++w) Y[w] |= uphill_count<DIMS>(Dc[w], u[w], a);
-            }
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                Dc[w] = (Dc[w] & ~Y[w]) | ((q2 - Dc[w]) & Y[w]);
-                X[w] ^= Y[w];
-            }
-        }
-    } else if (RULE == kRuleHeatBath) {  // every site draws
-        Philox4 u[4];
-#pragma unroll
-        for (int w = 0; w < 4; ++w)
-            u[w] = philox4x32_10(g0 + (uint32_t)w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) X[w] = heatbath_count<DIMS>(D[w], u[w], a);
-    } else {
-        bool need = false;
+        for (int r = 1; r < 10; ++r) ps.next_round();
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-            X[w] = downhill_mask<DIMS>(D[w]);
-            need |= X[w] != 0xFEFEFEFEu;
-        }
-        if (need) {
-            Philox4 u[4];
-#pragma unroll
-            for (int w = 0; w < 4; ++w)
-                u[w] = philox4x32_10(g0 + (uint32_t)w, a.t, (uint32_t)a.c, kTagSweep, a.key0,
-                                     a.key1);
-            // counting thresholds below each draw measured a little faster here
-            // than selecting one threshold per site (uphill_accept): it spreads
-            // the work over the integer ALU and the multiply-add pipe
-#pragma unroll
-            for (int w = 0; w < 4; ++w) X[w] |= uphill_count<DIMS>(D[w], u[w], a);
+            const uint32_t Y = flip_mask<DIMS, RULE>(Dc[w], ps.result(w), a);
+            if (RULE == kRuleMultiHit) {
+                constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
+                Dc[w] = (Dc[w] & ~Y) | ((q2 - Dc[w]) & Y);
+            }
+            X[w] ^= Y;
         }
     }
     uint32_t out[4];
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-        out[w] = sv[w] ^ X[w];  // 0x01 <-> 0xFF where flipped
+        out[w] = sv[w] ^ (X[w] & kByteFlip);
         if (MEASURE) {
-            m_neg += __popc(out[w] & kByteBit7);
+            m_sum = add_bytes(out[w], m_sum);
             if (a.c == 1) {
-                // 2*d_new = 2*(2 dims) - 2*d where flipped; X covers bits 1..7 there
+                // 2*d_new = 2*(2 dims) - 2*d where flipped
                 constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
                 const uint32_t Dn = (D[w] & ~X[w]) | ((q2 - D[w]) & X[w]);
-                e_acc = __dp4a((int)Dn, (int)kByteOnes, e_acc);
+                e_acc = add_bytes(Dn, e_acc);
             }
         }
     }
@@ -457,10 +390,10 @@ __device__ __forceinline__ uint4 window16(const uint4* other16, uint32_t o) {
 // 4v..4v+3) of the int8 colour array.  A vector inside one half row, away from
 // the x-wrap and the first/last row and plane, is updated as a whole from
 // 16-byte neighbour windows; any other vector word by word (int8_word).
-// Accumulates m_neg, n_sites and, in the white pass, e_acc as int8_word does.
+// Accumulates m_sum and, in the white pass, e_acc as int8_word does.
 template <int DIMS, bool MEASURE, int NC, int RULE = kRuleMetropolis>
 __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, uint32_t v,
-                                         int& e_acc, int& m_neg, int& n_sites) {
+                                         int& e_acc, int& m_sum) {
     const uint32_t h0 = 16u * v;
     const uint32_t r0 = h0 / g.W;
     const uint32_t xh0 = h0 - r0 * g.W;
@@ -476,7 +409,7 @@ __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, u
     if (!fast) {
 #pragma unroll 1
         for (uint32_t w = 4u * v; w < 4u * v + 4u; ++w)
-            if (4u * w < g.half) int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_neg, n_sites);
+            if (4u * w < g.half) int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_sum);
         return;
     }
     const uint4* other16 = static_cast<const uint4*>(a.other);
@@ -502,11 +435,8 @@ __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, u
     }
     int e_vec = 0;
     own16[v] = update_vec<DIMS, MEASURE, RULE>(s, nx, nxs, nym, nyp, nzm, nzp, 4u * v, a, e_vec,
-                                               m_neg);
-    if (MEASURE) {
-        n_sites += 16;
-        if (a.c == 1) e_acc += e_vec - 16 * 2 * DIMS;
-    }
+                                               m_sum);
+    if (MEASURE && a.c == 1) e_acc += e_vec - 16 * 2 * DIMS;
 }
 
 // ----------------------------------------------------------------------------

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
     const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
     uint4 om = zero, oc = zero, op = zero, sc = zero, zm = zero, zp = zero;
     bool reload = true;
-    int e_acc = 0, m_neg = 0, n_rows = 0;
+    int e_acc = 0, m_acc = 0, n_rows = 0;
     grid_dependency_wait();
     launch_dependents();
 
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
             }
             const uint32_t g0 = ((uint32_t)r * nv + (uint32_t)v) * 4u;  // Philox group of word 0
             const uint4 s = update_vec<DIMS, MEASURE, RULE>(sc, oc, sh, om, op, zm, zp, g0, a,
-                                                            e_acc, m_neg);
+                                                            e_acc, m_acc);
             Sv[(uint32_t)r * nv] = s;
             ++n_rows;
         }
@@ -145,7 +145,6 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
     }
     if (MEASURE) {
         e_acc -= n_rows * 16 * 2 * DIMS;          // E_white = sum_j (2 d_new_j - 2 dims)
-        const int m_acc = n_rows * 16 - 2 * m_neg;  // sum of the new spins
         block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
     }
 }
@@ -156,12 +155,12 @@ template <int DIMS, bool MEASURE, int RULE>
 __global__ void __launch_bounds__(256) pass_int8_vecs(PassArgs a, WordGeom g) {
     const uint32_t vecs = (g.half + 15u) >> 4;
     const uint32_t stride = gridDim.x * blockDim.x;
-    int e_acc = 0, m_neg = 0, n_sites = 0;
+    int e_acc = 0, m_acc = 0;
     grid_dependency_wait();
     launch_dependents();
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < vecs; v += stride)
-        int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_neg, n_sites);
-    if (MEASURE) block_reduce_add(e_acc, n_sites - 2 * m_neg, a.obs, a.c == 1);
+        int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_acc);
+    if (MEASURE) block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
 }
 
 // Canonical <-> layout conversion and initial states.  Item = one canonical

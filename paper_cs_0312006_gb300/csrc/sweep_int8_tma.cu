@@ -147,14 +147,13 @@ __device__ __forceinline__ void issue_tile(const PassArgs& a, const TmaGeom& tg,
 // pair), as their 8 words and byte-sliced disagreement counts D (byte j of D
 // is 2 d_j), taken from shared memory when the item is loaded; step(w) then
 // applies the rule to word w with its draw u (word w & 3 of call w: vector
-// w >> 2).  Metropolis takes the counting mask (uphill_count, which holds the
+// w >> 2).  Metropolis takes the counting mask (flip_mask, which holds the
 // downhill flips too); the heat bath reads thr[d] per site from a shared
-// table.  en sums 2 d_new per byte (at most 12 per word: eight words fit a
-// byte), mn sums 2 per spin -1 (at most 16 per byte).
+// table.  en sums 2 d_new, mn the new spins.
 template <int DIMS, bool MEASURE, int RULE>
 struct PairUpdate {
     uint32_t sv[8], D[8], rowg[2];
-    uint32_t en, mn;
+    int en, mn;
 
     __device__ __forceinline__ void set(int q, const uint4& S, const uint4& x, const uint4& xs,
                                         const uint4& ym, const uint4& yp, const uint4& zm,
@@ -168,7 +167,7 @@ struct PairUpdate {
         D[4 * q + 2] = disagreements<DIMS>(S.z, x.z, xs.z, ym.z, yp.z, zm.z, zp.z);
         D[4 * q + 3] = disagreements<DIMS>(S.w, x.w, xs.w, ym.w, yp.w, zm.w, zp.w);
         rowg[q] = row;
-        if (q == 0) en = mn = 0u;
+        if (q == 0) en = mn = 0;
     }
 
     __device__ __forceinline__ void step(int w, const Philox4& u, const PassArgs& a,
@@ -180,29 +179,29 @@ struct PairUpdate {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const uint32_t t = s_thb[(D[w] >> (8 * j + 1)) & 7u];
-                X |= uw[j] < t ? (0xFEu << (8 * j)) : 0u;
+                X |= uw[j] < t ? (0xFFu << (8 * j)) : 0u;
             }
         } else {
-            X = uphill_count<DIMS>(D[w], u, a);
+            X = flip_mask<DIMS, RULE>(D[w], u, a);
         }
-        const uint32_t out = sv[w] ^ X;
+        const uint32_t out = sv[w] ^ (X & kByteFlip);
         if (MEASURE) {
-            mn += out & kByteBit1;
+            mn = add_bytes(out, mn);
             if (a.c == 1) {
                 constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
-                en += (D[w] & ~X) | ((q2 - D[w]) & X);
+                en = add_bytes((D[w] & ~X) | ((q2 - D[w]) & X), en);
             }
         }
         sv[w] = out;
     }
 
     __device__ __forceinline__ void store(uint4* own_g, const PassArgs& a, int& e_acc,
-                                          int& m_neg) const {
+                                          int& m_acc) const {
         own_g[rowg[0]] = make_uint4(sv[0], sv[1], sv[2], sv[3]);
         own_g[rowg[1]] = make_uint4(sv[4], sv[5], sv[6], sv[7]);
         if (MEASURE) {
-            m_neg += __dp4a((int)mn, (int)kByteOnes, 0) >> 1;
-            if (a.c == 1) e_acc = __dp4a((int)en, (int)kByteOnes, e_acc);
+            m_acc += mn;
+            if (a.c == 1) e_acc += en;
         }
     }
 };
@@ -242,7 +241,7 @@ __global__ void __launch_bounds__(128, WALK == kWalkOne ? 6 : 4) pass_int8_tma(P
             issue_tile<DIMS>(a, tg, first + k * gridDim.x, smem + k * tg.stage_bytes, &bars[k],
                              k == 0 ? tg.extra_tx : 0u);
 
-    int e_acc = 0, m_neg = 0, n_vec = 0;
+    int e_acc = 0, m_acc = 0, n_vec = 0;
     uint4* own_g = static_cast<uint4*>(a.own);
     // (row pair, column) item -> pair index and column
     auto split = [&](uint32_t item, uint32_t& pr, uint32_t& v) {
@@ -354,7 +353,7 @@ __global__ void __launch_bounds__(128, WALK == kWalkOne ? 6 : 4) pass_int8_tma(P
                 }
             };
             auto finish = [&](const Pair& d) {
-                d.store(own_g, a, e_acc, m_neg);
+                d.store(own_g, a, e_acc, m_acc);
                 n_vec += 2;
             };
             auto update = [&](Pair& d, const Philox4 (&u)[8]) {
@@ -462,7 +461,7 @@ __global__ void __launch_bounds__(128, WALK == kWalkOne ? 6 : 4) pass_int8_tma(P
                 const uint32_t row = (z * (uint32_t)a.L + y) * nv + v;  // global vector index
                 int e_vec = 0;
                 own_g[row] = update_vec<DIMS, MEASURE, RULE>(own_s[i * nv + v], oc, sh, om, op,
-                                                             zm, zp, row * 4u, a, e_vec, m_neg);
+                                                             zm, zp, row * 4u, a, e_vec, m_acc);
                 e_acc += e_vec;
                 ++n_vec;
             }
@@ -476,7 +475,7 @@ __global__ void __launch_bounds__(128, WALK == kWalkOne ? 6 : 4) pass_int8_tma(P
     }
     if (MEASURE) {
         if (a.c == 1) e_acc -= n_vec * 16 * 2 * DIMS;  // E_white = sum (2 d_new - 2 dims)
-        block_reduce_add(e_acc, n_vec * 16 - 2 * m_neg, a.obs, a.c == 1);
+        block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
     }
 }
 
