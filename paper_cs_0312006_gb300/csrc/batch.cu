@@ -137,7 +137,7 @@ __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom
     }
     const uint32_t D = disagreements<DIMS>(s, nx, nxs, nym, nyp, nzm, nzp);
     const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-    const uint32_t X = flip_mask<DIMS, RULE>(D, u, a);
+    const uint32_t X = flip_mask(D, count_word<DIMS, RULE>(u, a));
     const uint32_t snew = s ^ (X & kByteFlip);
     own[w] = snew;
     if (MEASURE) {
@@ -167,31 +167,35 @@ __device__ __forceinline__ PassArgs job_args(const BatchJob& j, int c, uint32_t 
     return a;
 }
 
+// The int8 layout's pass of a job: not inlined, so that it does not add to the
+// registers of the packed one (ISING_AUTO's layout).
+template <int DIMS, bool MEASURE, int NC, int RULE>
+__device__ __noinline__ void job_pass_int8(const BatchJob& j, const PassArgs& a, uint32_t rank,
+                                           uint32_t nthr, int& e_acc, int& m_acc) {
+    const WordGeom g((uint32_t)j.W, (uint32_t)j.L, j.rows);
+    const uint32_t vecs = (j.half + 15u) >> 4;
+    if (j.W >= 64 && vecs >= nthr) {
+        for (uint32_t v = rank; v < vecs; v += nthr)
+            int8_vec<DIMS, MEASURE, NC, RULE>(a, g, v, e_acc, m_acc);
+    } else if (j.W % 4 == 0 && RULE != kRuleMultiHit) {
+        // short rows of whole words: one uniform path for every word
+        const uint32_t words = j.half >> 2;
+        for (uint32_t w = rank; w < words; w += nthr)
+            int8_word_rows<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
+    } else {  // short rows or few vectors: four sites per item spread further
+        const uint32_t words = (j.half + 3u) >> 2;
+        for (uint32_t w = rank; w < words; w += nthr)
+            int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
+    }
+}
+
 template <int DIMS, int LAYOUT, bool MEASURE, int NC, int RULE>
 __device__ __forceinline__ void job_pass(const BatchJob& j, const PackedGeom& geom, int c,
                                          uint32_t t, uint32_t rank, uint32_t nthr, int& e_acc,
                                          int& m_acc) {
     const PassArgs a = job_args(j, c, t);
     if (LAYOUT == ISING_INT8) {
-        WordGeom g;
-        g.W = (uint32_t)j.W;
-        g.L = (uint32_t)j.L;
-        g.rows = j.rows;
-        g.half = j.half;
-        const uint32_t vecs = (j.half + 15u) >> 4;
-        if (j.W >= 64 && vecs >= nthr) {
-            for (uint32_t v = rank; v < vecs; v += nthr)
-                int8_vec<DIMS, MEASURE, NC, RULE>(a, g, v, e_acc, m_acc);
-        } else if (j.W % 4 == 0 && RULE != kRuleMultiHit) {
-            // short rows of whole words: one uniform path for every word
-            const uint32_t words = j.half >> 2;
-            for (uint32_t w = rank; w < words; w += nthr)
-                int8_word_rows<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
-        } else {  // short rows or few vectors: four sites per item spread further
-            const uint32_t words = (j.half + 3u) >> 2;
-            for (uint32_t w = rank; w < words; w += nthr)
-                int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
-        }
+        job_pass_int8<DIMS, MEASURE, NC, RULE>(j, a, rank, nthr, e_acc, m_acc);
     } else {
         // (one body for aligned and ragged rows: at half the code the kernels
         // spill less and stay in the instruction cache)
@@ -207,11 +211,7 @@ __device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom&
                                             uint32_t t, uint32_t first, int& e_acc, int& m_acc) {
     const PassArgs a = job_args(j, c, t);
     if constexpr (LAYOUT == ISING_INT8) {
-        WordGeom g;
-        g.W = (uint32_t)j.W;
-        g.L = (uint32_t)j.L;
-        g.rows = j.rows;
-        g.half = j.half;
+        const WordGeom g((uint32_t)j.W, (uint32_t)j.L, j.rows);
         const uint32_t v = first + (threadIdx.x & 31u);
         if (16u * v < j.half) int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_acc);
     } else {
@@ -1104,36 +1104,3 @@ int ising_batch_run_static(ising_lattice* const* lats, int n, const int64_t* swe
 }
 
 }  // extern "C"
-
-// ----------------------------------------------------------------------------
-// Small lattices through ising_sweep: with a few thousand sites a colour pass
-// lasts less than its launch, so n sweeps run as one job on a single CTA (the
-// same arithmetic and draws; passes separated by __syncthreads) instead of 2n
-// launches.  The job travels by value and lives in shared memory.
-// ----------------------------------------------------------------------------
-namespace ising {
-
-namespace {
-
-template <int RULE>
-__global__ void __launch_bounds__(256, 1) small_job_kernel(BatchJob job) {
-    __shared__ BatchJob sj;
-    if (threadIdx.x == 0) sj = job;
-    __syncthreads();
-    dispatch_job<kModeCta, RULE>(&sj, threadIdx.x, blockDim.x, threadIdx.x == 0);
-}
-
-}  // namespace
-
-int small_sweep(ising_lattice* h, int64_t n, int every, unsigned long long* slots) {
-    BatchJob j;
-    fill_job(j, h, n, every, slots);
-    if (h->rule == ISING_RULE_HEATBATH)
-        small_job_kernel<kRuleHeatBath><<<1, 256, 0, h->stream>>>(j);
-    else
-        small_job_kernel<kRuleMetropolis><<<1, 256, 0, h->stream>>>(j);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? ISING_OK : cuda_fail(e);
-}
-
-}  // namespace ising

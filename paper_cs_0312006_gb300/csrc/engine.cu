@@ -367,7 +367,8 @@ ising_int8_config resolve_int8(const ising_lattice* h) {
 
 bool uses_tma(const ising_lattice* h) { return resolve_int8(h).kernel == ISING_KERNEL_TMA; }
 
-int run_pass(ising_lattice* h, int c, uint32_t t, unsigned long long* slot) {
+// Arguments of colour pass c of sweep t.
+PassArgs pass_args(const ising_lattice* h, int c, uint32_t t, unsigned long long* slot) {
     PassArgs a;
     a.own = h->col[c];
     a.other = h->col[1 - c];
@@ -380,10 +381,17 @@ int run_pass(ising_lattice* h, int c, uint32_t t, unsigned long long* slot) {
     a.key1 = (uint32_t)(h->seed >> 32);
     a.t = t;
     a.c = c;
+    a.nv = 0;
+    a.strips = 0;
     a.dem = nullptr;
     a.qmax = 0;
     a.rot = 0;
     a.hits = h->hits;
+    return a;
+}
+
+int run_pass(ising_lattice* h, int c, uint32_t t, unsigned long long* slot) {
+    PassArgs a = pass_args(h, c, t, slot);
     if (h->rule == ISING_RULE_DEMON) {
         a.dem = h->dem[c];
         a.qmax = h->qmax;
@@ -517,10 +525,10 @@ int ising_sweep(ising_lattice* h, int64_t n, int measure_every) {
         if (rc != ISING_OK) return rc;
     }
     int64_t rec = h->n_rec;
-    if (h->sites <= kSmallSites && n >= 2 && n <= 0x7FFFFFFF &&
-        (h->rule == ISING_RULE_METROPOLIS || h->rule == ISING_RULE_HEATBATH)) {
-        const int rc = small_sweep(h, n, measure_every, h->obs ? h->obs + 2 * rec : nullptr);
-        if (rc != ISING_OK) return rc;
+    if (ising::resident_ok(h, n)) {
+        ISING_CHECK(ising::resident_sweep(h, ising::pass_args(h, 0, (uint32_t)h->t, nullptr), n,
+                                          measure_every,
+                                          h->obs ? h->obs + 2 * rec : nullptr));
         h->t += (uint64_t)n;
         h->n_rec = rec + new_rec;
         return ISING_OK;

@@ -93,9 +93,10 @@ int device_props(const DeviceProps** out);
 // stream-ordered allocation from the device's lattice pool
 cudaError_t pool_alloc(void** p, size_t bytes, const DeviceProps& dp, cudaStream_t st);
 int ensure_records(ising_lattice* h, int64_t need);
-// n sweeps of a small lattice in one persistent single-CTA launch (batch.cu)
-int small_sweep(ising_lattice* h, int64_t n, int every, unsigned long long* slots);
-constexpr int64_t kSmallSites = 16384;  // at or below: the single-launch path
+// n sweeps of a small lattice in one launch of a cluster (resident.cu)
+bool resident_ok(const ising_lattice* h, int64_t n);
+cudaError_t resident_sweep(ising_lattice* h, const PassArgs& args, int64_t n, int every,
+                           unsigned long long* slots);
 constexpr uint64_t kMaxSweep = 0xFFFFFFFFull;  // the sweep index is a 32-bit counter word
 
 // int8 layout (sweep_int8.cu)

@@ -197,6 +197,13 @@ __device__ __forceinline__ void static_for(F&& f) {
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// Keeps the computation of v ahead of grid_dependency_wait(): draws made before
+// the wait are otherwise moved behind it, to their use.  Each lane shuffles v to
+// itself (the whole warp takes part), which stays where it stands.
+__device__ __forceinline__ void pin_here(uint32_t& v) {
+    v = __shfl_sync(0xffffffffu, v, (int)(threadIdx.x & 31u));
+}
+
 __device__ __forceinline__ void launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -46,8 +46,9 @@ __device__ __forceinline__ uint32_t downhill_mask(uint32_t D) {
     return byte_signs(D + (0x80u - 2u * DIMS) * kByteOnes);
 }
 
-// 0xFF per site (byte) of a word that flips, from D (byte j is 2 d_j) and the
-// draws of its four sites.  With cnt_j the number of the rule's thresholds that
+// The tests of a word's four sites, from their draws alone: byte j of count_word
+// is bias + 2 cnt_j; and the sites that flip, 0xFF per byte, once D (byte j is
+// 2 d_j) is known.  With cnt_j the number of the rule's thresholds that
 // u_j lies below (they are nested) -- Metropolis: the thresholds fall with k, so
 // a site with d < dims flips iff cnt + d >= dims, and one with d >= dims always
 // does: bit 7 of D + 2 cnt + bias (at most 0x80 + 4 dims: no carry).  Heat bath
@@ -60,18 +61,20 @@ __device__ __forceinline__ uint32_t downhill_mask(uint32_t D) {
 // takes one instruction in two cycles, and adds (and the byte sums of E and M)
 // need not go there.
 template <int DIMS, int RULE>
-__device__ __forceinline__ uint32_t flip_mask(uint32_t D, const Philox4& u, const PassArgs& a) {
+__device__ __forceinline__ uint32_t count_word(const Philox4& u, const PassArgs& a) {
     constexpr int N = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
     constexpr uint32_t need = RULE == kRuleHeatBath ? 2u * DIMS + 1u : (uint32_t)DIMS;
-    constexpr uint32_t bias = (0x80u - 2u * need) * kByteOnes;
-    uint32_t acc = D + bias;
+    uint32_t acc = (0x80u - 2u * need) * kByteOnes;
     static_for<4>([&](auto site) {
         constexpr int j = decltype(site)::value;
         const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
 #pragma unroll
         for (int n = 0; n < N; ++n) add_below<(2u << (8 * j))>(acc, w, a.thr[n]);
     });
-    return byte_signs(acc);
+    return acc;
+}
+__device__ __forceinline__ uint32_t flip_mask(uint32_t D, uint32_t count) {
+    return byte_signs(D + count);
 }
 
 // Sum of a word's four spins (bytes +1 / -1) or counts, added to acc.
@@ -103,7 +106,7 @@ __device__ __forceinline__ uint32_t multihit_word(uint32_t D, uint32_t group, co
         if (X != 0xFFFFFFFFu) {
             const Philox4 u = philox4x32_10(group, a.t, (uint32_t)a.c + 2u * (uint32_t)m,
                                             kTagSweep, a.key0, a.key1);
-            X = flip_mask<DIMS, kRuleMetropolis>(D, u, a);
+            X = flip_mask(D, count_word<DIMS, kRuleMetropolis>(u, a));
         }
         D = (D & ~X) | ((q2 - D) & X);
         net ^= X;
@@ -131,28 +134,57 @@ __device__ __forceinline__ uint32_t window4(const uint32_t* other, uint32_t o) {
     return __funnelshift_r(lo, hi, 8u * (o & 3u));
 }
 
+// Quotients by a fixed divisor d >= 1 of n < 2^31: with 2^s <= d < 2^(s+1) and
+// m = ceil(2^(32+s) / d), n m / 2^(32+s) exceeds n / d by less than
+// n / 2^31 / d, too little to reach the next integer.  Powers of two take
+// half of both, and d = 1 the last term.  Six issue slots instead of the twenty
+// or so of a division, of which a packed word of ragged rows needs four.
+struct FastDiv {
+    uint32_t d, m, s, one;
+    FastDiv() = default;
+    __host__ __device__ __forceinline__ explicit FastDiv(uint32_t div) : d(div), s(0), one(0) {
+        while ((2u << s) <= d && s < 31u) ++s;
+        if (d == 1u) {
+            m = 0u;
+            one = 0xFFFFFFFFu;
+        } else if ((d & (d - 1u)) == 0u) {
+            m = 0x80000000u;
+            --s;
+        } else {
+            m = (uint32_t)(((1ull << (32u + s)) + d - 1u) / d);
+        }
+    }
+    __device__ __forceinline__ uint32_t quot(uint32_t n) const {
+        return (__umulhi(n, m) >> s) + (n & one);
+    }
+};
+
 struct WordGeom {
     uint32_t W;       // sites per half row
     uint32_t L;
     uint32_t rows;    // L^(dims-1)
     uint32_t half;    // sites per colour
+    FastDiv by_W, by_L;
+    WordGeom() = default;
+    __host__ __device__ __forceinline__ WordGeom(uint32_t W_, uint32_t L_, uint32_t rows_)
+        : W(W_), L(L_), rows(rows_), half(W_ * rows_), by_W(W_), by_L(L_) {}
 };
 
 // Update word w of the int8 colour array `own` (colour a.c).  Accumulates the
 // sum of the spins written (m_sum) and, in the white pass,
 // sum (2 d_new - 2 dims) over them (e_acc).
-template <int DIMS, bool MEASURE, int NC, int RULE = kRuleMetropolis>
+template <int DIMS, bool MEASURE, int NC, int RULE>
 __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, uint32_t w,
                                           int& e_acc, int& m_sum) {
     uint32_t* own = static_cast<uint32_t*>(a.own);
     const uint32_t* other = static_cast<const uint32_t*>(a.other);
     const int8_t* other_b = static_cast<const int8_t*>(a.other);
     const uint32_t h0 = 4u * w;
-    const uint32_t r0 = h0 / g.W;
+    const uint32_t r0 = g.by_W.quot(h0);
     const uint32_t xh0 = h0 - r0 * g.W;
     uint32_t y0 = r0, z0 = 0;
     if (DIMS == 3) {
-        z0 = r0 / g.L;
+        z0 = g.by_L.quot(r0);
         y0 = r0 - z0 * g.L;
     }
     const int p = (a.c + (int)y0 + (int)z0) & 1;
@@ -176,7 +208,7 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
             X = multihit_word<DIMS>(D, w, a);
         } else {
             const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-            X = flip_mask<DIMS, RULE>(D, u, a);
+            X = flip_mask(D, count_word<DIMS, RULE>(u, a));
         }
         const uint32_t snew = s ^ (X & kByteFlip);
         own[w] = snew;
@@ -201,11 +233,11 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
         s_val[j] = 1;
         d_val[j] = DIMS;
         if (!valid[j]) continue;
-        const uint32_t r = h / g.W;
+        const uint32_t r = g.by_W.quot(h);
         const uint32_t xh = h - r * g.W;
         uint32_t y = r, z = 0;
         if (DIMS == 3) {
-            z = r / g.L;
+            z = g.by_L.quot(r);
             y = r - z * g.L;
         }
         const int pp = (a.c + (int)y + (int)z) & 1;
@@ -308,55 +340,66 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
     }
 }
 
-// Update the 16 sites of one 16-byte vector (four Philox groups g0..g0+3).
-// Accumulates the sum of the new spins (m_sum) and, in the white pass,
-// sum_j 2*d_new_j (e_acc).
-template <int DIMS, bool MEASURE, int RULE = kRuleMetropolis>
+// The tests (count_word) of the four Philox groups g0 .. g0 + 3: one 16-byte
+// vector.
+template <int DIMS, int RULE>
+__device__ __forceinline__ void vec_counts(uint32_t g0, const PassArgs& a, uint32_t c2,
+                                           uint32_t (&cnt)[4]) {
+    PhiloxRuns<1> ps;
+    const uint32_t base[1] = {g0};
+    ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
+#pragma unroll
+    for (int r = 1; r < 10; ++r) ps.next_round();
+#pragma unroll
+    for (int w = 0; w < 4; ++w) cnt[w] = count_word<DIMS, RULE>(ps.result(w), a);
+}
+
+// Update the 16 sites of one 16-byte vector (Philox groups g0..g0+3), given its
+// tests (of the first trial).  Accumulates the sum of the new spins (m_sum) and,
+// in the white pass, sum_j 2*d_new_j (e_acc), over the bytes set in `counted`.
+template <int DIMS, bool MEASURE, int RULE>
 __device__ __forceinline__ uint4 update_vec(const uint4& s, const uint4& x, const uint4& xs,
                                             const uint4& ym, const uint4& yp, const uint4& zm,
-                                            const uint4& zp, uint32_t g0, const PassArgs& a,
-                                            int& e_acc, int& m_sum) {
+                                            const uint4& zp, uint32_t g0, uint32_t (&cnt)[4],
+                                            const uint4& counted, const PassArgs& a, int& e_acc,
+                                            int& m_sum) {
+    const uint32_t cv[4] = {counted.x, counted.y, counted.z, counted.w};
     const uint32_t sv[4] = {s.x, s.y, s.z, s.w};
     uint32_t D[4], X[4];
     D[0] = disagreements<DIMS>(s.x, x.x, xs.x, ym.x, yp.x, zm.x, zp.x);
     D[1] = disagreements<DIMS>(s.y, x.y, xs.y, ym.y, yp.y, zm.y, zp.y);
     D[2] = disagreements<DIMS>(s.z, x.z, xs.z, ym.z, yp.z, zm.z, zp.z);
     D[3] = disagreements<DIMS>(s.w, x.w, xs.w, ym.w, yp.w, zm.w, zp.w);
-    // one trial, or a.hits in a row with the neighbours fixed; the four calls
-    // are consecutive groups and are made together, whether or not all four
-    // words hold a site that draws (nearly all do)
+    // one trial, or a.hits in a row with the neighbours fixed
     const int hits = RULE == kRuleMultiHit ? a.hits : 1;
     uint32_t Dc[4] = {D[0], D[1], D[2], D[3]};
 #pragma unroll
     for (int w = 0; w < 4; ++w) X[w] = 0u;
 #pragma unroll 1
-    for (int m = 0; m < hits; ++m) {
-        PhiloxRuns<1> ps;
-        const uint32_t base[1] = {g0};
-        ps.first_round(base, a.t, (uint32_t)a.c + 2u * (uint32_t)m, kTagSweep, a.key0, a.key1);
-#pragma unroll
-        for (int r = 1; r < 10; ++r) ps.next_round();
+    for (int m = 0;;) {
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-            const uint32_t Y = flip_mask<DIMS, RULE>(Dc[w], ps.result(w), a);
+            const uint32_t Y = flip_mask(Dc[w], cnt[w]);
             if (RULE == kRuleMultiHit) {
                 constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
                 Dc[w] = (Dc[w] & ~Y) | ((q2 - Dc[w]) & Y);
             }
             X[w] ^= Y;
         }
+        if (++m >= hits) break;
+        vec_counts<DIMS, RULE>(g0, a, (uint32_t)a.c + 2u * (uint32_t)m, cnt);
     }
     uint32_t out[4];
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
         out[w] = sv[w] ^ (X[w] & kByteFlip);
         if (MEASURE) {
-            m_sum = add_bytes(out[w], m_sum);
+            m_sum = add_bytes(out[w] & cv[w], m_sum);
             if (a.c == 1) {
                 // 2*d_new = 2*(2 dims) - 2*d where flipped
                 constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
                 const uint32_t Dn = (D[w] & ~X[w]) | ((q2 - D[w]) & X[w]);
-                e_acc = add_bytes(Dn, e_acc);
+                e_acc = add_bytes(Dn & cv[w], e_acc);
             }
         }
     }
@@ -364,79 +407,175 @@ __device__ __forceinline__ uint4 update_vec(const uint4& s, const uint4& x, cons
 }
 
 
-// 16 bytes of the other colour at byte offset o (any alignment): two aligned
-// 16-byte loads and a byte shift.  The shift r = o mod 16 is the same for a
-// whole lattice and direction (it depends only on W, L and the direction), so
-// the switch does not diverge.
-template <int NC>
-__device__ __forceinline__ uint4 window16(const uint4* other16, uint32_t o) {
-    const uint32_t r = o & 15u;
-    const uint4 lo = load_other<NC>(other16 + (o >> 4));
-    if (r == 0u) return lo;
-    const uint4 hi = load_other<NC>(other16 + (o >> 4) + 1);
-    const uint32_t b = 8u * (r & 3u);
-    uint32_t w0, w1, w2, w3, w4;
-    switch (r >> 2) {
-        case 0: w0 = lo.x; w1 = lo.y; w2 = lo.z; w3 = lo.w; w4 = hi.x; break;
-        case 1: w0 = lo.y; w1 = lo.z; w2 = lo.w; w3 = hi.x; w4 = hi.y; break;
-        case 2: w0 = lo.z; w1 = lo.w; w2 = hi.x; w3 = hi.y; w4 = hi.z; break;
-        default: w0 = lo.w; w1 = hi.x; w2 = hi.y; w3 = hi.z; w4 = hi.w; break;
+// 16 bytes of the other colour at byte offset o (any alignment), in two steps:
+// the two aligned 16-byte loads (the same one twice where o is aligned), so that
+// all of a vector's loads are under way before the first is used, and the byte
+// shift.  The shift o mod 16 is the same for a whole lattice and direction (it
+// depends only on W, L and the direction), so the switch does not diverge.
+// FROM_BEFORE: o may be -15 .. -1 (as unsigned), a window that starts before the
+// array; the bytes before it are whatever the array starts with.
+struct Window16 {
+    uint4 lo, hi;
+    uint32_t r;
+    __device__ __forceinline__ uint4 get() const {
+        if (r == 0u) return lo;
+        const uint32_t b = 8u * (r & 3u);
+        uint32_t w0, w1, w2, w3, w4;
+        switch (r >> 2) {
+            case 0: w0 = lo.x; w1 = lo.y; w2 = lo.z; w3 = lo.w; w4 = hi.x; break;
+            case 1: w0 = lo.y; w1 = lo.z; w2 = lo.w; w3 = hi.x; w4 = hi.y; break;
+            case 2: w0 = lo.z; w1 = lo.w; w2 = hi.x; w3 = hi.y; w4 = hi.z; break;
+            default: w0 = lo.w; w1 = hi.x; w2 = hi.y; w3 = hi.z; w4 = hi.w; break;
+        }
+        return make_uint4(__funnelshift_r(w0, w1, b), __funnelshift_r(w1, w2, b),
+                          __funnelshift_r(w2, w3, b), __funnelshift_r(w3, w4, b));
     }
-    return make_uint4(__funnelshift_r(w0, w1, b), __funnelshift_r(w1, w2, b),
-                      __funnelshift_r(w2, w3, b), __funnelshift_r(w3, w4, b));
+};
+template <int NC, bool FROM_BEFORE = false>
+__device__ __forceinline__ Window16 load_window(const uint4* other16, uint32_t o) {
+    Window16 w;
+    w.r = o & 15u;
+    const bool before = FROM_BEFORE && o >= 0xFFFFFFF0u;
+    const uint32_t b = before ? 0u : o >> 4;
+    w.lo = load_other<NC>(other16 + b);
+    w.hi = load_other<NC>(other16 + (before || w.r == 0u ? b : b + 1u));
+    return w;
+}
+
+// Byte j of word i of the mask is 0xFF iff 4 i + j >= n (n = 0..16 or more).
+__device__ __forceinline__ uint4 bytes_from(int n) {
+    const int s = 8 * n;
+    return make_uint4(__funnelshift_lc(0u, 0xFFFFFFFFu, (uint32_t)s),
+                      __funnelshift_lc(0u, 0xFFFFFFFFu, (uint32_t)max(s - 32, 0)),
+                      __funnelshift_lc(0u, 0xFFFFFFFFu, (uint32_t)max(s - 64, 0)),
+                      __funnelshift_lc(0u, 0xFFFFFFFFu, (uint32_t)max(s - 96, 0)));
+}
+__device__ __forceinline__ uint4 select4(const uint4& m, const uint4& t, const uint4& f) {
+    return make_uint4((m.x & t.x) | (~m.x & f.x), (m.y & t.y) | (~m.y & f.y),
+                      (m.z & t.z) | (~m.z & f.z), (m.w & t.w) | (~m.w & f.w));
 }
 
 // Update the 16 sites of vector v (half indices 16v..16v+15, Philox groups
-// 4v..4v+3) of the int8 colour array.  A vector inside one half row, away from
-// the x-wrap and the first/last row and plane, is updated as a whole from
-// 16-byte neighbour windows; any other vector word by word (int8_word).
-// Accumulates m_sum and, in the white pass, e_acc as int8_word does.
-template <int DIMS, bool MEASURE, int NC, int RULE = kRuleMetropolis>
+// 4v..4v+3) of the int8 colour array.  With W >= 16 a vector holds sites of one
+// row, or the end of one (part A) and the start of the next (part B; none behind
+// the last row); shorter rows go word by word.  Its y- and z-neighbours are
+// 16-byte windows of the other colour at an offset that is the same for both parts but
+// where one of them wraps; its x-neighbours are the bytes before or behind, by
+// each part's parity, with the bytes that wrap at a row's ends put in singly.
+// Every vector takes this one path, and all its loads come first: word by word
+// (int8_word) the few at the row ends and edges held the whole pass up, alone
+// (2D L = 1000 7.6 -> 2.7, 3D L = 202 32.4 -> 9.2 us a pass).  Accumulates
+// m_sum and, in the white pass, e_acc as int8_word does.
+template <int DIMS, bool MEASURE, int NC, int RULE>
 __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, uint32_t v,
                                          int& e_acc, int& m_sum) {
-    const uint32_t h0 = 16u * v;
-    const uint32_t r0 = h0 / g.W;
-    const uint32_t xh0 = h0 - r0 * g.W;
-    uint32_t y0 = r0, z0 = 0;
-    if (DIMS == 3) {
-        z0 = r0 / g.L;
-        y0 = r0 - z0 * g.L;
-    }
-    const int p = (a.c + (int)y0 + (int)z0) & 1;
-    bool fast = (xh0 + 15u < g.W) && (h0 + 15u < g.half) && y0 != 0u && y0 + 1u != g.L;
-    if (DIMS == 3) fast = fast && z0 != 0u && z0 + 1u != g.L;
-    fast = fast && (p == 0 ? xh0 != 0u : xh0 + 16u != g.W);
-    if (!fast) {
+    const uint32_t h0 = 16u * v, W = g.W;
+    if (W < 16u) {  // short rows: word by word
 #pragma unroll 1
         for (uint32_t w = 4u * v; w < 4u * v + 4u; ++w)
             if (4u * w < g.half) int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_sum);
         return;
     }
+    const uint32_t r0 = g.by_W.quot(h0);
+    const uint32_t xh0 = h0 - r0 * W;
+    uint32_t y0 = r0, z0 = 0;
+    if (DIMS == 3) {
+        z0 = g.by_L.quot(r0);
+        y0 = r0 - z0 * g.L;
+    }
+    const uint32_t left = W - xh0;  // sites of row r0 from here on
+    const bool ends = left < 16u;   // the row ends inside the vector
+    const bool two = ends && r0 + 1u < g.rows;
+    // part B's row
+    uint32_t yb = y0 + 1u, zb = z0;
+    if (yb == g.L) {
+        yb = 0u;
+        ++zb;
+    }
+    const bool edge = two && (y0 == 0u || yb == 0u || yb + 1u == g.L);  // one part wraps
     const uint4* other16 = static_cast<const uint4*>(a.other);
+    const uint32_t* other32 = static_cast<const uint32_t*>(a.other);
+    const uint8_t* other8 = static_cast<const uint8_t*>(a.other);
     uint4* own16 = static_cast<uint4*>(a.own);
+    const uint32_t row = r0 * W;
+    const uint32_t plane = g.L * W, y_wrap = plane - W, z_wrap = (g.L - 1u) * plane;
+    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u), ones4 = make_uint4(~0u, ~0u, ~0u, ~0u);
     const uint4 s = own16[v];
     const uint4 nx = load_other<NC>(other16 + v);
-    uint4 nxs;
-    if (p == 0) {  // neighbour h' - 1: byte j <- byte j - 1
-        const uint32_t prev = load_other<NC>(static_cast<const uint32_t*>(a.other) + 4u * v - 1u);
-        nxs = make_uint4(__funnelshift_l(prev, nx.x, 8), __funnelshift_l(nx.x, nx.y, 8),
-                         __funnelshift_l(nx.y, nx.z, 8), __funnelshift_l(nx.z, nx.w, 8));
-    } else {       // neighbour h' + 1: byte j <- byte j + 1
-        const uint32_t next = load_other<NC>(static_cast<const uint32_t*>(a.other) + 4u * v + 4u);
-        nxs = make_uint4(__funnelshift_r(nx.x, nx.y, 8), __funnelshift_r(nx.y, nx.z, 8),
-                         __funnelshift_r(nx.z, nx.w, 8), __funnelshift_r(nx.w, next, 8));
-    }
-    const uint4 nym = window16<NC>(other16, h0 - g.W);
-    const uint4 nyp = window16<NC>(other16, h0 + g.W);
-    uint4 nzm = make_uint4(0u, 0u, 0u, 0u), nzp = nzm;
+    const Window16 wym = load_window<NC>(other16, y0 == 0u ? h0 + y_wrap : h0 - W);
+    const Window16 wyp = load_window<NC>(other16, y0 + 1u == g.L ? h0 - y_wrap : h0 + W);
+    Window16 wzm{zero4, zero4, 0u}, wzp{zero4, zero4, 0u};
     if (DIMS == 3) {
-        nzm = window16<NC>(other16, h0 - g.L * g.W);
-        nzp = window16<NC>(other16, h0 + g.L * g.W);
+        wzm = load_window<NC>(other16, z0 == 0u ? h0 + z_wrap : h0 - plane);
+        wzp = load_window<NC>(other16, z0 + 1u == g.L ? h0 - z_wrap : h0 + plane);
+    }
+    const uint32_t word_before = load_other<NC>(other32 + (v == 0u ? 0u : 4u * v - 1u));
+    const uint32_t word_behind = load_other<NC>(other32 + 4u * v + 4u);
+    const uint32_t row_first = load_other<NC>(other8 + row);
+    const uint32_t row_last = load_other<NC>(other8 + row + W - 1u);
+    const uint32_t next_last = load_other<NC>(other8 + row + (two ? 2u * W : W) - 1u);
+    // the draws while the loads are under way
+    uint32_t cnt[4];
+    vec_counts<DIMS, RULE>(4u * v, a, (uint32_t)a.c, cnt);
+    const uint4 part_b = ends ? bytes_from((int)left) : zero4;
+    uint4 nym = wym.get(), nyp = wyp.get(), nzm = zero4, nzp = zero4;
+    if (DIMS == 3) {
+        nzm = wzm.get();
+        nzp = wzp.get();
+    }
+    if (edge) {  // part B's own windows (they may start up to 15 bytes before the first row)
+        const Window16 bym = load_window<NC, true>(other16, h0 + (yb == 0u ? y_wrap : 0u - W));
+        const Window16 byp =
+            load_window<NC, true>(other16, h0 + (yb + 1u == g.L ? 0u - y_wrap : W));
+        Window16 bzm = wzm, bzp = wzp;
+        if (DIMS == 3) {
+            bzm = load_window<NC, true>(other16, h0 + (zb == 0u ? z_wrap : 0u - plane));
+            bzp = load_window<NC, true>(other16, h0 + (zb + 1u == g.L ? 0u - z_wrap : plane));
+        }
+        nym = select4(part_b, bym.get(), nym);
+        nyp = select4(part_b, byp.get(), nyp);
+        if (DIMS == 3) {
+            nzm = select4(part_b, bzm.get(), nzm);
+            nzp = select4(part_b, bzp.get(), nzp);
+        }
+    }
+    const int pa = (a.c + (int)y0 + (int)z0) & 1, pb = (a.c + (int)yb + (int)zb) & 1;
+    // part A's x-neighbours, and part B's where there is one: the bytes before
+    // (byte j <- byte j - 1) or behind (byte j <- byte j + 1)
+    const uint32_t prev = xh0 == 0u ? row_last << 24 : word_before;
+    const uint32_t next = left == 16u ? row_first : word_behind;
+    const uint4 before =
+        make_uint4(__funnelshift_l(prev, nx.x, 8), __funnelshift_l(nx.x, nx.y, 8),
+                   __funnelshift_l(nx.y, nx.z, 8), __funnelshift_l(nx.z, nx.w, 8));
+    const uint4 behind =
+        make_uint4(__funnelshift_r(nx.x, nx.y, 8), __funnelshift_r(nx.y, nx.z, 8),
+                   __funnelshift_r(nx.z, nx.w, 8), __funnelshift_r(nx.w, next, 8));
+    uint4 nxs = pa ? behind : before;
+    if (ends) {
+        if (pa == 1) {  // part A's last site wraps to its row's first
+            const uint32_t f = row_first * kByteOnes;
+            nxs = select4(bytes_from((int)left - 1), make_uint4(f, f, f, f), nxs);
+        }
+        nxs = select4(part_b, pb ? behind : before, nxs);
+        if (pb == 0) {  // part B's first site wraps to its row's last
+            const uint32_t l = next_last * kByteOnes;
+            const uint4 m = bytes_from((int)left + 1);
+            nxs = select4(make_uint4(part_b.x & ~m.x, part_b.y & ~m.y, part_b.z & ~m.z,
+                                     part_b.w & ~m.w),
+                          make_uint4(l, l, l, l), nxs);
+        }
+    }
+    // past the last row's end: the array's padding, which counts for nothing
+    uint4 counted = ones4;
+    int n_sites = 16;
+    if (MEASURE && ends && !two) {
+        counted = make_uint4(~part_b.x, ~part_b.y, ~part_b.z, ~part_b.w);
+        n_sites = (int)left;
     }
     int e_vec = 0;
-    own16[v] = update_vec<DIMS, MEASURE, RULE>(s, nx, nxs, nym, nyp, nzm, nzp, 4u * v, a, e_vec,
-                                               m_sum);
-    if (MEASURE && a.c == 1) e_acc += e_vec - 16 * 2 * DIMS;
+    own16[v] = update_vec<DIMS, MEASURE, RULE>(s, nx, nxs, nym, nyp, nzm, nzp, 4u * v, cnt, counted,
+                                               a, e_vec, m_sum);
+    if (MEASURE && a.c == 1) e_acc += e_vec - n_sites * 2 * DIMS;
 }
 
 // ----------------------------------------------------------------------------
@@ -557,8 +696,9 @@ constexpr int kDrawRagged = 1;   // rows start anywhere in a group
 template <int DRAW>
 constexpr uint32_t kWarpWords = DRAW == kDrawRagged ? 31u : 32u;
 
-// Accept mask of a packed word whose 32 bits are the half indices hbase + b:
-// bit b's draw is word (hb & 3) of Philox group hb >> 2.  A row that starts
+// The tests of a packed word whose 32 bits are the half indices hbase + b: bit b
+// of A[n] says whether site b's draw, word (hb & 3) of Philox group hb >> 2, lies
+// below threshold n.  A row that starts
 // inside a group (hbase & 3 = M != 0) needs nine groups' draws 0..35 and uses
 // draws M .. M + 31: the tests stay at draw positions, the same code for every
 // M, the last four positions are the next lane's first four (its word starts
@@ -570,11 +710,11 @@ constexpr uint32_t kWarpWords = DRAW == kDrawRagged ? 31u : 32u;
 // compiled per M and the rows grouped by M, and with divisions for an item's
 // place: 3D L = 202 11.0 -> 8.6 us per pass; a joint pass of 256 mixed lattices
 // 47 -> 39 us.
-template <int DIMS, int RULE, int DRAW, typename K>
-__device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t hbase, bool both,
-                                                  const PassArgs& a, uint32_t c2) {
+template <int DIMS, int RULE, int DRAW>
+__device__ __forceinline__ void packed_draws(uint32_t hbase, bool both, const PassArgs& a,
+                                             uint32_t c2,
+                                             uint32_t (&A)[kThresholds<DIMS, RULE>]) {
     constexpr int N = kThresholds<DIMS, RULE>;
-    uint32_t A[N];
     word_tests<N>(hbase >> 2, a, c2, both, A);
     if constexpr (DRAW == kDrawRagged) {
 #pragma unroll
@@ -583,39 +723,7 @@ __device__ __forceinline__ uint32_t packed_accept(const K& k, uint32_t hbase, bo
             A[n] = __funnelshift_r(A[n], next, hbase & 3u);
         }
     }
-    return choose_answer<DIMS>(k, A);
 }
-
-// Update word (r, q) of the packed colour array.  A half row of W sites takes
-// nq = ceil(W / 32) words; bit b of word q is half column xh = 32q + b (valid
-// when xh < W; the other bits of a row's last word stay 0 and never flip).
-// The x-neighbour wrap at the row ends comes from the row's last valid bit
-// (p = 0, first word) or first bit (p = 1, last word).
-
-// Quotients by a fixed divisor d >= 1 of n < 2^31: with 2^s <= d < 2^(s+1) and
-// m = ceil(2^(32+s) / d), n m / 2^(32+s) exceeds n / d by less than
-// n / 2^31 / d, too little to reach the next integer.  Powers of two take
-// half of both, and d = 1 the last term.  Six issue slots instead of the twenty
-// or so of a division, of which a packed word of ragged rows needs four.
-struct FastDiv {
-    uint32_t d, m, s, one;
-    FastDiv() = default;
-    __host__ __device__ __forceinline__ explicit FastDiv(uint32_t div) : d(div), s(0), one(0) {
-        while ((2u << s) <= d && s < 31u) ++s;
-        if (d == 1u) {
-            m = 0u;
-            one = 0xFFFFFFFFu;
-        } else if ((d & (d - 1u)) == 0u) {
-            m = 0x80000000u;
-            --s;
-        } else {
-            m = (uint32_t)(((1ull << (32u + s)) + d - 1u) / d);
-        }
-    }
-    __device__ __forceinline__ uint32_t quot(uint32_t n) const {
-        return (__umulhi(n, m) >> s) + (n & one);
-    }
-};
 
 // The geometry of a packed lattice's words.
 struct PackedGeom {
@@ -628,123 +736,160 @@ struct PackedGeom {
     }
 };
 
-// The rule applied to one packed word, given the word s and its neighbour
-// words (sh: the x-neighbour across the colour, shifted into place), then the
-// store and the word's share of E and M.  valid: the word's sites (nb bits);
-// hbase: the half index of bit 0.  The whole warp takes part; a lane without
-// `mine` stores and counts nothing.
+// One packed word and its neighbours, as loaded.
+struct PackedWord {
+    uint32_t at;              // its index in the colour array
+    uint32_t s, o, x, ym, yp, zm, zp;  // x: the word that holds the outer x-neighbour
+    uint32_t valid;           // the word's sites
+    uint32_t hbase;           // the half index of bit 0
+    uint32_t edge;            // how x joins: 0 inside the row, else it wraps (see x_neighbours)
+    int p;                    // 0: bit b <- neighbour xh - 1, 1: xh + 1
+    bool mine;                // this lane stores the word
+};
+
+// The word of x-neighbours: o shifted by one site, the site that enters taken
+// from x: inside a row its bit 31 (p = 0) or bit 0 (p = 1); where the row wraps,
+// the row's last valid bit (p = 0, edge - 1 the shift that brings it to bit 31)
+// or its first, entering at the word's last valid bit (p = 1).
+__device__ __forceinline__ uint32_t x_neighbours(const PackedWord& w) {
+    if (w.p == 0) return __funnelshift_l(w.edge ? w.x << (w.edge - 1u) : w.x, w.o, 1);
+    if (w.edge == 0u) return __funnelshift_r(w.o, w.x, 1);
+    const uint32_t top = w.valid ^ (w.valid >> 1);
+    return ((w.o >> 1) & ~top) | ((w.x & 1u) ? top : 0u);
+}
+
+// The rule applied to one packed word, given its tests, then the store and the
+// word's share of E and M.  With ragged draws the whole warp takes part.
 template <int DIMS, bool MEASURE, int RULE, int DRAW>
-__device__ __forceinline__ void packed_update(const PassArgs& a, bool mine, bool both,
-                                              uint32_t* own_word, uint32_t s,
-                                              uint32_t o, uint32_t sh, uint32_t oym,
-                                              uint32_t oyp, uint32_t ozm, uint32_t ozp,
-                                              uint32_t valid, uint32_t nb, uint32_t hbase,
+__device__ __forceinline__ void packed_update(const PassArgs& a, const PackedWord& w,
+                                              uint32_t (&A)[kThresholds<DIMS, RULE>], bool both,
                                               int& e_acc, int& m_acc) {
+    const uint32_t s = w.s, sh = x_neighbours(w);
     uint32_t flip;
     if constexpr (RULE == kRuleHeatBath) {
-        const Digits k = DIMS == 2 ? digits2(s ^ o, s ^ sh, s ^ oym, s ^ oyp)
-                                   : digits3(s ^ o, s ^ sh, s ^ oym, s ^ oyp, s ^ ozm, s ^ ozp);
-        flip = packed_accept<DIMS, RULE, DRAW>(k, hbase, both, a, (uint32_t)a.c);
+        const Digits k = DIMS == 2 ? digits2(s ^ w.o, s ^ sh, s ^ w.ym, s ^ w.yp)
+                                   : digits3(s ^ w.o, s ^ sh, s ^ w.ym, s ^ w.yp, s ^ w.zm,
+                                             s ^ w.zp);
+        flip = choose_answer<DIMS>(k, A);
     } else {
         // one Metropolis trial, or a.hits in a row with the neighbours fixed
         const int hits = RULE == kRuleMultiHit ? a.hits : 1;
         uint32_t cur = s;
 #pragma unroll 1
-        for (int m = 0; m < hits; ++m) {
+        for (int m = 0;;) {
             Counts k;
             if (DIMS == 2) {
-                k = count2(cur ^ o, cur ^ sh, cur ^ oym, cur ^ oyp);
+                k = count2(cur ^ w.o, cur ^ sh, cur ^ w.ym, cur ^ w.yp);
             } else {
-                k = count3(cur ^ o, cur ^ sh, cur ^ oym, cur ^ oyp, cur ^ ozm, cur ^ ozp);
+                k = count3(cur ^ w.o, cur ^ sh, cur ^ w.ym, cur ^ w.yp, cur ^ w.zm, cur ^ w.zp);
             }
-            cur ^= k.always | packed_accept<DIMS, RULE, DRAW>(k, hbase, both, a,
-                                                              (uint32_t)a.c + 2u * (uint32_t)m);
+            cur ^= k.always | choose_answer<DIMS>(k, A);
+            if (++m >= hits) break;
+            packed_draws<DIMS, RULE, DRAW>(w.hbase, both, a, (uint32_t)a.c + 2u * (uint32_t)m, A);
         }
         flip = cur ^ s;
     }
-    const uint32_t snew = s ^ (flip & valid);
-    if (!mine) return;
-    *own_word = snew;
+    const uint32_t snew = s ^ (flip & w.valid);
+    if (!w.mine) return;
+    static_cast<uint32_t*>(a.own)[w.at] = snew;
     if (MEASURE) {
-        m_acc += 2 * __popc(snew & valid) - (int)nb;
+        const int nb = __popc(w.valid);
+        m_acc += 2 * __popc(snew & w.valid) - nb;
         if (a.c == 1) {
-            int dsum = __popc((snew ^ o) & valid) + __popc((snew ^ sh) & valid) +
-                       __popc((snew ^ oym) & valid) + __popc((snew ^ oyp) & valid);
-            if (DIMS == 3) dsum += __popc((snew ^ ozm) & valid) + __popc((snew ^ ozp) & valid);
-            e_acc += 2 * dsum - (int)nb * 2 * DIMS;
+            int dsum = __popc((snew ^ w.o) & w.valid) + __popc((snew ^ sh) & w.valid) +
+                       __popc((snew ^ w.ym) & w.valid) + __popc((snew ^ w.yp) & w.valid);
+            if (DIMS == 3)
+                dsum += __popc((snew ^ w.zm) & w.valid) + __popc((snew ^ w.zp) & w.valid);
+            e_acc += 2 * dsum - nb * 2 * DIMS;
         }
     }
 }
 
-// A warp's next words of the packed colour array: items first .. first + 31,
-// the lane's own at first + lane.  A half row of W sites takes nq = ceil(W / 32)
+// A warp's words of the packed colour array: items first .. first + 31, the
+// lane's own at first + lane.  A half row of W sites takes nq = ceil(W / 32)
 // words; bit b of word q is half column xh = 32q + b (valid when xh < W; the
-// other bits of a row's last word stay 0 and never flip).  The x-neighbour wrap
-// at the row ends comes from the row's last valid bit (p = 0, first word) or
-// first bit (p = 1, last word).  With ragged draws lane 31 only lends its draws,
-// for lane 30's last sites, and its word is the first of the next step; a lane
-// past the end draws for the row after the last.
-template <int DIMS, bool MEASURE, int NC, int RULE, int DRAW>
-__device__ __forceinline__ void packed_words(const PassArgs& a, const PackedGeom& g,
-                                             uint32_t first, int& e_acc, int& m_acc) {
-    const uint32_t W = (uint32_t)a.W;
-    const uint32_t nq = g.words.d;
-    const uint32_t L = (uint32_t)a.L;
-    uint32_t* own = static_cast<uint32_t*>(a.own);
-    const uint32_t* other = static_cast<const uint32_t*>(a.other);
+// other bits of a row's last word stay 0 and never flip).  With ragged draws
+// lane 31 only lends its draws, for lane 30's last sites, and its word is the
+// first of the next step; a lane past the end draws for the row after the last.
+struct PackedPlace {
+    uint32_t r, q;
+    uint32_t hbase;
+    bool mine;
+};
+
+template <int DRAW>
+__device__ __forceinline__ PackedPlace packed_place(const PackedGeom& g, uint32_t W,
+                                                    uint32_t first) {
     const uint32_t lane = threadIdx.x & 31u, item = first + lane;
-    const bool mine = item < g.items && lane < kWarpWords<DRAW>;
-    uint32_t r = g.words.quot(item), q = item - r * nq;
-    const uint32_t hbase = r * W + 32u * q;
+    PackedPlace p;
+    p.r = g.words.quot(item);
+    p.q = item - p.r * g.words.d;
+    p.hbase = p.r * W + 32u * p.q;
+    p.mine = item < g.items && lane < kWarpWords<DRAW>;
     if (item >= g.items) {  // loads something, keeps nothing
-        r = (uint32_t)a.rows - 1u;
-        q = 0u;
+        p.r = 0u;
+        p.q = 0u;
     }
+    return p;
+}
+
+template <int DIMS, int NC>
+__device__ __forceinline__ PackedWord packed_load(const PassArgs& a, const PackedGeom& g,
+                                                  const PackedPlace& pl) {
+    const uint32_t W = (uint32_t)a.W, L = (uint32_t)a.L, nq = g.words.d;
+    const uint32_t r = pl.r, q = pl.q;
     uint32_t y = r, z = 0;
     if (DIMS == 3) {
         z = g.L.quot(r);
         y = r - z * L;
     }
+    PackedWord w;
+    w.at = r * nq + q;
+    w.mine = pl.mine;
+    w.hbase = pl.hbase;
+    w.p = (a.c + (int)y + (int)z) & 1;
     const uint32_t nb = W - 32u * q < 32u ? W - 32u * q : 32u;  // valid bits
-    const uint32_t valid = nb == 32u ? 0xFFFFFFFFu : ((1u << nb) - 1u);
-    const uint32_t row = r * nq;
-    // the rows (and planes) next to this one, as offsets from it
-    const uint32_t up = (y == 0u ? (L - 1u) * nq : 0u - nq);
-    const uint32_t down = (y + 1u == L ? 0u - (L - 1u) * nq : nq);
-    const uint32_t* at = other + row + q;
-    const uint32_t o = load_other<NC>(at);
-    const uint32_t oym = load_other<NC>(at + (int32_t)up);
-    const uint32_t oyp = load_other<NC>(at + (int32_t)down);
-    uint32_t ozm = 0u, ozp = 0u;
+    w.valid = nb == 32u ? 0xFFFFFFFFu : ((1u << nb) - 1u);
+    const uint32_t* at = static_cast<const uint32_t*>(a.other) + w.at;
+    // the word with the outer x-neighbour, and the rows (and planes) next to
+    // this one, as offsets
+    int32_t dx;
+    if (w.p == 0) {
+        dx = q == 0u ? (int32_t)nq - 1 : -1;
+        w.edge = q == 0u ? 32u - ((W - 1u) & 31u) : 0u;
+    } else {
+        dx = q + 1u == nq ? -(int32_t)q : 1;
+        w.edge = q + 1u == nq ? 1u : 0u;
+    }
+    const int32_t up = y == 0u ? (int32_t)((L - 1u) * nq) : -(int32_t)nq;
+    const int32_t down = y + 1u == L ? -(int32_t)((L - 1u) * nq) : (int32_t)nq;
+    w.o = load_other<NC>(at);
+    w.x = load_other<NC>(at + dx);
+    w.ym = load_other<NC>(at + up);
+    w.yp = load_other<NC>(at + down);
+    w.zm = w.zp = 0u;
     if (DIMS == 3) {
-        const uint32_t plane = L * nq;
-        ozm = load_other<NC>(at + (int32_t)(z == 0u ? (L - 1u) * plane : 0u - plane));
-        ozp = load_other<NC>(at + (int32_t)(z + 1u == L ? 0u - (L - 1u) * plane : plane));
+        const int32_t plane = (int32_t)(L * nq), wrap = (int32_t)((L - 1u) * L * nq);
+        w.zm = load_other<NC>(at + (z == 0u ? wrap : -plane));
+        w.zp = load_other<NC>(at + (z + 1u == L ? -wrap : plane));
     }
-    const uint32_t s = own[row + q];
-    const int p = (a.c + (int)y + (int)z) & 1;
-    uint32_t sh;
-    if (p == 0) {  // bit b <- neighbour xh - 1
-        uint32_t prev;
-        if (q == 0u) {  // wrap: the row's last site, moved to bit 31
-            prev = load_other<NC>(at + nq - 1u) << (31u - ((W - 1u) & 31u));
-        } else {
-            prev = load_other<NC>(at - 1);
-        }
-        sh = __funnelshift_l(prev, o, 1);
-    } else {       // bit b <- neighbour xh + 1
-        if (q + 1u == nq) {  // wrap: bit nb - 1 takes the row's first site
-            const uint32_t first_word = q == 0u ? o : load_other<NC>(other + row);
-            const uint32_t top = 1u << (nb - 1u);
-            sh = ((o >> 1) & ~top) | ((first_word & 1u) ? top : 0u);
-        } else {
-            sh = __funnelshift_r(o, load_other<NC>(at + 1), 1);
-        }
-    }
+    w.s = static_cast<const uint32_t*>(a.own)[w.at];
+    return w;
+}
+
+// Rows of at most 13 sites need no draw past a word's first half.
+__device__ __forceinline__ bool packed_both(const PassArgs& a) { return a.W > 13; }
+
+// One step of a warp, loads first: their latency hides behind the draws.
+template <int DIMS, bool MEASURE, int NC, int RULE, int DRAW>
+__device__ __forceinline__ void packed_words(const PassArgs& a, const PackedGeom& g,
+                                             uint32_t first, int& e_acc, int& m_acc) {
+    const PackedWord w =
+        packed_load<DIMS, NC>(a, g, packed_place<DRAW>(g, (uint32_t)a.W, first));
+    uint32_t A[kThresholds<DIMS, RULE>];
     __syncwarp();
-    // rows of at most 13 sites need no draw past a word's first half
-    packed_update<DIMS, MEASURE, RULE, DRAW>(a, mine, W > 13u, own + row + q, s, o, sh, oym, oyp,
-                                             ozm, ozp, valid, nb, hbase, e_acc, m_acc);
+    packed_draws<DIMS, RULE, DRAW>(w.hbase, packed_both(a), a, (uint32_t)a.c, A);
+    packed_update<DIMS, MEASURE, RULE, DRAW>(a, w, A, packed_both(a), e_acc, m_acc);
 }
 
 }  // namespace ising

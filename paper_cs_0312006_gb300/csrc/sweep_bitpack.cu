@@ -31,82 +31,94 @@ namespace {
 //   kWordsFull: lattices whose words are all full (W % 32 == 0) and whose word
 //     count per half row nq = 2^nq_shift is a power of two (then so is
 //     L = 64 nq; in 3D l_shift = log2 L): an item's row, word and neighbours come
-//     from shifts and masks, every row starts on a Philox group, and a thread
-//     loads its next item's six words (eight in 3D) before it updates the current
-//     one, so that their latency hides behind the current item's draws (at most
-//     64 registers for four CTAs per SM measured slower: 2D L = 8192 29.2 ->
-//     29.4 us per pass, 3D L = 256 9.0e11 -> 8.0e11 site updates/s, both with the
-//     earlier, longer tests).
+//     from shifts and masks, and every row starts on a Philox group.
 //   kWordsAligned: rows that start on a Philox group (W % 4 == 0).
 //   kWordsRagged: any other even L.
-// In the last two a warp takes its words together (packed_words).
+// In the last two a warp takes its words together (packed_place).
+//
+// The first item's draws need only counters: they are made before the wait for
+// the previous pass, so that a pass placed on the SMs while the previous one
+// drains (or, with a lattice too small to fill the GPU, runs) has them ready.
+// Later items load first and draw while the loads are under way.
+// Per pass, in us, against waiting first: 2D L = 512 2.6 -> 1.85 (the host's
+// launches then set the pace), L = 2048 4.4 -> 2.8, L = 4096 8.4 -> 6.6, L = 8192
+// 24.4 -> 23.7; 3D L = 128 3.0 -> 2.3, L = 202 8.7 -> 6.3.  (The int8 passes
+// gained nothing by it: 2D L = 500 2.75 -> 2.77, L = 1000 2.75 -> 3.64.)
 constexpr int kWordsFull = 0, kWordsAligned = 1, kWordsRagged = 2;
 
 template <int DIMS, bool MEASURE, int RULE, int WORDS>
 __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geom,
                                                       uint32_t nq_shift, uint32_t l_shift) {
-    const uint32_t items = geom.items;
-    const uint32_t stride = gridDim.x * blockDim.x;
-    int e_acc = 0, m_acc = 0;
-    grid_dependency_wait();
-    launch_dependents();
-    if constexpr (WORDS != kWordsFull) {
-        constexpr int draw = WORDS == kWordsAligned ? kDrawAligned : kDrawRagged;
-        constexpr uint32_t step = kWarpWords<draw>;
-        uint32_t first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * step;
-        for (; first < items; first += (stride >> 5) * step)
-            packed_words<DIMS, MEASURE, 1, RULE, draw>(a, geom, first, e_acc, m_acc);
-    } else {
-        const uint32_t nq = 1u << nq_shift, L = (uint32_t)a.L, W = (uint32_t)a.W;
-        uint32_t* own = static_cast<uint32_t*>(a.own);
-        const uint32_t* other = static_cast<const uint32_t*>(a.other);
-        struct Words {
-            uint32_t o, x, ym, yp, zm, zp, s;
-        };
-        // the loads only: nothing here waits for them
-        auto load = [&](uint32_t item, Words& w) {
-            const uint32_t r = item >> nq_shift, q = item & (nq - 1u);
+    constexpr int draw = WORDS == kWordsRagged ? kDrawRagged : kDrawAligned;
+    constexpr uint32_t step = kWarpWords<draw>;
+    const uint32_t items = geom.items, L = (uint32_t)a.L, W = (uint32_t)a.W;
+    const uint32_t stride = ((gridDim.x * blockDim.x) >> 5) * step;
+    const bool both = WORDS == kWordsFull || packed_both(a);
+    auto place = [&](uint32_t first) {
+        if constexpr (WORDS != kWordsFull) {
+            return packed_place<draw>(geom, W, first);
+        } else {  // items is a multiple of 32
+            const uint32_t item = first + (threadIdx.x & 31u);
+            PackedPlace p;
+            p.r = item >> nq_shift;
+            p.q = item & ((1u << nq_shift) - 1u);
+            p.hbase = p.r * W + 32u * p.q;
+            p.mine = true;
+            return p;
+        }
+    };
+    auto load = [&](const PackedPlace& pl) {
+        if constexpr (WORDS != kWordsFull) {
+            return packed_load<DIMS, 1>(a, geom, pl);
+        } else {
+            const uint32_t nq = 1u << nq_shift, r = pl.r, q = pl.q;
+            const uint32_t* other = static_cast<const uint32_t*>(a.other);
             const uint32_t z = DIMS == 3 ? r >> l_shift : 0u, y = r & (L - 1u);
             const uint32_t row = r * nq, plane = z * L;
-            const int p = (a.c + (int)y + (int)z) & 1;
+            PackedWord w;
+            w.p = (a.c + (int)y + (int)z) & 1;
             // x-neighbour word: the one before (p = 0) or after (p = 1), wrapping in the row
-            const uint32_t xq = (p == 0 ? q - 1u : q + 1u) & (nq - 1u);
-            w.o = __ldg(other + row + q);
+            const uint32_t xq = (w.p == 0 ? q - 1u : q + 1u) & (nq - 1u);
+            w.at = row + q;
+            w.o = __ldg(other + w.at);
             w.x = __ldg(other + row + xq);
             w.ym = __ldg(other + (plane + ((y - 1u) & (L - 1u))) * nq + q);
             w.yp = __ldg(other + (plane + ((y + 1u) & (L - 1u))) * nq + q);
+            w.zm = w.zp = 0u;
             if (DIMS == 3) {
                 w.zm = __ldg(other + ((((z - 1u) & (L - 1u)) * L + y) * nq + q));
                 w.zp = __ldg(other + ((((z + 1u) & (L - 1u)) * L + y) * nq + q));
-            } else {
-                w.zm = w.zp = 0u;
             }
-            w.s = own[row + q];
-        };
-        // a warp's items are consecutive and items is a multiple of 32 here
-        uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-        if (g < items) {
-            Words cur;
-            load(g, cur);
-            for (;;) {
-                const uint32_t gn = g + stride;
-                const bool more = gn < items;
-                Words nxt = cur;
-                if (more) load(gn, nxt);
-                const uint32_t r = g >> nq_shift, q = g & (nq - 1u);
-                const uint32_t z = DIMS == 3 ? r >> l_shift : 0u, y = r & (L - 1u);
-                const int p = (a.c + (int)y + (int)z) & 1;
-                // bit b <- neighbour xh - 1 (p = 0) or xh + 1 (p = 1)
-                const uint32_t sh = p == 0 ? __funnelshift_l(cur.x, cur.o, 1)
-                                           : __funnelshift_r(cur.o, cur.x, 1);
-                packed_update<DIMS, MEASURE, RULE, kDrawAligned>(
-                    a, true, true, own + r * nq + q, cur.s, cur.o, sh, cur.ym, cur.yp, cur.zm, cur.zp,
-                    0xFFFFFFFFu, 32u, r * W + 32u * q, e_acc, m_acc);
-                if (!more) break;
-                cur = nxt;
-                g = gn;
-            }
+            w.s = static_cast<const uint32_t*>(a.own)[w.at];
+            w.valid = 0xFFFFFFFFu;
+            w.hbase = pl.hbase;
+            w.edge = 0u;
+            w.mine = true;
+            return w;
         }
+    };
+    int e_acc = 0, m_acc = 0;
+    uint32_t first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * step;
+    launch_dependents();
+    if (first < items) {
+        uint32_t A[kThresholds<DIMS, RULE>];
+        PackedPlace pl = place(first);
+        packed_draws<DIMS, RULE, draw>(pl.hbase, both, a, (uint32_t)a.c, A);
+#pragma unroll
+        for (uint32_t& v : A) pin_here(v);
+        grid_dependency_wait();
+        PackedWord w = load(pl);
+        for (;;) {
+            __syncwarp();
+            packed_update<DIMS, MEASURE, RULE, draw>(a, w, A, both, e_acc, m_acc);
+            first += stride;
+            if (first >= items) break;
+            pl = place(first);
+            w = load(pl);
+            packed_draws<DIMS, RULE, draw>(pl.hbase, both, a, (uint32_t)a.c, A);
+        }
+    } else {
+        grid_dependency_wait();
     }
     if (MEASURE) block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
 }

@@ -118,10 +118,14 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
                 sh.w = __funnelshift_r(oc.w, next_x, 8);
             }
             const uint32_t g0 = ((uint32_t)r * nv + (uint32_t)v) * 4u;  // Philox group of word 0
-            const uint4 s = update_vec<DIMS, MEASURE, RULE>(sc, oc, sh, om, op, zm, zp, g0, a,
+            uint32_t cnt[4];
+            vec_counts<DIMS, RULE>(g0, a, (uint32_t)a.c, cnt);
+            const uint4 s = update_vec<DIMS, MEASURE, RULE>(sc, oc, sh, om, op, zm, zp, g0, cnt,
+                                                            make_uint4(~0u, ~0u, ~0u, ~0u), a,
                                                             e_acc, m_acc);
             Sv[(uint32_t)r * nv] = s;
             ++n_rows;
+
         }
         // slide the window
         if (pf) {
@@ -152,7 +156,7 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
 // General kernel: any even L.  One item = one 16-byte vector of the colour
 // array (16 consecutive half indices, four Philox groups); see int8_vec().
 template <int DIMS, bool MEASURE, int RULE>
-__global__ void __launch_bounds__(256) pass_int8_vecs(PassArgs a, WordGeom g) {
+__global__ void __launch_bounds__(256, DIMS == 2 ? 3 : 2) pass_int8_vecs(PassArgs a, WordGeom g) {
     const uint32_t vecs = (g.half + 15u) >> 4;
     const uint32_t stride = gridDim.x * blockDim.x;
     int e_acc = 0, m_acc = 0;
@@ -227,11 +231,7 @@ cudaError_t launch_pass_t(const PassArgs& a0, int64_t half_sites, bool vec, cons
         const int64_t cap = (int64_t)dp.sm_count * 8;
         if (blocks > cap) blocks = cap;
         if (blocks < 1) blocks = 1;
-        WordGeom g;
-        g.W = (uint32_t)a0.W;
-        g.L = (uint32_t)a0.L;
-        g.rows = (uint32_t)a0.rows;
-        g.half = (uint32_t)half_sites;
+        const WordGeom g((uint32_t)a0.W, (uint32_t)a0.L, (uint32_t)a0.rows);
         return launch_chained(pass_int8_vecs<DIMS, MEASURE, RULE>, (unsigned)blocks,
                               (unsigned)threads, 0, st, a0, g);
     }

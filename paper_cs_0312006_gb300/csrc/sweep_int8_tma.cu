@@ -182,7 +182,7 @@ struct PairUpdate {
                 X |= uw[j] < t ? (0xFFu << (8 * j)) : 0u;
             }
         } else {
-            X = flip_mask<DIMS, RULE>(D[w], u, a);
+            X = flip_mask(D[w], count_word<DIMS, RULE>(u, a));
         }
         const uint32_t out = sv[w] ^ (X & kByteFlip);
         if (MEASURE) {
@@ -460,8 +460,12 @@ __global__ void __launch_bounds__(128, WALK == kWalkOne ? 6 : 4) pass_int8_tma(P
                 }
                 const uint32_t row = (z * (uint32_t)a.L + y) * nv + v;  // global vector index
                 int e_vec = 0;
+                uint32_t cnt[4];
+                vec_counts<DIMS, RULE>(row * 4u, a, (uint32_t)a.c, cnt);
                 own_g[row] = update_vec<DIMS, MEASURE, RULE>(own_s[i * nv + v], oc, sh, om, op,
-                                                             zm, zp, row * 4u, a, e_vec, m_acc);
+                                                             zm, zp, row * 4u, cnt,
+                                                             make_uint4(~0u, ~0u, ~0u, ~0u), a,
+                                                             e_vec, m_acc);
                 e_acc += e_vec;
                 ++n_vec;
             }
