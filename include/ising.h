@@ -53,7 +53,8 @@ enum {
 /* Kernels for the int8 colour pass (same results; see ising_set_kernel). */
 enum {
     ISING_KERNEL_AUTO = 0,  /* a registered configuration (ising_set_int8_config), else staged
-                               for 2D with 4096 <= L <= 16384 and strip otherwise (measured) */
+                               for 2D with 4096 <= L <= 16384 and for 3D with L / 32 a power of
+                               two from L = 256 on, and strip otherwise (measured) */
     ISING_KERNEL_STRIP = 1, /* per-thread row strips, neighbour rows in registers */
     ISING_KERNEL_TMA = 2    /* tiles staged in shared memory by bulk (TMA) copies */
 };
@@ -291,7 +292,8 @@ typedef struct ising_int8_config {
 int ising_set_int8_config(int dims, int L_min, int L_max, const ising_int8_config *cfg);
 
 /* Drop every registered configuration (ISING_KERNEL_AUTO returns to the
- * built-in choice: the staged kernel for 2D 4096 <= L <= 16384). */
+ * built-in choice: the staged kernel for 2D 4096 <= L <= 16384 and 3D L = 256,
+ * 512, 1024). */
 int ising_clear_int8_configs(void);
 
 /* The configuration the lattice's int8 passes run now (registered or

@@ -137,7 +137,7 @@ __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom
     }
     const uint32_t D = disagreements<DIMS>(s, nx, nxs, nym, nyp, nzm, nzp);
     const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-    const uint32_t X = flip_mask(D, count_word<DIMS, RULE>(u, a));
+    const uint32_t X = flip_mask<DIMS, RULE>(D, u, a);
     const uint32_t snew = s ^ (X & kByteFlip);
     own[w] = snew;
     if (MEASURE) {

@@ -61,10 +61,11 @@ __device__ __forceinline__ uint32_t downhill_mask(uint32_t D) {
 // takes one instruction in two cycles, and adds (and the byte sums of E and M)
 // need not go there.
 template <int DIMS, int RULE>
-__device__ __forceinline__ uint32_t count_word(const Philox4& u, const PassArgs& a) {
+__device__ __forceinline__ uint32_t count_word(const Philox4& u, const PassArgs& a,
+                                               uint32_t D = 0u) {
     constexpr int N = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
     constexpr uint32_t need = RULE == kRuleHeatBath ? 2u * DIMS + 1u : (uint32_t)DIMS;
-    uint32_t acc = (0x80u - 2u * need) * kByteOnes;
+    uint32_t acc = D + (0x80u - 2u * need) * kByteOnes;
     static_for<4>([&](auto site) {
         constexpr int j = decltype(site)::value;
         const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
@@ -75,6 +76,11 @@ __device__ __forceinline__ uint32_t count_word(const Philox4& u, const PassArgs&
 }
 __device__ __forceinline__ uint32_t flip_mask(uint32_t D, uint32_t count) {
     return byte_signs(D + count);
+}
+// Both where D is known by then (an add less).
+template <int DIMS, int RULE>
+__device__ __forceinline__ uint32_t flip_mask(uint32_t D, const Philox4& u, const PassArgs& a) {
+    return byte_signs(count_word<DIMS, RULE>(u, a, D));
 }
 
 // Sum of a word's four spins (bytes +1 / -1) or counts, added to acc.
@@ -106,7 +112,7 @@ __device__ __forceinline__ uint32_t multihit_word(uint32_t D, uint32_t group, co
         if (X != 0xFFFFFFFFu) {
             const Philox4 u = philox4x32_10(group, a.t, (uint32_t)a.c + 2u * (uint32_t)m,
                                             kTagSweep, a.key0, a.key1);
-            X = flip_mask(D, count_word<DIMS, kRuleMetropolis>(u, a));
+            X = flip_mask<DIMS, kRuleMetropolis>(D, u, a);
         }
         D = (D & ~X) | ((q2 - D) & X);
         net ^= X;
@@ -208,7 +214,7 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
             X = multihit_word<DIMS>(D, w, a);
         } else {
             const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
-            X = flip_mask(D, count_word<DIMS, RULE>(u, a));
+            X = flip_mask<DIMS, RULE>(D, u, a);
         }
         const uint32_t snew = s ^ (X & kByteFlip);
         own[w] = snew;
@@ -340,27 +346,31 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
     }
 }
 
-// The tests (count_word) of the four Philox groups g0 .. g0 + 3: one 16-byte
-// vector.
-template <int DIMS, int RULE>
-__device__ __forceinline__ void vec_counts(uint32_t g0, const PassArgs& a, uint32_t c2,
-                                           uint32_t (&cnt)[4]) {
-    PhiloxRuns<1> ps;
+// The draws of the four Philox groups g0 .. g0 + 3 (one 16-byte vector) ...
+__device__ __forceinline__ void vec_draws(uint32_t g0, const PassArgs& a, uint32_t c2,
+                                          PhiloxRuns<1>& ps) {
     const uint32_t base[1] = {g0};
     ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
 #pragma unroll
     for (int r = 1; r < 10; ++r) ps.next_round();
+}
+// ... and their tests (count_word).
+template <int DIMS, int RULE>
+__device__ __forceinline__ void vec_counts(uint32_t g0, const PassArgs& a, uint32_t c2,
+                                           uint32_t (&cnt)[4]) {
+    PhiloxRuns<1> ps;
+    vec_draws(g0, a, c2, ps);
 #pragma unroll
     for (int w = 0; w < 4; ++w) cnt[w] = count_word<DIMS, RULE>(ps.result(w), a);
 }
 
-// Update the 16 sites of one 16-byte vector (Philox groups g0..g0+3), given its
-// tests (of the first trial).  Accumulates the sum of the new spins (m_sum) and,
+// Update the 16 sites of one 16-byte vector (Philox groups g0..g0+3); flips(w, D)
+// is the flip mask of word w in the first trial.  Accumulates the sum of the new spins (m_sum) and,
 // in the white pass, sum_j 2*d_new_j (e_acc), over the bytes set in `counted`.
-template <int DIMS, bool MEASURE, int RULE>
+template <int DIMS, bool MEASURE, int RULE, typename F>
 __device__ __forceinline__ uint4 update_vec(const uint4& s, const uint4& x, const uint4& xs,
                                             const uint4& ym, const uint4& yp, const uint4& zm,
-                                            const uint4& zp, uint32_t g0, uint32_t (&cnt)[4],
+                                            const uint4& zp, uint32_t g0, F&& flips,
                                             const uint4& counted, const PassArgs& a, int& e_acc,
                                             int& m_sum) {
     const uint32_t cv[4] = {counted.x, counted.y, counted.z, counted.w};
@@ -372,22 +382,26 @@ __device__ __forceinline__ uint4 update_vec(const uint4& s, const uint4& x, cons
     D[3] = disagreements<DIMS>(s.w, x.w, xs.w, ym.w, yp.w, zm.w, zp.w);
     // one trial, or a.hits in a row with the neighbours fixed
     const int hits = RULE == kRuleMultiHit ? a.hits : 1;
-    uint32_t Dc[4] = {D[0], D[1], D[2], D[3]};
+    uint32_t Dc[4];
 #pragma unroll
-    for (int w = 0; w < 4; ++w) X[w] = 0u;
+    for (int w = 0; w < 4; ++w) {
+        X[w] = flips(w, D[w]);
+        constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
+        if (RULE == kRuleMultiHit) Dc[w] = (D[w] & ~X[w]) | ((q2 - D[w]) & X[w]);
+    }
+    if (RULE == kRuleMultiHit) {
 #pragma unroll 1
-    for (int m = 0;;) {
+        for (int m = 1; m < hits; ++m) {
+            uint32_t cnt[4];
+            vec_counts<DIMS, RULE>(g0, a, (uint32_t)a.c + 2u * (uint32_t)m, cnt);
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            const uint32_t Y = flip_mask(Dc[w], cnt[w]);
-            if (RULE == kRuleMultiHit) {
+            for (int w = 0; w < 4; ++w) {
                 constexpr uint32_t q2 = 4u * DIMS * kByteOnes;
+                const uint32_t Y = flip_mask(Dc[w], cnt[w]);
                 Dc[w] = (Dc[w] & ~Y) | ((q2 - Dc[w]) & Y);
+                X[w] ^= Y;
             }
-            X[w] ^= Y;
         }
-        if (++m >= hits) break;
-        vec_counts<DIMS, RULE>(g0, a, (uint32_t)a.c + 2u * (uint32_t)m, cnt);
     }
     uint32_t out[4];
 #pragma unroll
@@ -573,8 +587,9 @@ __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, u
         n_sites = (int)left;
     }
     int e_vec = 0;
-    own16[v] = update_vec<DIMS, MEASURE, RULE>(s, nx, nxs, nym, nyp, nzm, nzp, 4u * v, cnt, counted,
-                                               a, e_vec, m_sum);
+    auto flips = [&](int w, uint32_t D) { return flip_mask(D, cnt[w]); };
+    own16[v] = update_vec<DIMS, MEASURE, RULE>(s, nx, nxs, nym, nyp, nzm, nzp, 4u * v, flips,
+                                               counted, a, e_vec, m_sum);
     if (MEASURE && a.c == 1) e_acc += e_vec - n_sites * 2 * DIMS;
 }
 

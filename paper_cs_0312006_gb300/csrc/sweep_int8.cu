@@ -118,9 +118,12 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
                 sh.w = __funnelshift_r(oc.w, next_x, 8);
             }
             const uint32_t g0 = ((uint32_t)r * nv + (uint32_t)v) * 4u;  // Philox group of word 0
-            uint32_t cnt[4];
-            vec_counts<DIMS, RULE>(g0, a, (uint32_t)a.c, cnt);
-            const uint4 s = update_vec<DIMS, MEASURE, RULE>(sc, oc, sh, om, op, zm, zp, g0, cnt,
+            PhiloxRuns<1> ps;
+            vec_draws(g0, a, (uint32_t)a.c, ps);
+            auto flips = [&](int w, uint32_t D) {
+                return flip_mask<DIMS, RULE>(D, ps.result(w), a);
+            };
+            const uint4 s = update_vec<DIMS, MEASURE, RULE>(sc, oc, sh, om, op, zm, zp, g0, flips,
                                                             make_uint4(~0u, ~0u, ~0u, ~0u), a,
                                                             e_acc, m_acc);
             Sv[(uint32_t)r * nv] = s;

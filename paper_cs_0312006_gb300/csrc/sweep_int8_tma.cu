@@ -39,11 +39,13 @@ constexpr int kStages = 2;
 
 // Rows per tile: about 8 KiB of own-colour rows (two rows of a 2D L = 8192
 // lattice, which measured best there against 1, 4 and 8), at least 2 and at
-// most 64 rows, a power of two that divides L.
-__host__ __device__ inline int tile_rows(int L) {
+// most 64 rows, a power of two that divides L.  In 3D a tile of half that where
+// it comes out even: 32 rows of L = 256 are one (row pair, column) item for each
+// of 128 threads (10.9 us a pass against 11.8 with 64 rows).
+__host__ __device__ inline int tile_rows(int dims, int L) {
     const int W = L / 2;
     int R = 2;
-    while (R < 64 && 2 * R * W <= 8192 && L % (2 * R) == 0) R *= 2;
+    while (R < 64 && 2 * R * W <= (dims == 3 ? 8191 : 8192) && L % (2 * R) == 0) R *= 2;
     while (R > 1 && L % R != 0) R >>= 1;
     return R;
 }
@@ -182,7 +184,7 @@ struct PairUpdate {
                 X |= uw[j] < t ? (0xFFu << (8 * j)) : 0u;
             }
         } else {
-            X = flip_mask(D[w], count_word<DIMS, RULE>(u, a));
+            X = flip_mask<DIMS, RULE>(D[w], u, a);
         }
         const uint32_t out = sv[w] ^ (X & kByteFlip);
         if (MEASURE) {
@@ -460,10 +462,13 @@ __global__ void __launch_bounds__(128, WALK == kWalkOne ? 6 : 4) pass_int8_tma(P
                 }
                 const uint32_t row = (z * (uint32_t)a.L + y) * nv + v;  // global vector index
                 int e_vec = 0;
-                uint32_t cnt[4];
-                vec_counts<DIMS, RULE>(row * 4u, a, (uint32_t)a.c, cnt);
+                PhiloxRuns<1> ps;
+                vec_draws(row * 4u, a, (uint32_t)a.c, ps);
+                auto flips = [&](int w, uint32_t D) {
+                    return flip_mask<DIMS, RULE>(D, ps.result(w), a);
+                };
                 own_g[row] = update_vec<DIMS, MEASURE, RULE>(own_s[i * nv + v], oc, sh, om, op,
-                                                             zm, zp, row * 4u, cnt,
+                                                             zm, zp, row * 4u, flips,
                                                              make_uint4(~0u, ~0u, ~0u, ~0u), a,
                                                              e_vec, m_acc);
                 e_acc += e_vec;
@@ -492,7 +497,7 @@ cudaError_t launch_tma_t(const PassArgs& a, const DeviceProps& dp, int* err, uin
     // default: tile_rows() (2D L = 8192: two rows, measured best against 1, 4
     // and 8) and 128 threads, each taking its (row pair, column) items two at
     // a time; a tuned configuration may ask for other rows per tile
-    const int R = rows_per_tile > 0 ? rows_per_tile : tile_rows(a.L);
+    const int R = rows_per_tile > 0 ? rows_per_tile : tile_rows(DIMS, a.L);
     const int threads = 128;  // two items per thread per 2-row tile at L = 8192
     tg.R = R;
     tg.bands = a.L / R;
@@ -531,7 +536,7 @@ cudaError_t launch_tma_t(const PassArgs& a, const DeviceProps& dp, int* err, uin
 bool int8_tma_ok(int dims, int L, int rows_per_tile) {
     const int W = L / 2;
     if (W % 16 != 0) return false;
-    const int R = rows_per_tile > 0 ? rows_per_tile : tile_rows(L);
+    const int R = rows_per_tile > 0 ? rows_per_tile : tile_rows(dims, L);
     if (R < 1 || L % R != 0) return false;
     const size_t stage = (size_t)(2 * R + 2) * W + (dims == 3 ? 2u * R * W : 0u);
     return (size_t)kStages * stage <= 200 * 1024;
@@ -556,7 +561,7 @@ static cudaError_t int8_pass_tma_rule(const PassArgs& a, int dims, bool measure,
         return int8_pass_tma_walk<RULE, kWalkLoop>(a, dims, measure, dp, err, extra_tx, st, R,
                                                    ctas);
     } else {
-        const int rows = R > 0 ? R : tile_rows(a.L);
+        const int rows = R > 0 ? R : tile_rows(dims, a.L);
         const int items = (rows / 2) * (a.W / 16);  // (row pair, column) items per tile
         if (items == 2 * 128)                        // 128 threads per CTA
             return int8_pass_tma_walk<RULE, kWalkTwo>(a, dims, measure, dp, err, extra_tx, st, R,
@@ -569,16 +574,21 @@ static cudaError_t int8_pass_tma_rule(const PassArgs& a, int dims, bool measure,
     }
 }
 
-// Where the staged kernel measured faster than the strip kernel on GB300: 2D
-// with long rows (L >= 4096) while two CTAs' stages fit in one SM's shared
-// memory (L <= 16384: 8.38e11 against 7.76e11 site updates/s per pass at
-// L = 16384; at L = 32768 one CTA per SM gives 7.24e11 against the strip
-// kernel's 8.02e11).  With short rows (3D, small 2D) a tile holds about one
-// vector per thread and its barriers dominate.
+// Where the staged kernel measured faster than the strip kernel on GB300 (us a
+// pass, Metropolis / heat bath):
+//   2D with long rows (L >= 4096) while two CTAs' stages fit in one SM's shared
+//   memory (L <= 16384): L = 8192 31.0 / 32.4 against 38.2 / 43.8, L = 4096 10.4
+//   against 11.3; L = 3072 9.1 / 9.4 against 7.2 / 8.0.  At L = 32768 one CTA per
+//   SM measured 10 % slower than the strips.
+//   3D from L = 256 where the default tile is one item for every thread (W / 16
+//   a power of two): L = 256 10.9 / 11.2 against 13.0 / 15.2, L = 512 71.6 / 74.3
+//   against 95.7 / 111.  Elsewhere some threads of a tile idle: L = 320 25.4
+//   against 24.0, L = 288 20.5 against 17.9, L = 384 40.3 against 38.2.
 bool int8_tma_preferred(int dims, int L) {
-    if (dims != 2 || L < 4096 || !int8_tma_ok(dims, L, 0)) return false;
-    const int W = L / 2, R = tile_rows(L);
-    return 2 * (size_t)kStages * (size_t)(2 * R + 2) * W <= 200 * 1024;
+    if (!int8_tma_ok(dims, L, 0)) return false;
+    const int W = L / 2, R = tile_rows(dims, L), nv = W / 16;
+    if (dims == 3) return L >= 256 && (nv & (nv - 1)) == 0 && R / 2 * nv == 128;
+    return L >= 4096 && 2 * (size_t)kStages * (size_t)(2 * R + 2) * W <= 200 * 1024;
 }
 
 cudaError_t int8_pass_tma(const PassArgs& a, int dims, bool measure, int rule,
