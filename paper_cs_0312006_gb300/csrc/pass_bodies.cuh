@@ -773,12 +773,15 @@ __device__ __forceinline__ uint32_t x_neighbours(const PackedWord& w) {
     return ((w.o >> 1) & ~top) | ((w.x & 1u) ? top : 0u);
 }
 
-// The rule applied to one packed word, given its tests, then the store and the
-// word's share of E and M.  With ragged draws the whole warp takes part.
+// The rule applied to one packed word, given its tests (of the first trial; in
+// `later`, if set, those of trials 1 .. n_later, one word a thread of the block
+// per trial and threshold), then the store and the word's share of E and M.  With
+// ragged draws the whole warp takes part.
 template <int DIMS, bool MEASURE, int RULE, int DRAW>
 __device__ __forceinline__ void packed_update(const PassArgs& a, const PackedWord& w,
                                               uint32_t (&A)[kThresholds<DIMS, RULE>], bool both,
-                                              int& e_acc, int& m_acc) {
+                                              int& e_acc, int& m_acc,
+                                              const uint32_t* later = nullptr, int n_later = 0) {
     const uint32_t s = w.s, sh = x_neighbours(w);
     uint32_t flip;
     if constexpr (RULE == kRuleHeatBath) {
@@ -800,6 +803,12 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, const PackedWor
             }
             cur ^= k.always | choose_answer<DIMS>(k, A);
             if (++m >= hits) break;
+            if (RULE == kRuleMultiHit && m <= n_later) {
+#pragma unroll
+                for (int n = 0; n < kThresholds<DIMS, RULE>; ++n)
+                    A[n] = later[((m - 1) * kThresholds<DIMS, RULE> + n) * (int)blockDim.x];
+                continue;
+            }
             packed_draws<DIMS, RULE, DRAW>(w.hbase, both, a, (uint32_t)a.c + 2u * (uint32_t)m, A);
         }
         flip = cur ^ s;

@@ -46,6 +46,11 @@ namespace {
 // gained nothing by it: 2D L = 500 2.75 -> 2.77, L = 1000 2.75 -> 3.64.)
 constexpr int kWordsFull = 0, kWordsAligned = 1, kWordsRagged = 2;
 
+// Multi-hit: the first item's later trials drawn ahead too, up to this many, kept
+// in shared memory (three hits, us a pass: 2D L = 512 3.6 -> 2.1, L = 2048 7.6 ->
+// 5.4, L = 8192 66 either way).
+constexpr int kLaterTrials = 3;
+
 template <int DIMS, bool MEASURE, int RULE, int WORDS>
 __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geom,
                                                       uint32_t nq_shift, uint32_t l_shift) {
@@ -106,12 +111,28 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
         packed_draws<DIMS, RULE, draw>(pl.hbase, both, a, (uint32_t)a.c, A);
 #pragma unroll
         for (uint32_t& v : A) pin_here(v);
+        constexpr int N = kThresholds<DIMS, RULE>;
+        __shared__ uint32_t s_later[RULE == kRuleMultiHit ? kLaterTrials * N * 256 : 1];
+        uint32_t* later = s_later + (RULE == kRuleMultiHit ? threadIdx.x : 0u);
+        int n_later = 0;
+        if constexpr (RULE == kRuleMultiHit) {
+            n_later = a.hits - 1 < kLaterTrials ? a.hits - 1 : kLaterTrials;
+#pragma unroll 1
+            for (int m = 0; m < n_later; ++m) {
+                uint32_t B[N];
+                packed_draws<DIMS, RULE, draw>(pl.hbase, both, a,
+                                               (uint32_t)a.c + 2u * (uint32_t)(m + 1), B);
+#pragma unroll
+                for (int n = 0; n < N; ++n) later[(m * N + n) * 256] = B[n];
+            }
+        }
         grid_dependency_wait();
         PackedWord w = load(pl);
         for (;;) {
             __syncwarp();
-            packed_update<DIMS, MEASURE, RULE, draw>(a, w, A, both, e_acc, m_acc);
+            packed_update<DIMS, MEASURE, RULE, draw>(a, w, A, both, e_acc, m_acc, later, n_later);
             first += stride;
+            n_later = 0;
             if (first >= items) break;
             pl = place(first);
             w = load(pl);
