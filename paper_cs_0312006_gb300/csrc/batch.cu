@@ -9,15 +9,14 @@
 // colour pass of all of them) and the small ones the persistent kernel, a CTA
 // each; with a cluster size given, all go through the persistent kernel.
 //
-// Work queue of the persistent kernel: one job per lattice, holding everything its sweeps need (spin
-// arrays, thresholds, key, first sweep index, sweep count, measurement
-// interval, record slots).  Jobs are ordered by work (sites x sweeps),
-// largest first, and split in two queues at a size threshold:
+// Work queue of the persistent kernel: one job per lattice, holding everything
+// its sweeps need (spin arrays, thresholds, key, first sweep index, sweep
+// count, measurement interval, record slots).  Jobs are ordered by work
+// (sites x sweeps), largest first, and split in two queues at a size threshold:
 //   - large jobs are run by a thread-block cluster: the CTAs of the cluster
 //     share the job's words, and consecutive colour passes are separated by
-//     the hardware cluster barrier (release/acquire at cluster scope), with
-//     the other colour read through L2 so that words written by another CTA
-//     of the cluster are seen;
+//     the hardware cluster barrier (release/acquire at cluster scope), which
+//     also makes the words another CTA of the cluster wrote visible;
 //   - small jobs are run by one CTA each, passes separated by __syncthreads.
 // Each cluster (then each CTA) takes the next job with one atomicAdd on a
 // queue counter and runs all of the job's sweeps before taking another, so

@@ -1,7 +1,8 @@
 // engine.cu -- host side of the C ABI declared in include/ising.h: lattice
 // handles, acceptance thresholds, the per-sweep launch sequence and the E/M
 // record buffer.  All simulation arithmetic runs in the kernels of
-// sweep_int8.cu / sweep_bitpack.cu.
+// sweep_int8.cu / sweep_int8_tma.cu / sweep_bitpack.cu / sweep_demon.cu, and of
+// resident.cu for runs of sweeps of small lattices.
 #include <cmath>
 #include <cstdlib>
 #include <cstring>

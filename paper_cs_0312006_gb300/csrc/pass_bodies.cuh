@@ -1,8 +1,10 @@
-// pass_bodies.cuh -- per-word bodies of a colour pass, shared by the
-// per-lattice kernels (sweep_int8.cu, sweep_bitpack.cu) and the batched
-// persistent kernel (batch.cu).
+// pass_bodies.cuh -- per-word and per-vector bodies of a colour pass, shared by
+// the per-lattice kernels (sweep_int8.cu, sweep_int8_tma.cu, sweep_bitpack.cu),
+// the small lattices' cluster kernel (resident.cu) and the batched kernels
+// (batch.cu).
 //
-// The int8 body works for any even L: a word of the colour array holds the
+// The int8 word body (int8_word, rows of less than a 16-site vector; longer rows
+// take int8_vec) works for any even L: a word of the colour array holds the
 // four half indices h = 4w..4w+3 (one Philox group), whatever rows they fall
 // in.  A word that lies inside one half row, away from the x-wrap and from
 // the first and last row (and plane) of the lattice, takes the byte-sliced
@@ -29,13 +31,10 @@ constexpr uint32_t kByteBit7 = 0x80808080u;
 constexpr uint32_t kByteOnes = 0x01010101u;
 
 // Load modes for the other colour: 1 = read-only path (ld.global.nc, only when
-// nothing writes the array during the kernel), 2 = L2 only (ld.global.cg, for
-// data written by other CTAs of a cluster earlier in the same kernel), 0 = a
-// plain coherent load.
+// nothing writes the array during the kernel), 0 = a plain coherent load.
 template <int NC, typename T>
 __device__ __forceinline__ T load_other(const T* p) {
     if (NC == 1) return __ldg(p);
-    if (NC == 2) return __ldcg(p);
     return *p;
 }
 

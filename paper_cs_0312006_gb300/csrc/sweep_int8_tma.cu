@@ -21,6 +21,11 @@
 // tile's copies land, the second item's round by round between the first
 // item's word updates.
 //
+// Bound by instruction issue: 2D L = 8192 31.0 us a pass in the default shape
+// (33.5 before the threshold tests became a compare and a predicated add each and
+// E and M byte dot products; 17.0 is the generator alone).  The rates beside the
+// single choices below are those of the day each was made, both sides alike.
+//
 // Waits on an mbarrier are bounded: if a phase does not complete within the
 // limit the kernel raises the error flag, waits (bounded again) for its own
 // copies still in flight, and returns; the host reports ISING_ETIMEOUT.
@@ -213,7 +218,7 @@ struct PairUpdate {
 // kWalkLoop otherwise.  The first two instances hold no loop over items and no
 // guard, which keeps them clear of the register cap; the one-item instance
 // runs six CTAs per SM (at most 85 registers; 3D L = 256 with 32-row tiles:
-// 6.7e11 at four, 7.0e11 at five, 7.2e11 site updates/s at six).
+// 6.7e11 at four, 7.0e11 at five, 7.2e11 site updates/s at six; 7.7e11 since).
 constexpr int kWalkLoop = 0, kWalkTwo = 1, kWalkOne = 2;
 
 template <int DIMS, bool MEASURE, int RULE, int WALK>
