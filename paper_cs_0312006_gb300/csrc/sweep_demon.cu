@@ -326,13 +326,22 @@ __device__ __forceinline__ void demon_packed_measure(uint32_t snew, uint32_t o, 
     }
 }
 
-// Rows of whole 16-byte groups (W % 128 == 0): four consecutive words per
-// item, every stream read and written as 16-byte vectors.
-template <int DIMS, bool MEASURE>
-__global__ void __launch_bounds__(256) pass_demon_packed4(PassArgs a) {
+constexpr int kPacked4Threads = 128;
+
+// Rows of whole 16-byte groups (W % 128 == 0): four consecutive words of ROWS
+// consecutive rows per item, every stream read and written as 16-byte vectors.
+// Bound by L2 and latency up to L = 16384, by HBM above.  Two rows (2D) share two
+// of their three rows of the other colour and put ten loads in flight instead of
+// six: L = 8192 4.8 -> 4.3 us a pass (with 256-thread CTAs of one row 1.7 waves,
+// now one of 72 registers a thread).  128-thread CTAs let the next pass's start
+// sooner: L = 2048 2.3 -> 2.0, L = 4096 2.8 -> 2.5, 3D L = 512 10.2 -> 9.1 us.
+template <int DIMS, bool MEASURE, int ROWS>
+__global__ void __launch_bounds__(kPacked4Threads, DIMS == 3 ? 6 : ROWS == 2 ? 7 : 8)
+    pass_demon_packed4(PassArgs a) {
+    static_assert(DIMS == 2 || ROWS == 1, "planes are walked a row at a time");
     const uint32_t W = (uint32_t)a.W, L = (uint32_t)a.L, rows = (uint32_t)a.rows;
     const uint32_t nq = W >> 5, n4 = nq >> 2;
-    const uint32_t items = rows * n4, words = rows * nq;
+    const uint32_t items = rows / ROWS * n4, words = rows * nq;
     uint4* own = static_cast<uint4*>(a.own);
     const uint4* other = static_cast<const uint4*>(a.other);
     const uint32_t* other_w = static_cast<const uint32_t*>(a.other);
@@ -343,60 +352,70 @@ __global__ void __launch_bounds__(256) pass_demon_packed4(PassArgs a) {
     grid_dependency_wait();
     launch_dependents();
     for (uint32_t item = blockIdx.x * blockDim.x + threadIdx.x; item < items; item += stride) {
-        const uint32_t r = item / n4, g = item - r * n4;
+        const uint32_t pair = item / n4, g = item - pair * n4, r = pair * ROWS;
         uint32_t y = r, z = 0u;
         if (DIMS == 3) {
             z = r / L;
             y = r - z * L;
         }
         const uint32_t plane = z * L;
-        const uint4 o = __ldg(other + r * n4 + g);
-        const uint4 oym = __ldg(other + (plane + (y == 0u ? L - 1u : y - 1u)) * n4 + g);
-        const uint4 oyp = __ldg(other + (plane + (y + 1u == L ? 0u : y + 1u)) * n4 + g);
+        uint4 o[ROWS + 2];  // the other colour's rows y - 1 .. y + ROWS
+        o[0] = __ldg(other + (plane + (y == 0u ? L - 1u : y - 1u)) * n4 + g);
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) o[i + 1] = __ldg(other + (r + i) * n4 + g);
+        o[ROWS + 1] = __ldg(other + (plane + (y + ROWS == L ? 0u : y + ROWS)) * n4 + g);
         uint4 ozm = make_uint4(0u, 0u, 0u, 0u), ozp = ozm;
         if (DIMS == 3) {
             ozm = __ldg(other + ((z == 0u ? L - 1u : z - 1u) * L + y) * n4 + g);
             ozp = __ldg(other + ((z + 1u == L ? 0u : z + 1u) * L + y) * n4 + g);
         }
-        const uint4 sv = own[r * n4 + g];
-        const uint32_t rd = r >= a.rot ? r - a.rot : r + rows - a.rot;  // storage row
-        uint4 qa = Q0[rd * n4 + g], qb = Q1[rd * n4 + g];
-        const int p = (a.c + (int)y + (int)z) & 1;
-        const uint32_t row = r * nq;
-        uint4 sh;
-        if (p == 0) {  // bit b <- neighbour xh - 1; word 0 takes the previous word's bit 31
-            const uint32_t prev = g == 0u ? __ldg(other_w + row + nq - 1u)
-                                          : __ldg(other_w + row + 4u * g - 1u);
-            sh = make_uint4(__funnelshift_l(prev, o.x, 1), __funnelshift_l(o.x, o.y, 1),
-                            __funnelshift_l(o.y, o.z, 1), __funnelshift_l(o.z, o.w, 1));
-        } else {       // bit b <- neighbour xh + 1
-            const uint32_t next = g + 1u == n4 ? __ldg(other_w + row) : __ldg(other_w + row + 4u * g + 4u);
-            sh = make_uint4(__funnelshift_r(o.x, o.y, 1), __funnelshift_r(o.y, o.z, 1),
-                            __funnelshift_r(o.z, o.w, 1), __funnelshift_r(o.w, next, 1));
+        uint4 sv[ROWS], qa[ROWS], qb[ROWS];
+        uint32_t rd[ROWS], edge[ROWS];  // storage row; the word beside the group
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            sv[i] = own[(r + i) * n4 + g];
+            rd[i] = r + i >= a.rot ? r + i - a.rot : r + i + rows - a.rot;
+            qa[i] = Q0[rd[i] * n4 + g];
+            qb[i] = Q1[rd[i] * n4 + g];
+            const uint32_t* row = other_w + (r + i) * nq;
+            edge[i] = (a.c + (int)y + i + (int)z) & 1
+                          ? __ldg(row + (g + 1u == n4 ? 0u : 4u * g + 4u))
+                          : __ldg(row + (g == 0u ? nq : 4u * g) - 1u);
         }
-        const uint32_t fx = demon_packed_bits<DIMS>(sv.x, o.x, sh.x, oym.x, oyp.x, ozm.x, ozp.x,
-                                                    0xFFFFFFFFu, qa.x, qb.x);
-        const uint32_t fy = demon_packed_bits<DIMS>(sv.y, o.y, sh.y, oym.y, oyp.y, ozm.y, ozp.y,
-                                                    0xFFFFFFFFu, qa.y, qb.y);
-        const uint32_t fz = demon_packed_bits<DIMS>(sv.z, o.z, sh.z, oym.z, oyp.z, ozm.z, ozp.z,
-                                                    0xFFFFFFFFu, qa.z, qb.z);
-        const uint32_t fw = demon_packed_bits<DIMS>(sv.w, o.w, sh.w, oym.w, oyp.w, ozm.w, ozp.w,
-                                                    0xFFFFFFFFu, qa.w, qb.w);
-        const uint4 sn = make_uint4(sv.x ^ fx, sv.y ^ fy, sv.z ^ fz, sv.w ^ fw);
-        own[r * n4 + g] = sn;
-        if (fx | fy | fz | fw) {
-            Q0[rd * n4 + g] = qa;
-            Q1[rd * n4 + g] = qb;
-        }
-        if (MEASURE) {
-            demon_packed_measure<DIMS>(sn.x, o.x, sh.x, oym.x, oyp.x, ozm.x, ozp.x, 0xFFFFFFFFu,
-                                       32u, a.c, e_acc, m_acc);
-            demon_packed_measure<DIMS>(sn.y, o.y, sh.y, oym.y, oyp.y, ozm.y, ozp.y, 0xFFFFFFFFu,
-                                       32u, a.c, e_acc, m_acc);
-            demon_packed_measure<DIMS>(sn.z, o.z, sh.z, oym.z, oyp.z, ozm.z, ozp.z, 0xFFFFFFFFu,
-                                       32u, a.c, e_acc, m_acc);
-            demon_packed_measure<DIMS>(sn.w, o.w, sh.w, oym.w, oyp.w, ozm.w, ozp.w, 0xFFFFFFFFu,
-                                       32u, a.c, e_acc, m_acc);
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const uint4 m = o[i], n = o[i + 1], q = o[i + 2];
+            uint4 sh;
+            if (((a.c + (int)y + i + (int)z) & 1) == 0)  // bit b <- neighbour xh - 1
+                sh = make_uint4(__funnelshift_l(edge[i], n.x, 1), __funnelshift_l(n.x, n.y, 1),
+                                __funnelshift_l(n.y, n.z, 1), __funnelshift_l(n.z, n.w, 1));
+            else                                         // bit b <- neighbour xh + 1
+                sh = make_uint4(__funnelshift_r(n.x, n.y, 1), __funnelshift_r(n.y, n.z, 1),
+                                __funnelshift_r(n.z, n.w, 1), __funnelshift_r(n.w, edge[i], 1));
+            const uint32_t fx = demon_packed_bits<DIMS>(sv[i].x, n.x, sh.x, m.x, q.x, ozm.x, ozp.x,
+                                                        0xFFFFFFFFu, qa[i].x, qb[i].x);
+            const uint32_t fy = demon_packed_bits<DIMS>(sv[i].y, n.y, sh.y, m.y, q.y, ozm.y, ozp.y,
+                                                        0xFFFFFFFFu, qa[i].y, qb[i].y);
+            const uint32_t fz = demon_packed_bits<DIMS>(sv[i].z, n.z, sh.z, m.z, q.z, ozm.z, ozp.z,
+                                                        0xFFFFFFFFu, qa[i].z, qb[i].z);
+            const uint32_t fw = demon_packed_bits<DIMS>(sv[i].w, n.w, sh.w, m.w, q.w, ozm.w, ozp.w,
+                                                        0xFFFFFFFFu, qa[i].w, qb[i].w);
+            const uint4 sn = make_uint4(sv[i].x ^ fx, sv[i].y ^ fy, sv[i].z ^ fz, sv[i].w ^ fw);
+            own[(r + i) * n4 + g] = sn;
+            if (fx | fy | fz | fw) {
+                Q0[rd[i] * n4 + g] = qa[i];
+                Q1[rd[i] * n4 + g] = qb[i];
+            }
+            if (MEASURE) {
+                demon_packed_measure<DIMS>(sn.x, n.x, sh.x, m.x, q.x, ozm.x, ozp.x, 0xFFFFFFFFu,
+                                           32u, a.c, e_acc, m_acc);
+                demon_packed_measure<DIMS>(sn.y, n.y, sh.y, m.y, q.y, ozm.y, ozp.y, 0xFFFFFFFFu,
+                                           32u, a.c, e_acc, m_acc);
+                demon_packed_measure<DIMS>(sn.z, n.z, sh.z, m.z, q.z, ozm.z, ozp.z, 0xFFFFFFFFu,
+                                           32u, a.c, e_acc, m_acc);
+                demon_packed_measure<DIMS>(sn.w, n.w, sh.w, m.w, q.w, ozm.w, ozp.w, 0xFFFFFFFFu,
+                                           32u, a.c, e_acc, m_acc);
+            }
         }
     }
     if (MEASURE) block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
@@ -589,20 +608,34 @@ cudaError_t demon_pass(const PassArgs& a, int dims, int64_t half_sites, bool mea
 
 cudaError_t demon_packed_pass(const PassArgs& a, int dims, bool measure, const DeviceProps& dp,
                               cudaStream_t st) {
-    const bool vec = a.W % 128 == 0;
-    const int64_t items = a.rows * (int64_t)((a.W + 31) >> 5) / (vec ? 4 : 1);
+    if (a.W % 128 == 0) {
+        // Two rows an item only where that makes one wave of what would be more.
+        // Sixteen CTAs per SM with a loop, but a CTA for every 128 items where
+        // the data is out of L2 and nothing is added up at the end of a CTA: L =
+        // 32768 72.4 (256-thread CTAs, eight per SM) -> 68.3 us, 3D L = 1024 77.1
+        // -> 71.5; with E and M, or in L2, that is slower (3D L = 512 10.1
+        // against 9.1 us, 2D L = 20480 29.9 against 28.1).
+        const int64_t ctas = (int64_t)dp.sm_count * kPacked4Threads;
+        int64_t items = a.rows * (int64_t)(a.W / 128);
+        const bool pairs = dims == 2 && measure && items > 8 * ctas && items <= 2 * 7 * ctas;
+        if (pairs) items /= 2;
+        const int64_t blocks = (items + kPacked4Threads - 1) / kPacked4Threads;
+        const bool out_of_l2 = a.rows * (int64_t)(a.W / 32) * 24 > (1 << 27);
+        const int64_t cap = !measure && out_of_l2 ? 1 << 30 : (int64_t)dp.sm_count * 16;
+        const unsigned g = (unsigned)(blocks < cap ? blocks : cap);
+        constexpr unsigned n = kPacked4Threads;
+        if (pairs) return launch_chained(pass_demon_packed4<2, true, 2>, g, n, 0, st, a);
+        if (dims == 2)
+            return measure ? launch_chained(pass_demon_packed4<2, true, 1>, g, n, 0, st, a)
+                           : launch_chained(pass_demon_packed4<2, false, 1>, g, n, 0, st, a);
+        return measure ? launch_chained(pass_demon_packed4<3, true, 1>, g, n, 0, st, a)
+                       : launch_chained(pass_demon_packed4<3, false, 1>, g, n, 0, st, a);
+    }
+    const int64_t items = a.rows * (int64_t)((a.W + 31) >> 5);
     int64_t blocks = (items + 255) / 256;
     const int64_t cap = (int64_t)dp.sm_count * 8;
     if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
     const unsigned g = (unsigned)blocks;
-    if (vec) {
-        if (dims == 2)
-            return measure ? launch_chained(pass_demon_packed4<2, true>, g, 256u, 0, st, a)
-                           : launch_chained(pass_demon_packed4<2, false>, g, 256u, 0, st, a);
-        return measure ? launch_chained(pass_demon_packed4<3, true>, g, 256u, 0, st, a)
-                       : launch_chained(pass_demon_packed4<3, false>, g, 256u, 0, st, a);
-    }
     if (dims == 2)
         return measure ? launch_chained(pass_demon_packed<2, true>, g, 256u, 0, st, a)
                        : launch_chained(pass_demon_packed<2, false>, g, 256u, 0, st, a);
