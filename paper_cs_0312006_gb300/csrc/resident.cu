@@ -356,17 +356,21 @@ cudaError_t launch_resident_layout(const ResidentArgs& k, int layout, unsigned r
 // 1.65, L = 512 2.15; ragged L = 100 1.05, L = 510 3.1; 3D L = 32 0.96, L = 64
 // 2.4, ragged L = 26 1.4, L = 62 3.3.  A pass grows with the words, ragged ones
 // costing 1.6 times as much, so the line is where it meets the pass kernels': 2.7
-// us for int8 and 1.85 for packed.  The launch, the load and the store take 8 us,
-// which from two int8 sweeps and four packed ones on is less than their passes;
-// rows of less than a vector go word by word in the int8 pass kernels (8 us a
-// pass), so those always come here.
+// us for int8 and 1.85 for packed.  The launch, the load and the store take 3 to
+// 6 us, by size, which two int8 sweeps' passes outlast; packed ones, in us a call
+// of back-to-back calls (here / pass kernels): two sweeps 2D L = 16 5.2 / 7.3, L =
+// 128 6.2 / 7.2, but ragged L = 50 8.2 / 7.3 and L = 256 8.2 / 7.2; three L = 50
+// 10.3 / 10.6, L = 256 9.3 / 10.6, but L = 250 14.1 / 10.7; one sweep L = 64 6.2 /
+// 4.0 in either layout.  Rows of less than a vector go word by word in the int8
+// pass kernels (4 us a pass and more), so those always come here.
 bool resident_ok(const ising_lattice* h, int64_t n) {
     if (h->rule != ISING_RULE_METROPOLIS && h->rule != ISING_RULE_HEATBATH) return false;
     if (n > 0x7FFFFFFF) return false;
     const bool packed = h->layout == ISING_BITPACK;
     const int64_t words = h->rows * ((h->W + 3) / 4);
     const int64_t cost = h->W % 4 == 0 ? words : words * 8 / 5;
-    return cost <= (packed ? 22000 : 42000) && n >= (packed ? 4 : h->W < 16 ? 1 : 2);
+    if (!packed) return cost <= 42000 && n >= (h->W < 16 ? 1 : 2);
+    return cost <= 22000 && n >= (h->W % 4 == 0 && words <= 2048 ? 2 : cost <= 8192 ? 3 : 4);
 }
 
 cudaError_t resident_sweep(ising_lattice* h, const PassArgs& args, int64_t n, int every,
