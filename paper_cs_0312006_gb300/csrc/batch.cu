@@ -200,7 +200,7 @@ __device__ __forceinline__ void job_pass(const BatchJob& j, const PackedGeom& ge
         // spill less and stay in the instruction cache)
         constexpr uint32_t step = kWarpWords<kDrawRagged>;
         for (uint32_t first = (rank >> 5) * step; first < geom.items; first += (nthr >> 5) * step)
-            packed_words<DIMS, MEASURE, NC, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
+            packed_words<DIMS, MEASURE, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
     }
 }
 
@@ -214,7 +214,7 @@ __device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom&
         const uint32_t v = first + (threadIdx.x & 31u);
         if (16u * v < j.half) int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_acc);
     } else {
-        packed_words<DIMS, MEASURE, 1, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
+        packed_words<DIMS, MEASURE, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
     }
 }
 

@@ -192,8 +192,15 @@ __device__ __forceinline__ void static_for(F&& f) {
 // once all earlier kernels of the stream have completed and their writes are
 // visible (a pass reads the colour the previous pass wrote and writes the
 // colour it read), and it is a no-op for a kernel launched without the
-// attribute.  launch_dependents() then lets the next pass's CTAs be placed as
-// SMs free up; they in turn wait before touching memory.
+// attribute.  launch_dependents(), always behind that wait, then lets the next
+// pass's CTAs be placed as SMs free up; they in turn wait before touching memory.
+// At most two passes are on the GPU at once, the second still waiting.
+//
+// What an earlier pass wrote is read with ordinary loads.  A read-only load
+// (ld.global.nc, __ldg) is defined only for data that nothing writes during the
+// kernel's lifetime, and a chained kernel's begins before the kernel that writes
+// its input has ended: the compiler may move such a load above the wait, and an SM
+// may answer it from a copy older than the wait.
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }

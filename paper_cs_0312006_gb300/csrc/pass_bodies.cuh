@@ -856,7 +856,7 @@ __device__ __forceinline__ PackedPlace packed_place(const PackedGeom& g, uint32_
     return p;
 }
 
-template <int DIMS, int NC>
+template <int DIMS>
 __device__ __forceinline__ PackedWord packed_load(const PassArgs& a, const PackedGeom& g,
                                                   const PackedPlace& pl) {
     const uint32_t W = (uint32_t)a.W, L = (uint32_t)a.L, nq = g.words.d;
@@ -886,15 +886,15 @@ __device__ __forceinline__ PackedWord packed_load(const PassArgs& a, const Packe
     }
     const int32_t up = y == 0u ? (int32_t)((L - 1u) * nq) : -(int32_t)nq;
     const int32_t down = y + 1u == L ? -(int32_t)((L - 1u) * nq) : (int32_t)nq;
-    w.o = load_other<NC>(at);
-    w.x = load_other<NC>(at + dx);
-    w.ym = load_other<NC>(at + up);
-    w.yp = load_other<NC>(at + down);
+    w.o = *at;
+    w.x = at[dx];
+    w.ym = at[up];
+    w.yp = at[down];
     w.zm = w.zp = 0u;
     if (DIMS == 3) {
         const int32_t plane = (int32_t)(L * nq), wrap = (int32_t)((L - 1u) * L * nq);
-        w.zm = load_other<NC>(at + (z == 0u ? wrap : -plane));
-        w.zp = load_other<NC>(at + (z + 1u == L ? -wrap : plane));
+        w.zm = at[z == 0u ? wrap : -plane];
+        w.zp = at[z + 1u == L ? -wrap : plane];
     }
     w.s = static_cast<const uint32_t*>(a.own)[w.at];
     return w;
@@ -904,11 +904,11 @@ __device__ __forceinline__ PackedWord packed_load(const PassArgs& a, const Packe
 __device__ __forceinline__ bool packed_both(const PassArgs& a) { return a.W > 13; }
 
 // One step of a warp, loads first: their latency hides behind the draws.
-template <int DIMS, bool MEASURE, int NC, int RULE, int DRAW>
+template <int DIMS, bool MEASURE, int RULE, int DRAW>
 __device__ __forceinline__ void packed_words(const PassArgs& a, const PackedGeom& g,
                                              uint32_t first, int& e_acc, int& m_acc) {
     const PackedWord w =
-        packed_load<DIMS, NC>(a, g, packed_place<DRAW>(g, (uint32_t)a.W, first));
+        packed_load<DIMS>(a, g, packed_place<DRAW>(g, (uint32_t)a.W, first));
     uint32_t A[kThresholds<DIMS, RULE>];
     __syncwarp();
     packed_draws<DIMS, RULE, DRAW>(w.hbase, packed_both(a), a, (uint32_t)a.c, A);

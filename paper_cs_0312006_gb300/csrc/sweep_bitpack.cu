@@ -38,17 +38,18 @@ namespace {
 //
 // The first item's draws need only counters: they are made before the wait for
 // the previous pass, so that a pass placed on the SMs while the previous one
-// drains (or, with a lattice too small to fill the GPU, runs) has them ready.
-// Later items load first and draw while the loads are under way.
-// Per pass, in us, against waiting first: 2D L = 512 2.6 -> 1.85 (the host's
-// launches then set the pace), L = 2048 4.4 -> 2.8, L = 4096 8.4 -> 6.6, L = 8192
-// 24.4 -> 23.7; 3D L = 128 3.0 -> 2.3, L = 202 8.7 -> 6.3.  (The int8 passes
+// drains has them ready.  The next pass is let in only behind the wait: a lattice
+// that leaves SMs free would otherwise have three passes or more on the GPU at
+// once.  Later items load first and draw while the loads are under way.
+// Per pass, in us, against waiting first: 2D L = 512 2.6 -> 1.8 (the host's
+// launches then set the pace), L = 2048 4.4 -> 3.0, L = 4096 8.4 -> 6.5, L = 8192
+// 24.4 -> 23.6; 3D L = 128 3.0 -> 2.2, L = 202 8.7 -> 6.4.  (The int8 passes
 // gained nothing by it: 2D L = 500 2.75 -> 2.77, L = 1000 2.75 -> 3.64.)
 constexpr int kWordsFull = 0, kWordsAligned = 1, kWordsRagged = 2;
 
 // Multi-hit: the first item's later trials drawn ahead too, up to this many, kept
-// in shared memory (three hits, us a pass: 2D L = 512 3.6 -> 2.1, L = 2048 7.6 ->
-// 5.4, L = 8192 66 either way).
+// in shared memory (three hits, us a pass: 2D L = 512 3.6 -> 3.3, L = 2048 7.6 ->
+// 5.8, L = 8192 66 either way).
 constexpr int kLaterTrials = 3;
 
 template <int DIMS, bool MEASURE, int RULE, int WORDS>
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
     };
     auto load = [&](const PackedPlace& pl) {
         if constexpr (WORDS != kWordsFull) {
-            return packed_load<DIMS, 1>(a, geom, pl);
+            return packed_load<DIMS>(a, geom, pl);
         } else {
             const uint32_t nq = 1u << nq_shift, r = pl.r, q = pl.q;
             const uint32_t* other = static_cast<const uint32_t*>(a.other);
@@ -85,14 +86,14 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
             // x-neighbour word: the one before (p = 0) or after (p = 1), wrapping in the row
             const uint32_t xq = (w.p == 0 ? q - 1u : q + 1u) & (nq - 1u);
             w.at = row + q;
-            w.o = __ldg(other + w.at);
-            w.x = __ldg(other + row + xq);
-            w.ym = __ldg(other + (plane + ((y - 1u) & (L - 1u))) * nq + q);
-            w.yp = __ldg(other + (plane + ((y + 1u) & (L - 1u))) * nq + q);
+            w.o = other[w.at];
+            w.x = other[row + xq];
+            w.ym = other[(plane + ((y - 1u) & (L - 1u))) * nq + q];
+            w.yp = other[(plane + ((y + 1u) & (L - 1u))) * nq + q];
             w.zm = w.zp = 0u;
             if (DIMS == 3) {
-                w.zm = __ldg(other + ((((z - 1u) & (L - 1u)) * L + y) * nq + q));
-                w.zp = __ldg(other + ((((z + 1u) & (L - 1u)) * L + y) * nq + q));
+                w.zm = other[(((z - 1u) & (L - 1u)) * L + y) * nq + q];
+                w.zp = other[(((z + 1u) & (L - 1u)) * L + y) * nq + q];
             }
             w.s = static_cast<const uint32_t*>(a.own)[w.at];
             w.valid = 0xFFFFFFFFu;
@@ -104,7 +105,6 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
     };
     int e_acc = 0, m_acc = 0;
     uint32_t first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * step;
-    launch_dependents();
     if (first < items) {
         uint32_t A[kThresholds<DIMS, RULE>];
         PackedPlace pl = place(first);
@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
             }
         }
         grid_dependency_wait();
+        launch_dependents();
         PackedWord w = load(pl);
         for (;;) {
             __syncwarp();
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
         }
     } else {
         grid_dependency_wait();
+        launch_dependents();
     }
     if (MEASURE) block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
 }
