@@ -102,7 +102,7 @@ __device__ __forceinline__ void group_sync() {
 // word of its own row taken cyclically (funnel-shifted by one byte).  Every
 // word, row ends and wrap rows included, takes this one path, with the rule
 // and draws of int8_word (word w's draw is Philox group w).
-template <int DIMS, bool MEASURE, int NC, int RULE>
+template <int DIMS, bool MEASURE, int RULE>
 __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom& g, uint32_t w,
                                                int& e_acc, int& m_sum) {
     uint32_t* own = static_cast<uint32_t*>(a.own);
@@ -117,22 +117,22 @@ __device__ __forceinline__ void int8_word_rows(const PassArgs& a, const WordGeom
     const int p = (a.c + (int)y + (int)z) & 1;
     const uint32_t row0 = r * nq;
     const uint32_t s = own[w];
-    const uint32_t nx = load_other<NC>(other + w);
+    const uint32_t nx = other[w];
     uint32_t nxs;
     if (p == 0) {  // byte j <- byte j - 1 of the row, cyclically
-        const uint32_t prev = load_other<NC>(other + row0 + (q == 0u ? nq - 1u : q - 1u));
+        const uint32_t prev = other[row0 + (q == 0u ? nq - 1u : q - 1u)];
         nxs = __funnelshift_l(prev, nx, 8);
     } else {       // byte j <- byte j + 1 of the row, cyclically
-        const uint32_t next = load_other<NC>(other + row0 + (q + 1u == nq ? 0u : q + 1u));
+        const uint32_t next = other[row0 + (q + 1u == nq ? 0u : q + 1u)];
         nxs = __funnelshift_r(nx, next, 8);
     }
     const uint32_t plane = z * g.L;
-    const uint32_t nym = load_other<NC>(other + (plane + (y == 0u ? g.L - 1u : y - 1u)) * nq + q);
-    const uint32_t nyp = load_other<NC>(other + (plane + (y + 1u == g.L ? 0u : y + 1u)) * nq + q);
+    const uint32_t nym = other[(plane + (y == 0u ? g.L - 1u : y - 1u)) * nq + q];
+    const uint32_t nyp = other[(plane + (y + 1u == g.L ? 0u : y + 1u)) * nq + q];
     uint32_t nzm = 0u, nzp = 0u;
     if (DIMS == 3) {
-        nzm = load_other<NC>(other + ((z == 0u ? g.L - 1u : z - 1u) * g.L + y) * nq + q);
-        nzp = load_other<NC>(other + ((z + 1u == g.L ? 0u : z + 1u) * g.L + y) * nq + q);
+        nzm = other[((z == 0u ? g.L - 1u : z - 1u) * g.L + y) * nq + q];
+        nzp = other[((z + 1u == g.L ? 0u : z + 1u) * g.L + y) * nq + q];
     }
     const uint32_t D = disagreements<DIMS>(s, nx, nxs, nym, nyp, nzm, nzp);
     const Philox4 u = philox4x32_10(w, a.t, (uint32_t)a.c, kTagSweep, a.key0, a.key1);
@@ -168,33 +168,33 @@ __device__ __forceinline__ PassArgs job_args(const BatchJob& j, int c, uint32_t 
 
 // The int8 layout's pass of a job: not inlined, so that it does not add to the
 // registers of the packed one (ISING_AUTO's layout).
-template <int DIMS, bool MEASURE, int NC, int RULE>
+template <int DIMS, bool MEASURE, int RULE>
 __device__ __noinline__ void job_pass_int8(const BatchJob& j, const PassArgs& a, uint32_t rank,
                                            uint32_t nthr, int& e_acc, int& m_acc) {
     const WordGeom g((uint32_t)j.W, (uint32_t)j.L, j.rows);
     const uint32_t vecs = (j.half + 15u) >> 4;
     if (j.W >= 64 && vecs >= nthr) {
         for (uint32_t v = rank; v < vecs; v += nthr)
-            int8_vec<DIMS, MEASURE, NC, RULE>(a, g, v, e_acc, m_acc);
+            int8_vec<DIMS, MEASURE, RULE>(a, g, v, e_acc, m_acc);
     } else if (j.W % 4 == 0 && RULE != kRuleMultiHit) {
         // short rows of whole words: one uniform path for every word
         const uint32_t words = j.half >> 2;
         for (uint32_t w = rank; w < words; w += nthr)
-            int8_word_rows<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
+            int8_word_rows<DIMS, MEASURE, RULE>(a, g, w, e_acc, m_acc);
     } else {  // short rows or few vectors: four sites per item spread further
         const uint32_t words = (j.half + 3u) >> 2;
         for (uint32_t w = rank; w < words; w += nthr)
-            int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_acc);
+            int8_word<DIMS, MEASURE, RULE>(a, g, w, e_acc, m_acc);
     }
 }
 
-template <int DIMS, int LAYOUT, bool MEASURE, int NC, int RULE>
+template <int DIMS, int LAYOUT, bool MEASURE, int RULE>
 __device__ __forceinline__ void job_pass(const BatchJob& j, const PackedGeom& geom, int c,
                                          uint32_t t, uint32_t rank, uint32_t nthr, int& e_acc,
                                          int& m_acc) {
     const PassArgs a = job_args(j, c, t);
     if (LAYOUT == ISING_INT8) {
-        job_pass_int8<DIMS, MEASURE, NC, RULE>(j, a, rank, nthr, e_acc, m_acc);
+        job_pass_int8<DIMS, MEASURE, RULE>(j, a, rank, nthr, e_acc, m_acc);
     } else {
         // (one body for aligned and ragged rows: at half the code the kernels
         // spill less and stay in the instruction cache)
@@ -212,7 +212,7 @@ __device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom&
     if constexpr (LAYOUT == ISING_INT8) {
         const WordGeom g((uint32_t)j.W, (uint32_t)j.L, j.rows);
         const uint32_t v = first + (threadIdx.x & 31u);
-        if (16u * v < j.half) int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_acc);
+        if (16u * v < j.half) int8_vec<DIMS, MEASURE, RULE>(a, g, v, e_acc, m_acc);
     } else {
         packed_words<DIMS, MEASURE, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
     }
@@ -220,11 +220,10 @@ __device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom&
 
 template <int DIMS, int LAYOUT, int MODE, int RULE>
 __device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader) {
-    // plain loads in both modes: the passes of a cluster job are separated by
-    // the cluster barrier, whose release/acquire (cluster scope) makes the
-    // other CTAs' writes of the previous pass visible to them (3 % faster on
-    // the 2048-lattice mix than reading through L2 only)
-    constexpr int NC = 0;
+    // (the passes of a cluster job are separated by the cluster barrier, whose
+    // release/acquire at cluster scope makes the other CTAs' writes of the
+    // previous pass visible to plain loads: 3 % faster on the 2048-lattice mix
+    // than reading through L2 only)
     const BatchJob j = *jp;
     // in shared memory: the kernel runs at its register cap
     __shared__ PackedGeom geom;
@@ -239,9 +238,9 @@ __device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader)
         int e = 0, m = 0;
         for (int c = 0; c < 2; ++c) {
             if (measure)
-                job_pass<DIMS, LAYOUT, true, NC, RULE>(j, geom, c, t, rank, nthr, e, m);
+                job_pass<DIMS, LAYOUT, true, RULE>(j, geom, c, t, rank, nthr, e, m);
             else
-                job_pass<DIMS, LAYOUT, false, NC, RULE>(j, geom, c, t, rank, nthr, e, m);
+                job_pass<DIMS, LAYOUT, false, RULE>(j, geom, c, t, rank, nthr, e, m);
             group_sync<MODE>();  // this pass's writes before the next pass reads them
         }
         if (measure) {
@@ -318,8 +317,8 @@ __global__ void __launch_bounds__(256, RULE == kRuleHeatBath ? 2 : 3) batch_kern
 // 100 sweeps of 2048, where clusters balance: 45.8, 43.0, 43.7.
 template <int RULE>
 __global__ void __launch_bounds__(256, RULE == kRuleHeatBath ? 2 : 3)
-    joint_pass_kernel(const BatchJob* __restrict__ jobs, const PackedGeom* __restrict__ geoms,
-                      const JointChunk* __restrict__ chunks, int n_chunks, uint32_t s, int c) {
+    joint_pass_kernel(const BatchJob* jobs, const PackedGeom* geoms, const JointChunk* chunks,
+                      int n_chunks, uint32_t s, int c) {
     const int lane = threadIdx.x & 31;
     const int warps = (int)(gridDim.x * blockDim.x) >> 5;
     int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5;

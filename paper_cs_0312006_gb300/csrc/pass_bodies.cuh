@@ -15,9 +15,9 @@
 // finds each neighbour from the site's coordinates.  Both paths apply the
 // same rule and the same draw (word h & 3 of Philox(seed; h >> 2, t, c, 0)).
 //
-// NC selects how the other colour is read (see load_other): the per-lattice
-// pass kernels use the read-only path; the batched kernel, which runs both
-// colour passes of many sweeps in one launch, uses coherent loads.
+// The other colour is read with ordinary loads throughout: a chained pass lives
+// while the pass before it still writes that colour, and the batched kernel runs
+// both colours' passes in one launch (see grid_dependency_wait()).
 #pragma once
 
 #include <cstdint>
@@ -29,14 +29,6 @@ namespace ising {
 constexpr uint32_t kByteBit1 = 0x02020202u;
 constexpr uint32_t kByteBit7 = 0x80808080u;
 constexpr uint32_t kByteOnes = 0x01010101u;
-
-// Load modes for the other colour: 1 = read-only path (ld.global.nc, only when
-// nothing writes the array during the kernel), 0 = a plain coherent load.
-template <int NC, typename T>
-__device__ __forceinline__ T load_other(const T* p) {
-    if (NC == 1) return __ldg(p);
-    return *p;
-}
 
 // 0xFF per site whose flip is decided without a draw: byte j of D is 2 d_j, and
 // bit 7 of D + bias is set iff d_j >= dims (dE <= 0).
@@ -131,11 +123,10 @@ __device__ __forceinline__ uint32_t disagreements(uint32_t s, uint32_t n0, uint3
 
 // Four bytes of the other colour starting at byte offset o (o >= 0; the array
 // is padded so that the word after the last one may be read).
-template <int NC>
 __device__ __forceinline__ uint32_t window4(const uint32_t* other, uint32_t o) {
-    const uint32_t lo = load_other<NC>(other + (o >> 2));
+    const uint32_t lo = other[o >> 2];
     if ((o & 3u) == 0u) return lo;
-    const uint32_t hi = load_other<NC>(other + (o >> 2) + 1);
+    const uint32_t hi = other[(o >> 2) + 1];
     return __funnelshift_r(lo, hi, 8u * (o & 3u));
 }
 
@@ -178,7 +169,7 @@ struct WordGeom {
 // Update word w of the int8 colour array `own` (colour a.c).  Accumulates the
 // sum of the spins written (m_sum) and, in the white pass,
 // sum (2 d_new - 2 dims) over them (e_acc).
-template <int DIMS, bool MEASURE, int NC, int RULE>
+template <int DIMS, bool MEASURE, int RULE>
 __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, uint32_t w,
                                           int& e_acc, int& m_sum) {
     uint32_t* own = static_cast<uint32_t*>(a.own);
@@ -198,14 +189,14 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
     fast = fast && (p == 0 ? xh0 != 0u : xh0 + 4u != g.W);
     if (fast) {
         const uint32_t s = own[w];
-        const uint32_t nx = load_other<NC>(other + w);
-        const uint32_t nxs = p == 0 ? window4<NC>(other, h0 - 1u) : window4<NC>(other, h0 + 1u);
-        const uint32_t nym = window4<NC>(other, h0 - g.W);
-        const uint32_t nyp = window4<NC>(other, h0 + g.W);
+        const uint32_t nx = other[w];
+        const uint32_t nxs = p == 0 ? window4(other, h0 - 1u) : window4(other, h0 + 1u);
+        const uint32_t nym = window4(other, h0 - g.W);
+        const uint32_t nyp = window4(other, h0 + g.W);
         uint32_t nzm = 0u, nzp = 0u;
         if (DIMS == 3) {
-            nzm = window4<NC>(other, h0 - g.L * g.W);
-            nzp = window4<NC>(other, h0 + g.L * g.W);
+            nzm = window4(other, h0 - g.L * g.W);
+            nzp = window4(other, h0 + g.L * g.W);
         }
         const uint32_t D = disagreements<DIMS>(s, nx, nxs, nym, nyp, nzm, nzp);
         uint32_t X;
@@ -253,14 +244,12 @@ __device__ __forceinline__ void int8_word(const PassArgs& a, const WordGeom& g, 
         const uint32_t rym = plane + (y == 0u ? g.L - 1u : y - 1u);
         const uint32_t ryp = plane + (y + 1u == g.L ? 0u : y + 1u);
         const int s = own_b[h];
-        int hsum = load_other<NC>(other_b + r * g.W + xm) + load_other<NC>(other_b + r * g.W + xp) +
-                   load_other<NC>(other_b + rym * g.W + xh) +
-                   load_other<NC>(other_b + ryp * g.W + xh);
+        int hsum = other_b[r * g.W + xm] + other_b[r * g.W + xp] + other_b[rym * g.W + xh] +
+                   other_b[ryp * g.W + xh];
         if (DIMS == 3) {
             const uint32_t rzm = (z == 0u ? g.L - 1u : z - 1u) * g.L + y;
             const uint32_t rzp = (z + 1u == g.L ? 0u : z + 1u) * g.L + y;
-            hsum += load_other<NC>(other_b + rzm * g.W + xh) +
-                    load_other<NC>(other_b + rzp * g.W + xh);
+            hsum += other_b[rzm * g.W + xh] + other_b[rzp * g.W + xh];
         }
         s_val[j] = s;
         d_val[j] = (2 * DIMS - s * hsum) >> 1;  // k = s*h = 2*(dims - d)
@@ -444,14 +433,14 @@ struct Window16 {
                           __funnelshift_r(w2, w3, b), __funnelshift_r(w3, w4, b));
     }
 };
-template <int NC, bool FROM_BEFORE = false>
+template <bool FROM_BEFORE = false>
 __device__ __forceinline__ Window16 load_window(const uint4* other16, uint32_t o) {
     Window16 w;
     w.r = o & 15u;
     const bool before = FROM_BEFORE && o >= 0xFFFFFFF0u;
     const uint32_t b = before ? 0u : o >> 4;
-    w.lo = load_other<NC>(other16 + b);
-    w.hi = load_other<NC>(other16 + (before || w.r == 0u ? b : b + 1u));
+    w.lo = other16[b];
+    w.hi = other16[before || w.r == 0u ? b : b + 1u];
     return w;
 }
 
@@ -479,14 +468,14 @@ __device__ __forceinline__ uint4 select4(const uint4& m, const uint4& t, const u
 // (int8_word) the few at the row ends and edges held the whole pass up, alone
 // (2D L = 1000 7.6 -> 2.7, 3D L = 202 32.4 -> 9.2 us a pass).  Accumulates
 // m_sum and, in the white pass, e_acc as int8_word does.
-template <int DIMS, bool MEASURE, int NC, int RULE>
+template <int DIMS, bool MEASURE, int RULE>
 __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, uint32_t v,
                                          int& e_acc, int& m_sum) {
     const uint32_t h0 = 16u * v, W = g.W;
     if (W < 16u) {  // short rows: word by word
 #pragma unroll 1
         for (uint32_t w = 4u * v; w < 4u * v + 4u; ++w)
-            if (4u * w < g.half) int8_word<DIMS, MEASURE, NC, RULE>(a, g, w, e_acc, m_sum);
+            if (4u * w < g.half) int8_word<DIMS, MEASURE, RULE>(a, g, w, e_acc, m_sum);
         return;
     }
     const uint32_t r0 = g.by_W.quot(h0);
@@ -514,19 +503,19 @@ __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, u
     const uint32_t plane = g.L * W, y_wrap = plane - W, z_wrap = (g.L - 1u) * plane;
     const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u), ones4 = make_uint4(~0u, ~0u, ~0u, ~0u);
     const uint4 s = own16[v];
-    const uint4 nx = load_other<NC>(other16 + v);
-    const Window16 wym = load_window<NC>(other16, y0 == 0u ? h0 + y_wrap : h0 - W);
-    const Window16 wyp = load_window<NC>(other16, y0 + 1u == g.L ? h0 - y_wrap : h0 + W);
+    const uint4 nx = other16[v];
+    const Window16 wym = load_window(other16, y0 == 0u ? h0 + y_wrap : h0 - W);
+    const Window16 wyp = load_window(other16, y0 + 1u == g.L ? h0 - y_wrap : h0 + W);
     Window16 wzm{zero4, zero4, 0u}, wzp{zero4, zero4, 0u};
     if (DIMS == 3) {
-        wzm = load_window<NC>(other16, z0 == 0u ? h0 + z_wrap : h0 - plane);
-        wzp = load_window<NC>(other16, z0 + 1u == g.L ? h0 - z_wrap : h0 + plane);
+        wzm = load_window(other16, z0 == 0u ? h0 + z_wrap : h0 - plane);
+        wzp = load_window(other16, z0 + 1u == g.L ? h0 - z_wrap : h0 + plane);
     }
-    const uint32_t word_before = load_other<NC>(other32 + (v == 0u ? 0u : 4u * v - 1u));
-    const uint32_t word_behind = load_other<NC>(other32 + 4u * v + 4u);
-    const uint32_t row_first = load_other<NC>(other8 + row);
-    const uint32_t row_last = load_other<NC>(other8 + row + W - 1u);
-    const uint32_t next_last = load_other<NC>(other8 + row + (two ? 2u * W : W) - 1u);
+    const uint32_t word_before = other32[v == 0u ? 0u : 4u * v - 1u];
+    const uint32_t word_behind = other32[4u * v + 4u];
+    const uint32_t row_first = other8[row];
+    const uint32_t row_last = other8[row + W - 1u];
+    const uint32_t next_last = other8[row + (two ? 2u * W : W) - 1u];
     // the draws while the loads are under way
     uint32_t cnt[4];
     vec_counts<DIMS, RULE>(4u * v, a, (uint32_t)a.c, cnt);
@@ -537,13 +526,13 @@ __device__ __forceinline__ void int8_vec(const PassArgs& a, const WordGeom& g, u
         nzp = wzp.get();
     }
     if (edge) {  // part B's own windows (they may start up to 15 bytes before the first row)
-        const Window16 bym = load_window<NC, true>(other16, h0 + (yb == 0u ? y_wrap : 0u - W));
+        const Window16 bym = load_window<true>(other16, h0 + (yb == 0u ? y_wrap : 0u - W));
         const Window16 byp =
-            load_window<NC, true>(other16, h0 + (yb + 1u == g.L ? 0u - y_wrap : W));
+            load_window<true>(other16, h0 + (yb + 1u == g.L ? 0u - y_wrap : W));
         Window16 bzm = wzm, bzp = wzp;
         if (DIMS == 3) {
-            bzm = load_window<NC, true>(other16, h0 + (zb == 0u ? z_wrap : 0u - plane));
-            bzp = load_window<NC, true>(other16, h0 + (zb + 1u == g.L ? 0u - z_wrap : plane));
+            bzm = load_window<true>(other16, h0 + (zb == 0u ? z_wrap : 0u - plane));
+            bzp = load_window<true>(other16, h0 + (zb + 1u == g.L ? 0u - z_wrap : plane));
         }
         nym = select4(part_b, bym.get(), nym);
         nyp = select4(part_b, byp.get(), nyp);

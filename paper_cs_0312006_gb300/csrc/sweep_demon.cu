@@ -103,10 +103,10 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 3) pass_demon_strip(PassA
     const int r_begin = (int)(((int64_t)sidx * rows) / S);
     const int len = active ? (int)(((int64_t)(sidx + 1) * rows) / S) - r_begin : 0;
     const int max_len = (rows + S - 1) / S;
-    const uint4* __restrict__ O = reinterpret_cast<const uint4*>(a.other) + v;
+    const uint4* O = reinterpret_cast<const uint4*>(a.other) + v;
     uint4* __restrict__ Sv = reinterpret_cast<uint4*>(a.own) + v;
     uint4* __restrict__ Q = reinterpret_cast<uint4*>(a.dem) + v;
-    const uint32_t* __restrict__ Ow = reinterpret_cast<const uint32_t*>(a.other);
+    const uint32_t* Ow = reinterpret_cast<const uint32_t*>(a.other);
     const uint32_t vm_word = 4u * (uint32_t)wrap_prev(v, nv) + 3u;
     const uint32_t vp_word = 4u * (uint32_t)wrap_next(v, nv);
     const uint32_t lo_bias = (0x80u - (uint32_t)DIMS) * kByteOnes;
@@ -134,26 +134,26 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 3) pass_demon_strip(PassA
         const int r = r_begin + i;
         const int rd_next = rd + 1 == rows ? 0 : rd + 1;
         if (valid && reload) {
-            om = __ldg(O + (uint32_t)(plane + wrap_prev(y, L)) * nv);
-            oc = __ldg(O + (uint32_t)r * nv);
-            op = __ldg(O + (uint32_t)(plane + wrap_next(y, L)) * nv);
+            om = O[(uint32_t)(plane + wrap_prev(y, L)) * nv];
+            oc = O[(uint32_t)r * nv];
+            op = O[(uint32_t)(plane + wrap_next(y, L)) * nv];
             sc = Sv[(uint32_t)r * nv];
             qc = Q[(uint32_t)rd * nv];
             if (DIMS == 3) {
-                zm = __ldg(O + (uint32_t)(plane_m + y) * nv);
-                zp = __ldg(O + (uint32_t)(plane_p + y) * nv);
+                zm = O[(uint32_t)(plane_m + y) * nv];
+                zp = O[(uint32_t)(plane_p + y) * nv];
             }
         }
         // prefetch row r + 1 while it stays in this plane
         const bool pf = (i + 1 < len) && (y + 1 < L);
         uint4 op_n = zero, sc_n = zero, qc_n = zero, zm_n = zero, zp_n = zero;
         if (pf) {
-            op_n = __ldg(O + (uint32_t)(plane + (y + 2 < L ? y + 2 : y + 2 - L)) * nv);
+            op_n = O[(uint32_t)(plane + (y + 2 < L ? y + 2 : y + 2 - L)) * nv];
             sc_n = Sv[(uint32_t)(r + 1) * nv];
             qc_n = Q[(uint32_t)rd_next * nv];
             if (DIMS == 3) {
-                zm_n = __ldg(O + (uint32_t)(plane_m + y + 1) * nv);
-                zp_n = __ldg(O + (uint32_t)(plane_p + y + 1) * nv);
+                zm_n = O[(uint32_t)(plane_m + y + 1) * nv];
+                zp_n = O[(uint32_t)(plane_p + y + 1) * nv];
             }
         }
         uint32_t prev_w = __shfl_up_sync(0xffffffffu, oc.w, 1);
@@ -162,13 +162,13 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 3) pass_demon_strip(PassA
             const int p = (a.c + y + z) & 1;
             uint4 sh;
             if (p == 0) {
-                if (lane == 0 || v == 0) prev_w = __ldg(Ow + (uint32_t)r * nv * 4u + vm_word);
+                if (lane == 0 || v == 0) prev_w = Ow[(uint32_t)r * nv * 4u + vm_word];
                 sh.x = __funnelshift_l(prev_w, oc.x, 8);
                 sh.y = __funnelshift_l(oc.x, oc.y, 8);
                 sh.z = __funnelshift_l(oc.y, oc.z, 8);
                 sh.w = __funnelshift_l(oc.z, oc.w, 8);
             } else {
-                if (lane == 31 || v == nv - 1) next_x = __ldg(Ow + (uint32_t)r * nv * 4u + vp_word);
+                if (lane == 31 || v == nv - 1) next_x = Ow[(uint32_t)r * nv * 4u + vp_word];
                 sh.x = __funnelshift_r(oc.x, oc.y, 8);
                 sh.y = __funnelshift_r(oc.y, oc.z, 8);
                 sh.z = __funnelshift_r(oc.z, oc.w, 8);
@@ -360,14 +360,14 @@ __global__ void __launch_bounds__(kPacked4Threads, DIMS == 3 ? 6 : ROWS == 2 ? 7
         }
         const uint32_t plane = z * L;
         uint4 o[ROWS + 2];  // the other colour's rows y - 1 .. y + ROWS
-        o[0] = __ldg(other + (plane + (y == 0u ? L - 1u : y - 1u)) * n4 + g);
+        o[0] = other[(plane + (y == 0u ? L - 1u : y - 1u)) * n4 + g];
 #pragma unroll
-        for (int i = 0; i < ROWS; ++i) o[i + 1] = __ldg(other + (r + i) * n4 + g);
-        o[ROWS + 1] = __ldg(other + (plane + (y + ROWS == L ? 0u : y + ROWS)) * n4 + g);
+        for (int i = 0; i < ROWS; ++i) o[i + 1] = other[(r + i) * n4 + g];
+        o[ROWS + 1] = other[(plane + (y + ROWS == L ? 0u : y + ROWS)) * n4 + g];
         uint4 ozm = make_uint4(0u, 0u, 0u, 0u), ozp = ozm;
         if (DIMS == 3) {
-            ozm = __ldg(other + ((z == 0u ? L - 1u : z - 1u) * L + y) * n4 + g);
-            ozp = __ldg(other + ((z + 1u == L ? 0u : z + 1u) * L + y) * n4 + g);
+            ozm = other[((z == 0u ? L - 1u : z - 1u) * L + y) * n4 + g];
+            ozp = other[((z + 1u == L ? 0u : z + 1u) * L + y) * n4 + g];
         }
         uint4 sv[ROWS], qa[ROWS], qb[ROWS];
         uint32_t rd[ROWS], edge[ROWS];  // storage row; the word beside the group
@@ -379,8 +379,8 @@ __global__ void __launch_bounds__(kPacked4Threads, DIMS == 3 ? 6 : ROWS == 2 ? 7
             qb[i] = Q1[rd[i] * n4 + g];
             const uint32_t* row = other_w + (r + i) * nq;
             edge[i] = (a.c + (int)y + i + (int)z) & 1
-                          ? __ldg(row + (g + 1u == n4 ? 0u : 4u * g + 4u))
-                          : __ldg(row + (g == 0u ? nq : 4u * g) - 1u);
+                          ? row[g + 1u == n4 ? 0u : 4u * g + 4u]
+                          : row[(g == 0u ? nq : 4u * g) - 1u];
         }
 #pragma unroll
         for (int i = 0; i < ROWS; ++i) {
@@ -447,28 +447,28 @@ __global__ void __launch_bounds__(256) pass_demon_packed(PassArgs a) {
         const uint32_t nb = W - 32u * q < 32u ? W - 32u * q : 32u;
         const uint32_t valid = nb == 32u ? 0xFFFFFFFFu : ((1u << nb) - 1u);
         const uint32_t plane = z * L, row = r * nq;
-        const uint32_t o = __ldg(other + row + q);
-        const uint32_t oym = __ldg(other + (plane + (y == 0u ? L - 1u : y - 1u)) * nq + q);
-        const uint32_t oyp = __ldg(other + (plane + (y + 1u == L ? 0u : y + 1u)) * nq + q);
+        const uint32_t o = other[row + q];
+        const uint32_t oym = other[(plane + (y == 0u ? L - 1u : y - 1u)) * nq + q];
+        const uint32_t oyp = other[(plane + (y + 1u == L ? 0u : y + 1u)) * nq + q];
         uint32_t ozm = 0u, ozp = 0u;
         if (DIMS == 3) {
-            ozm = __ldg(other + ((z == 0u ? L - 1u : z - 1u) * L + y) * nq + q);
-            ozp = __ldg(other + ((z + 1u == L ? 0u : z + 1u) * L + y) * nq + q);
+            ozm = other[((z == 0u ? L - 1u : z - 1u) * L + y) * nq + q];
+            ozp = other[((z + 1u == L ? 0u : z + 1u) * L + y) * nq + q];
         }
         const uint32_t s = own[row + q];
         const int p = (a.c + (int)y + (int)z) & 1;
         uint32_t sh;
         if (p == 0) {  // bit b <- neighbour xh - 1
-            const uint32_t prev = q == 0u ? __ldg(other + row + nq - 1u) << (31u - ((W - 1u) & 31u))
-                                          : __ldg(other + row + q - 1u);
+            const uint32_t prev = q == 0u ? other[row + nq - 1u] << (31u - ((W - 1u) & 31u))
+                                          : other[row + q - 1u];
             sh = __funnelshift_l(prev, o, 1);
         } else {       // bit b <- neighbour xh + 1
             if (q + 1u == nq) {
-                const uint32_t first = q == 0u ? o : __ldg(other + row);
+                const uint32_t first = q == 0u ? o : other[row];
                 const uint32_t top = 1u << (nb - 1u);
                 sh = ((o >> 1) & ~top) | ((first & 1u) ? top : 0u);
             } else {
-                sh = __funnelshift_r(o, __ldg(other + row + q + 1u), 1);
+                sh = __funnelshift_r(o, other[row + q + 1u], 1);
             }
         }
         const Digits d = DIMS == 2 ? digits2(s ^ o, s ^ sh, s ^ oym, s ^ oyp)

@@ -54,9 +54,9 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
     const int r_begin = (int)(((int64_t)sidx * rows) / S);
     const int len = active ? (int)(((int64_t)(sidx + 1) * rows) / S) - r_begin : 0;
     const int max_len = (rows + S - 1) / S;
-    const uint4* __restrict__ O = reinterpret_cast<const uint4*>(a.other) + v;
+    const uint4* O = reinterpret_cast<const uint4*>(a.other) + v;
     uint4* __restrict__ Sv = reinterpret_cast<uint4*>(a.own) + v;
-    const uint32_t* __restrict__ Ow = reinterpret_cast<const uint32_t*>(a.other);
+    const uint32_t* Ow = reinterpret_cast<const uint32_t*>(a.other);
     const uint32_t vm_word = 4u * (uint32_t)wrap_prev(v, nv) + 3u;  // last word of column v-1
     const uint32_t vp_word = 4u * (uint32_t)wrap_next(v, nv);       // first word of column v+1
 
@@ -78,24 +78,24 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
         const bool valid = i < len;
         const int r = r_begin + i;
         if (valid && reload) {
-            om = __ldg(O + (uint32_t)(plane + wrap_prev(y, L)) * nv);
-            oc = __ldg(O + (uint32_t)r * nv);
-            op = __ldg(O + (uint32_t)(plane + wrap_next(y, L)) * nv);
+            om = O[(uint32_t)(plane + wrap_prev(y, L)) * nv];
+            oc = O[(uint32_t)r * nv];
+            op = O[(uint32_t)(plane + wrap_next(y, L)) * nv];
             sc = Sv[(uint32_t)r * nv];
             if (DIMS == 3) {
-                zm = __ldg(O + (uint32_t)(plane_m + y) * nv);
-                zp = __ldg(O + (uint32_t)(plane_p + y) * nv);
+                zm = O[(uint32_t)(plane_m + y) * nv];
+                zp = O[(uint32_t)(plane_p + y) * nv];
             }
         }
         // prefetch row r + 1 while it stays in this plane
         const bool pf = (i + 1 < len) && (y + 1 < L);
         uint4 op_n = zero, sc_n = zero, zm_n = zero, zp_n = zero;
         if (pf) {
-            op_n = __ldg(O + (uint32_t)(plane + (y + 2 < L ? y + 2 : y + 2 - L)) * nv);
+            op_n = O[(uint32_t)(plane + (y + 2 < L ? y + 2 : y + 2 - L)) * nv];
             sc_n = Sv[(uint32_t)(r + 1) * nv];
             if (DIMS == 3) {
-                zm_n = __ldg(O + (uint32_t)(plane_m + y + 1) * nv);
-                zp_n = __ldg(O + (uint32_t)(plane_p + y + 1) * nv);
+                zm_n = O[(uint32_t)(plane_m + y + 1) * nv];
+                zp_n = O[(uint32_t)(plane_p + y + 1) * nv];
             }
         }
         // x-neighbour bytes shifted by one site (all lanes take part in the shuffles)
@@ -105,13 +105,13 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
             const int p = (a.c + y + z) & 1;
             uint4 sh;
             if (p == 0) {
-                if (lane == 0 || v == 0) prev_w = __ldg(Ow + (uint32_t)r * nv * 4u + vm_word);
+                if (lane == 0 || v == 0) prev_w = Ow[(uint32_t)r * nv * 4u + vm_word];
                 sh.x = __funnelshift_l(prev_w, oc.x, 8);
                 sh.y = __funnelshift_l(oc.x, oc.y, 8);
                 sh.z = __funnelshift_l(oc.y, oc.z, 8);
                 sh.w = __funnelshift_l(oc.z, oc.w, 8);
             } else {
-                if (lane == 31 || v == nv - 1) next_x = __ldg(Ow + (uint32_t)r * nv * 4u + vp_word);
+                if (lane == 31 || v == nv - 1) next_x = Ow[(uint32_t)r * nv * 4u + vp_word];
                 sh.x = __funnelshift_r(oc.x, oc.y, 8);
                 sh.y = __funnelshift_r(oc.y, oc.z, 8);
                 sh.z = __funnelshift_r(oc.z, oc.w, 8);
@@ -128,7 +128,6 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 4 : 2) pass_int8_strip(PassAr
                                                             e_acc, m_acc);
             Sv[(uint32_t)r * nv] = s;
             ++n_rows;
-
         }
         // slide the window
         if (pf) {
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(256, DIMS == 2 ? 3 : 2) pass_int8_vecs(PassArg
     grid_dependency_wait();
     launch_dependents();
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < vecs; v += stride)
-        int8_vec<DIMS, MEASURE, 1, RULE>(a, g, v, e_acc, m_acc);
+        int8_vec<DIMS, MEASURE, RULE>(a, g, v, e_acc, m_acc);
     if (MEASURE) block_reduce_add(e_acc, m_acc, a.obs, a.c == 1);
 }
 

@@ -70,3 +70,63 @@ def check(eng, ahead, dims, L, layout, rule, **kw):
 @pytest.mark.parametrize("rule", [METROPOLIS, HEATBATH, MULTIHIT])
 def test_packed(eng, ahead, dims, L, rule):
     check(eng, ahead, dims, L, BITPACK, rule)
+
+
+# strips, strips in 3D, rows that end inside a vector, the staged kernel
+@pytest.mark.parametrize("dims,L,staged", [(2, 512, False), (3, 64, False), (2, 600, False),
+                                           (3, 98, False), (2, 512, True), (3, 64, True)])
+@pytest.mark.parametrize("rule", [METROPOLIS, HEATBATH, MULTIHIT])
+def test_int8(eng, ahead, dims, L, staged, rule):
+    check(eng, ahead, dims, L, INT8, rule,
+          kernel=eng.KERNEL_TMA if staged else eng.KERNEL_STRIP)
+
+
+@pytest.mark.parametrize("L,layout", [(512, INT8), (600, INT8), (512, BITPACK), (600, BITPACK)])
+def test_demon(eng, ahead, L, layout):
+    import torch
+    q = np.random.default_rng(L).integers(0, 4, L * L, dtype=np.uint8)
+    s = oracle.init(2, L, 7)
+    s_o, q_o, E_o, M_o = oracle.run_demon(2, L, s, q, 3, SWEEPS, EVERY)
+    want, start = torch.from_numpy(s_o).cuda(), torch.from_numpy(s).cuda()
+    got = torch.empty_like(want)
+    lat = eng.Lattice(2, L, 0.43, 7, layout=layout)
+    for k in range(REPEATS // 2):
+        lat.set_demons(q, qmax=3)
+        lat.set_rule(2)
+        lat.set_spins_async(start.data_ptr())
+        ahead.sweep(2, 2)
+        for _ in range(SWEEPS):
+            lat.sweep(1, EVERY)
+        lat.get_spins_async(got.data_ptr())
+        E, M = lat.observables()
+        ahead.observables()
+        assert np.array_equal(E, E_o) and np.array_equal(M, M_o), (L, layout, k)
+        assert torch.equal(got, want) and np.array_equal(lat.get_demons(), q_o), (L, layout, k)
+    lat.close()
+
+
+def test_joint(eng, ahead):
+    """A batch's joint passes, launch after launch (each reads the job table that
+    the end of the launch before it has moved on)."""
+    import torch
+    shapes = [(3, 64, BITPACK), (2, 512, INT8), (2, 600, BITPACK), (3, 98, INT8)]
+    lats = [eng.Lattice(d, L, 0.43 if d == 2 else 0.22, 3 * L, layout=y) for d, L, y in shapes]
+    want = [wanted(d, L, METROPOLIS) for d, L, _ in shapes]
+    got = [torch.empty(L ** d, dtype=torch.int8, device="cuda") for d, L, _ in shapes]
+    batch = eng.Batch(lats, [EVERY] * len(lats), [EVERY] * len(lats), big_sites=1)
+    for k in range(REPEATS):
+        for lat in lats:
+            lat.init()
+        ahead.sweep(2, 2)
+        for _ in range(SWEEPS // EVERY):
+            batch.launch()
+        batch.sync()
+        ahead.observables()
+        for lat, g, (s_o, E_o, M_o) in zip(lats, got, want):
+            lat.get_spins_async(g.data_ptr())
+            E, M = lat.observables()
+            assert np.array_equal(E, E_o) and np.array_equal(M, M_o), k
+            assert np.array_equal(g.cpu().numpy(), s_o), k
+    batch.close()
+    for lat in lats:
+        lat.close()
