@@ -446,7 +446,10 @@ int ising_batch_create(ising_batch **out, ising_lattice *const *lats, int n,
  * earlier size).  May be called while an earlier launch of the batch is still
  * running: that launch keeps its own lattices and counts, and the new ones
  * follow it on the batch stream.  The new lattices are moved to the batch
- * stream; a captured graph is dropped and recaptured at the next launch.
+ * stream; a captured graph is dropped and recaptured at the next launch.  If it
+ * fails for want of memory the batch holds no lattices: ising_batch_launch
+ * returns ISING_EINVAL until an update succeeds (after ISING_EINVAL for its own
+ * arguments the old set stays).
  * For loops that change the set every round (continuous batching) without
  * creating and destroying a batch each time. */
 int ising_batch_update(ising_batch *b, ising_lattice *const *lats, int n,

@@ -480,6 +480,7 @@ struct ising_batch {
     std::vector<int> rule;       // each lattice's rule when the batch was made
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t uploaded = nullptr;
+    bool ready = false;        // members, queues and tables are complete
     bool table_valid = false;  // device table equals the host mirror's continuation
     bool order_dirty = true;   // the device order array must be uploaded
     int64_t launches = 0;
@@ -650,7 +651,8 @@ int check_members(ising_lattice* const* lats, int n, const int64_t* sweeps,
 // Take a new lattice list: move the lattices to the batch stream, build the
 // per-rule queues (largest work first, split at the size thresholds) and make
 // room in the tables.  Growing the tables frees the old ones in stream order,
-// after any launch already queued.
+// after any launch already queued.  A failure on the way (an allocation) leaves
+// the batch without a complete set: `ready` stays false, and launches are refused.
 int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int64_t* sweeps,
                    const int* measure_every) {
     const ising_batch_opts& o = b->opts;
@@ -658,6 +660,7 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
         const int rc = ising_set_stream(lats[i], b->stream);
         if (rc != ISING_OK) return rc;
     }
+    b->ready = false;
     b->lats.assign(lats, lats + n);
     b->sweeps.assign(sweeps, sweeps + n);
     b->every.resize(n);
@@ -737,6 +740,7 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
     }
     b->table_valid = false;
     b->order_dirty = true;
+    b->ready = true;
     return ISING_OK;
 }
 
@@ -807,7 +811,7 @@ int ising_batch_update(ising_batch* b, ising_lattice* const* lats, int n, const 
 }
 
 int ising_batch_launch(ising_batch* b) {
-    if (!b) return ISING_EINVAL;
+    if (!b || !b->ready) return ISING_EINVAL;
     const int n = (int)b->lats.size();
     // host-side checks and record space, then the job table if it changed
     bool moved = !b->table_valid;

@@ -1,0 +1,79 @@
+"""The engine's host code without a GPU: its objects linked against a stand-in
+for the CUDA runtime (``_fake_cudart.c``) in which kernels only leave their names
+and an allocation can be made to fail."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+INT8, BITPACK = 0, 1
+
+
+@pytest.fixture(scope="module")
+def fake_library(tmp_path_factory):
+    from paper_cs_0312006_gb300 import _build
+    objects = os.path.join(_build.OUT_DIR, "obj", "*.o")
+    _build.build(force=len(glob.glob(objects)) != len(_build.sources()))
+    out = str(tmp_path_factory.mktemp("host") / "libising_host.so")
+    # -Bsymbolic: a CUDA runtime loaded earlier in the process does not take over
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-o", out,
+                    os.path.join(HERE, "_fake_cudart.c"), *sorted(glob.glob(objects)),
+                    "-lstdc++", "-lpthread", "-lm"], check=True)
+    return out
+
+
+@pytest.fixture()
+def eng(fake_library, monkeypatch):
+    from paper_cs_0312006_gb300 import _build, engine
+    monkeypatch.setattr(_build, "LIB_PATH", fake_library)
+    monkeypatch.setattr(engine, "_lib", None)
+    lib = engine.load_library()
+    lib.fake_launches.argtypes = [ctypes.c_char_p]
+    lib.fake_fail_allocation(-1)
+    lib.fake_clear_launches()
+    yield engine
+    lib.fake_fail_allocation(-1)
+    lib.ising_clear_int8_configs()
+
+
+def launches(eng, part):
+    return eng.load_library().fake_launches(part.encode())
+
+
+@pytest.mark.parametrize("cluster_size", [0, 2])
+def test_failed_update_refuses_to_launch(eng, cluster_size):
+    """Whichever allocation of an update fails, the batch launches nothing until
+    an update succeeds; then it launches all of its lattices again."""
+    lib = eng.load_library()
+    few = [eng.Lattice(2, 64, 0.4, 1, layout=BITPACK)]
+    many = [eng.Lattice(2, L, 0.4, L, layout=layout) for L in (32, 64, 130)
+            for layout in (INT8, BITPACK)]
+    failures = 0
+    for k in range(20):
+        batch = eng.Batch(few, 3, cluster_size=cluster_size, big_sites=1)
+        batch.launch()
+        lib.fake_fail_allocation(k)
+        try:
+            batch.update(many, 2)
+        except eng.IsingError as e:
+            failures += 1
+            assert e.code == eng.ENOMEM
+            assert not lib.fake_fail_pending()
+            lib.fake_clear_launches()
+            with pytest.raises(eng.IsingError) as refused:
+                batch.launch()
+            assert refused.value.code == eng.EINVAL
+            assert launches(eng, "") == 0
+            batch.sync()
+            batch.update(many, 2)
+        lib.fake_fail_allocation(-1)
+        lib.fake_clear_launches()
+        batch.launch()
+        assert launches(eng, "joint_pass_kernel") == (4 if cluster_size == 0 else 0)
+        batch.sync()
+        batch.close()
+    assert failures == (10 if cluster_size == 0 else 4)
