@@ -54,7 +54,10 @@ enum {
 enum {
     ISING_KERNEL_AUTO = 0,  /* a registered configuration (ising_set_int8_config), else staged
                                for 2D with 4096 <= L <= 16384 and for 3D with L / 32 a power of
-                               two from L = 256 on, and strip otherwise (measured) */
+                               two from L = 256 on, and strip otherwise (measured); without a
+                               registered one, runs of two sweeps or more of small lattices
+                               (Metropolis or heat bath, up to 2D L = 576 and 3D L = 64) are one
+                               launch that holds the lattice in shared memory */
     ISING_KERNEL_STRIP = 1, /* per-thread row strips, neighbour rows in registers */
     ISING_KERNEL_TMA = 2    /* tiles staged in shared memory by bulk (TMA) copies */
 };
@@ -251,16 +254,18 @@ int ising_get_spins_async(ising_lattice *lat, int8_t *out);
  * (L^dims bytes).  Asynchronous on the handle's stream. */
 int ising_export_device(ising_lattice *lat, int8_t *dev_out);
 
-/* Choose the int8 pass kernel of a lattice (ISING_KERNEL_*).  The staged
- * kernel needs L % 32 == 0 and tiles that fit in shared memory; otherwise, and
- * for the bit-packed layout, the choice is recorded but the general kernels
- * run.  Results never depend on it. */
+/* Choose the int8 pass kernel of a lattice (ISING_KERNEL_*): its sweeps then run
+ * as that kernel's passes, whatever their number.  The staged kernel needs
+ * L % 32 == 0 and tiles that fit in shared memory; otherwise, and for the
+ * bit-packed layout, the choice is recorded but the general kernels run.  Results
+ * never depend on it. */
 int ising_set_kernel(ising_lattice *lat, int kernel);
 
-/* The int8 pass kernel the lattice's sweeps run, with ISING_KERNEL_AUTO and the
- * size limits resolved: ISING_KERNEL_TMA or ISING_KERNEL_STRIP (which also
- * stands for the general kernel used when L/2 is not a multiple of 16).  For
- * the bit-packed layout *kernel is set to -1. */
+/* The int8 pass kernel the lattice's sweeps run (all but the runs that are one
+ * launch, see ISING_KERNEL_AUTO), with ISING_KERNEL_AUTO and the size limits
+ * resolved: ISING_KERNEL_TMA or ISING_KERNEL_STRIP (which also stands for the
+ * general kernel used when L/2 is not a multiple of 16).  For the bit-packed
+ * layout *kernel is set to -1. */
 int ising_get_kernel(const ising_lattice *lat, int *kernel);
 
 /*
@@ -284,10 +289,11 @@ typedef struct ising_int8_config {
 /* Register `cfg` for int8 lattices of `dims` with L_min <= L <= L_max: their
  * ISING_KERNEL_AUTO passes (and, for tile_rows and ctas_per_sm, their
  * ISING_KERNEL_TMA passes) run it from the next sweep on; a later
- * registration overrides an earlier one where they overlap; a configuration
- * the staged kernel cannot take for some L (tile rows not dividing L, stages
- * too large for shared memory) runs the general kernels there.  Process-wide
- * (all devices); thread-safe.  ISING_EINVAL for dims not in {2, 3}, an empty
+ * registration overrides an earlier one where they overlap; lattices with a
+ * registered configuration run passes whatever the number of sweeps (see
+ * ISING_KERNEL_AUTO); a configuration the staged kernel cannot take for some L
+ * (tile rows not dividing L, stages too large for shared memory) runs the general
+ * kernels there.  Process-wide (all devices); thread-safe.  ISING_EINVAL for dims not in {2, 3}, an empty
  * range or a value out of range. */
 int ising_set_int8_config(int dims, int L_min, int L_max, const ising_int8_config *cfg);
 

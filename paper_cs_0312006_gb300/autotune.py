@@ -162,7 +162,9 @@ def tune_int8(dims: int, L: int, L_range=None, sweeps: int = 5, use_cache: bool 
     """Measure every int8 pass configuration on a (dims, L) lattice, check
     that all give bit-identical spins and E/M, and register the fastest for
     lattices with L in ``L_range`` (default: L alone) so that
-    ISING_KERNEL_AUTO runs it.  Returns {"config": ..., "results": [...]}."""
+    ISING_KERNEL_AUTO runs it.  The passes are timed one sweep a call; runs of
+    sweeps of small lattices (up to 2D L = 576, 3D L = 64), one launch without a
+    registered configuration, are passes with one.  Returns {"config": ..., "results": [...]}."""
     from . import engine
     lo, hi = L_range or (L, L)
     key = f"int8|{_device_name()}|{dims}|{L}"

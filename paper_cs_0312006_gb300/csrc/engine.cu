@@ -366,6 +366,14 @@ ising_int8_config resolve_int8(const ising_lattice* h) {
     return c;
 }
 
+// The caller leaves the choice to the engine: no kernel set, none registered for
+// the lattice's shape (both are about the int8 passes only).
+bool built_in_choice(const ising_lattice* h) {
+    ising_int8_config tuned;
+    return h->layout == ISING_BITPACK ||
+           (h->kernel == ISING_KERNEL_AUTO && !find_policy(h->dims, h->L, &tuned));
+}
+
 bool uses_tma(const ising_lattice* h) { return resolve_int8(h).kernel == ISING_KERNEL_TMA; }
 
 // Arguments of colour pass c of sweep t.
@@ -526,7 +534,7 @@ int ising_sweep(ising_lattice* h, int64_t n, int measure_every) {
         if (rc != ISING_OK) return rc;
     }
     int64_t rec = h->n_rec;
-    if (ising::resident_ok(h, n)) {
+    if (ising::resident_ok(h, n) && built_in_choice(h)) {
         ISING_CHECK(ising::resident_sweep(h, ising::pass_args(h, 0, (uint32_t)h->t, nullptr), n,
                                           measure_every,
                                           h->obs ? h->obs + 2 * rec : nullptr));

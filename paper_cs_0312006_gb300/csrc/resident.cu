@@ -362,7 +362,9 @@ cudaError_t launch_resident_layout(const ResidentArgs& k, int layout, unsigned r
 // 128 6.2 / 7.2, but ragged L = 50 8.2 / 7.3 and L = 256 8.2 / 7.2; three L = 50
 // 10.3 / 10.6, L = 256 9.3 / 10.6, but L = 250 14.1 / 10.7; one sweep L = 64 6.2 /
 // 4.0 in either layout.  Rows of less than a vector go word by word in the int8
-// pass kernels (4 us a pass and more), so those always come here.
+// pass kernels (4 us a pass and more), so those always come here.  (Unless the
+// caller names an int8 kernel, by ising_set_kernel or a registered configuration:
+// ising_sweep then runs that one's passes.)
 bool resident_ok(const ising_lattice* h, int64_t n) {
     if (h->rule != ISING_RULE_METROPOLIS && h->rule != ISING_RULE_HEATBATH) return false;
     if (n > 0x7FFFFFFF) return false;

@@ -77,3 +77,35 @@ def test_failed_update_refuses_to_launch(eng, cluster_size):
         batch.sync()
         batch.close()
     assert failures == (10 if cluster_size == 0 else 4)
+
+
+def kernels_of(eng, lat, n):
+    eng.load_library().fake_clear_launches()
+    lat.sweep(n, 1)
+    return {part: launches(eng, part) for part in ("resident_kernel", "pass_int8_strip",
+                                                   "pass_int8_vecs", "pass_int8_tma",
+                                                   "pass_packed")
+            if launches(eng, part)}
+
+
+@pytest.mark.parametrize("dims,L", [(2, 64), (2, 160), (2, 512), (3, 32), (3, 64)])
+def test_chosen_kernel_runs(eng, dims, L):
+    """Runs of sweeps of small lattices are one launch, unless the caller names an
+    int8 kernel or registers a configuration: then its passes run."""
+    strip, staged, whole = {"pass_int8_strip": 8}, {"pass_int8_tma": 8}, {"resident_kernel": 1}
+    assert kernels_of(eng, eng.Lattice(dims, L, 0.3, 1), 4) == whole
+    for kernel, want in ((eng.KERNEL_STRIP, strip), (eng.KERNEL_TMA, staged)):
+        lat = eng.Lattice(dims, L, 0.3, 1, kernel=kernel)
+        assert kernels_of(eng, lat, 4) == want
+        lat.set_kernel(eng.KERNEL_AUTO)
+        assert kernels_of(eng, lat, 4) == whole
+    lat = eng.Lattice(dims, L, 0.3, 1)
+    packed = eng.Lattice(dims, L, 0.3, 1, layout=BITPACK)
+    as_before = kernels_of(eng, packed, 4)
+    eng.set_int8_config(dims, L, L, eng.KERNEL_TMA, tile_rows=1)
+    assert kernels_of(eng, lat, 4) == staged
+    assert kernels_of(eng, packed, 4) == as_before  # the choice is about int8 passes
+    eng.set_int8_config(dims, L, L, eng.KERNEL_STRIP)
+    assert kernels_of(eng, lat, 4) == strip
+    eng.clear_int8_configs()
+    assert kernels_of(eng, lat, 4) == whole
