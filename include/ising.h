@@ -402,29 +402,36 @@ int ising_release_cached_memory(void);
 
 /*
  * Batched form: many independent lattices (any mix of dims, L, layout, beta,
- * seed) advanced by one persistent launch, with the same arithmetic and draws
- * as ising_sweep, so each lattice ends bit-identical to running it alone.
- * Lattices with at least huge_sites sites are advanced by the per-lattice
- * pass kernels (each pass over the whole GPU) on the batch stream; the others
- * are jobs of one persistent kernel, taken largest first from a device work
- * queue: lattices with at least big_sites sites are run by a thread-block
- * cluster of cluster_size CTAs (colour passes separated by the hardware
- * cluster barrier), smaller ones by a single CTA each.  The launch is captured once
- * in a CUDA graph and replayed; each launch advances lattice i by sweeps[i]
- * sweeps and records E/M after sweep u iff (u + 1) % measure_every[i] == 0.
+ * seed) advanced together, with the same arithmetic and draws as ising_sweep, so
+ * each lattice ends bit-identical to running it alone.  Each launch advances
+ * lattice i by sweeps[i] sweeps and records E/M after sweep u iff
+ * (u + 1) % measure_every[i] == 0.  A lattice takes one of three ways:
+ *   - per-lattice pass kernels (each pass over the whole GPU) on the batch
+ *     stream: at least huge_sites sites, and the rules without another form;
+ *   - joint passes: one launch per colour pass of all lattices that take part,
+ *     two per sweep, as many sweeps as the longest of them has;
+ *   - one persistent launch, in which the lattices are jobs taken largest first
+ *     from a device work queue: those with at least big_sites sites by a
+ *     thread-block cluster of cluster_size CTAs (colour passes separated by the
+ *     hardware cluster barrier), smaller ones by a single CTA each.  This launch
+ *     is captured once in a CUDA graph and replayed.
+ * With a cluster size given, nothing takes joint passes.  With cluster_size 0 the
+ * engine compares both ways' times, by the lattices' sizes and sweep counts, and
+ * gives the joint passes those that would keep the queue waiting.
  */
 typedef struct ising_batch ising_batch; /* opaque */
 
 typedef struct ising_batch_opts {
     int block_threads;  /* threads per CTA: 128 or 256 (0: 256) */
     int cluster_size;   /* CTAs per cluster for large lattices, 1..8; 1 runs every
-                           lattice on a single CTA.  0: large lattices advance
-                           together, one launch per colour pass of all of them
-                           (clusters of 4 in ising_batch_run_static) */
-    int64_t big_sites;  /* from how many sites a lattice counts as large (0: 2^18
-                           with clusters, 2^12 with joint passes) */
+                           lattice on a single CTA.  0: the engine chooses between
+                           joint passes and the queue (clusters of 4 there, as in
+                           ising_batch_run_static) */
+    int64_t big_sites;  /* from how many sites a lattice counts as large: taken by a
+                           cluster or, with cluster_size 0 and a value given here, by
+                           joint passes (0: 2^18, or the engine's choice) */
     int use_graph;      /* >= 0: capture the persistent launch in a CUDA graph and
-                           replay it; < 0: plain launches */
+                           replay it; < 0: plain launches (joint passes always are) */
     int64_t huge_sites; /* lattices this large use the per-lattice kernels
                            (0: 2^22; < 0: never) */
 } ising_batch_opts;
@@ -435,9 +442,11 @@ typedef struct ising_batch_opts {
  * give a value >= 1 per lattice; opts may be NULL.  All lattices are moved to
  * `stream` (as by ising_set_stream).  The batch borrows the handles: between
  * ising_batch_launch and ising_batch_sync they must not be used directly, and
- * they must outlive the batch.  Device memory: a job table (96 B per lattice).
- * Lattices of each update rule (ISING_RULE_*) form their own queues, run by
- * one persistent launch per rule present; demon-dynamics and multi-hit
+ * they must outlive the batch.  Device memory: a job table (96 B per lattice) and,
+ * with joint passes, a geometry (36 B) per lattice and 8 B per 992 sites of a
+ * colour (bit-packed full words; 512 sites in int8).
+ * Lattices of each update rule (ISING_RULE_*) form their own queues and joint
+ * passes, run one rule after the other; demon-dynamics and multi-hit
  * lattices are advanced by the per-lattice kernels like the huge ones.  A lattice's rule
  * must not change while the batch exists (ising_batch_launch then returns
  * ISING_EINVAL).
@@ -461,15 +470,19 @@ int ising_batch_create(ising_batch **out, ising_lattice *const *lats, int n,
 int ising_batch_update(ising_batch *b, ising_lattice *const *lats, int n,
                        const int64_t *sweeps, const int *measure_every);
 
-/* Advance every lattice of the batch by its sweeps (asynchronous). */
+/* Advance every lattice of the batch by its sweeps (asynchronous: it returns once
+ * everything is queued.  CUDA holds a caller back while about a thousand
+ * launches are queued already, so with joint passes or per-lattice kernels a
+ * launch of more sweeps than some hundreds returns as its last sweeps start). */
 int ising_batch_launch(ising_batch *b);
 
 /* Wait for the batch's launches; afterwards the lattices may be used
  * directly (ising_observables, ising_get_spins, ...). */
 int ising_batch_sync(ising_batch *b);
 
-/* Resident grid size, the number of jobs in the cluster / CTA queues and the
- * number of lattices advanced by the per-lattice kernels. */
+/* Resident grid size (the larger of both forms'), the number of lattices in joint
+ * passes or the cluster queue, of those in the CTA queue and of those advanced by
+ * the per-lattice kernels. */
 int ising_batch_info(const ising_batch *b, int *grid, int *n_big, int *n_small, int *n_huge);
 
 /* Free the batch (not the lattices).  NULL is accepted. */
@@ -478,12 +491,12 @@ void ising_batch_destroy(ising_batch *b);
 /*
  * The batched form in one call: advance lattice i of lats[0..n-1] by
  * sweeps[i] sweeps (Sec. 2.2's black and white passes, the same arithmetic and
- * draws as ising_sweep) in one persistent launch on `stream`, recording E/M
+ * draws as ising_sweep) in one launch of a batch on `stream`, recording E/M
  * after sweep u iff (u + 1) % measure_every == 0 into each handle's own record
  * buffer (read them with ising_observables or ising_observables_gather).
  * Equivalent to ising_batch_create (default options, no graph) +
  * ising_batch_launch + ising_batch_sync + ising_batch_destroy: it moves the
- * lattices to `stream`, allocates the job table for the call, and returns
+ * lattices to `stream`, allocates the tables for the call, and returns
  * once the sweeps are done.  Errors as at those calls (ISING_EINVAL for
  * n < 1, measure_every < 1, a NULL or repeated lattice, a negative count).
  */

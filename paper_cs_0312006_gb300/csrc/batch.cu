@@ -4,10 +4,11 @@
 //
 // Lattices of at least huge_sites sites are advanced with the per-lattice
 // pass kernels (each pass spread over the whole GPU), issued on the batch's
-// stream ahead of the rest.  When the caller leaves the cluster size open, the
-// large ones of the rest take joint passes (joint_pass_kernel: one launch per
-// colour pass of all of them) and the small ones the persistent kernel, a CTA
-// each; with a cluster size given, all go through the persistent kernel.
+// stream ahead of the rest.  When the caller leaves the cluster size open, those
+// of the rest for which that is the shorter way (choose_joint) take joint passes
+// (joint_pass_kernel: one launch per colour pass of all of them) and the others the
+// persistent kernel; with a cluster size given, all go through the persistent
+// kernel.
 //
 // Work queue of the persistent kernel: one job per lattice, holding everything
 // its sweeps need (spin arrays, thresholds, key, first sweep index, sweep
@@ -71,11 +72,10 @@ static void fill_job(BatchJob& j, const ising_lattice* h, int64_t nsweeps, int e
     j.measure_every = every;
 }
 
-// From this many sites a lattice of a batch takes part in the joint passes; the
-// others run a CTA each, all their sweeps at once (256 mixed lattices: 4.0 ms
-// here, 4.2 from 2^14 sites on and 5.3 from 2^16, a CTA's slowest lattice then
-// outlasting the rest; 2^10 the same as here).
-constexpr int64_t kJointSites = 1 << 12;
+// Batches whose cluster size is left open: what runs in the persistent kernel
+// takes a cluster of four from 2^18 sites on, a CTA below.
+constexpr int64_t kClusterSites = 1 << 18;
+constexpr int kOpenCluster = 4;
 
 // A warp's share of a joint pass: the items of a job from `first` on.
 struct JointChunk {
@@ -307,14 +307,11 @@ __global__ void __launch_bounds__(256, RULE == kRuleHeatBath ? 2 : 3) batch_kern
     }
 }
 
-// One colour pass of many lattices in one launch (the large lattices of a
-// batch whose cluster size is left open).  A chunk is a warp's step of one job:
-// 31 or 32 words of a packed lattice, 32 16-site vectors of an int8 one.  Every
-// pass spreads over the whole GPU, so lattices of any mix finish together; a
-// cluster per lattice left the largest lattice on a few SMs long after the rest
-// were done.  50 sweeps of 256 mixed lattices: 11.5 ms with clusters of four,
-// 5.9 of eight, 4.0 in joint passes; of 64: 5.3, 2.4, 0.9; of 16: 4.1, 1.9, 0.7;
-// 100 sweeps of 2048, where clusters balance: 45.8, 43.0, 43.7.
+// One colour pass of many lattices in one launch (see choose_joint).  A chunk is a
+// warp's step of one job: 31 or 32 words of a packed lattice, 32 16-site vectors of
+// an int8 one.  Every pass spreads over the whole GPU, so lattices of any mix
+// finish together; a cluster per lattice leaves the largest lattice on a few SMs
+// long after the rest are done.
 template <int RULE>
 __global__ void __launch_bounds__(256, RULE == kRuleHeatBath ? 2 : 3)
     joint_pass_kernel(const BatchJob* jobs, const PackedGeom* geoms, const JointChunk* chunks,
@@ -466,7 +463,9 @@ struct ising_batch {
     int* d_counters = nullptr;   // two per rule
     RuleQueues q[2];             // [ISING_RULE_METROPOLIS], [ISING_RULE_HEATBATH]
     int grid[2] = {0, 0};        // resident CTAs of each rule's kernel (0: not yet known)
-    bool joint = false;          // large lattices in joint passes (opts.cluster_size was 0)
+    bool joint = false;          // joint passes may be taken (opts.cluster_size was 0) ...
+    bool by_cost = false;        // ... by choose_joint, not from opts.big_sites on
+    int cluster = 1;             // CTAs per cluster of the persistent launch
     std::vector<int> joint_jobs[2];  // [rule]
     JointQueue jq[2];
     JointChunk* d_chunks = nullptr;
@@ -497,7 +496,7 @@ cudaError_t launch_batch_kernel(ising_batch* b, cudaStream_t st) {
     for (int r = 0; r < 2 && e == cudaSuccess; ++r) {
         const RuleQueues& q = b->q[r];
         if (q.n_big + q.n_small == 0) continue;
-        e = launch_rule(r, q.grid, b->opts.block_threads, b->opts.cluster_size, b->d_jobs,
+        e = launch_rule(r, q.grid, b->opts.block_threads, b->cluster, b->d_jobs,
                         b->d_order + q.offset, q.n_big, q.n_small, b->d_counters + 2 * r, st);
     }
     return e;
@@ -530,6 +529,94 @@ void free_batch(ising_batch* b) {
     if (b->h_jobs) cudaFreeHost(b->h_jobs);
     if (b->h_order) cudaFreeHost(b->h_order);
     delete b;
+}
+
+// What a pass of a lattice costs, in us by its items (32-site words, 16-site
+// vectors) over a rate: run by a CTA that has an SM to itself (besides 0.9 us a
+// pass), as a share of a GPU full of such CTAs or clusters, and as a share of a
+// joint pass (besides its launch, `pass` us: the host's two launches a sweep, or
+// one wave of word-by-word rows).  The rates are those of batches of 1 to 1024
+// equal lattices, 2D L = 64 - 1024 and 3D L = 16 - 96, by the body that takes the
+// rows.
+struct PassCost {
+    double alone, queue, joint, pass;
+};
+PassCost pass_cost(const ising_lattice* h) {
+    double cta, queue, joint, pass = 2.9, items = (double)(h->half_sites + 15) / 16;
+    if (h->layout == ISING_BITPACK) {
+        items = (double)h->rows * (double)((h->W + 31) / 32);
+        cta = 200, queue = 35e3, joint = 28e3;
+    } else if (h->W >= 64) {
+        cta = 310, queue = 55e3, joint = 36e3;
+    } else if (h->W >= 16) {
+        cta = 155, queue = 29e3, joint = 24e3;
+    } else {
+        cta = 170, queue = 23e3, joint = 9e3, pass = 7.0;
+    }
+    return PassCost{items / cta, items / queue, items / joint, pass};
+}
+
+// Which of `jobs` (one update rule's) take joint passes, when the caller names
+// neither a cluster size nor a size to go by: those whose own chain of passes
+// would last longest, as many as make the sum of both parts shortest.  The queue's
+// part lasts as long as its longest chain (CTAs sharing an SM slow one another down,
+// by 2.4 from three dozen on) or all its work at its rate, the joint part its
+// passes' launches and work.  So a few small lattices stay with a CTA each, a
+// batch that fills the GPU with CTAs or clusters too, and what would leave it idle
+// goes jointly.  Us a pass, joint / queue (a CTA each, below 2^18 sites, clusters of
+// four above), bit-packed: 4 of 2D L = 64 2.8 / 1.1, 16 of L = 128 3.3 / 3.1, of L =
+// 192 3.4 / 5.5, of L = 512 5.2 / 10.5; 64 of L = 256 5.2 / 13.5; 256 of L = 256
+// 12.5 / 13.6, of L = 1024 146 / 116; 1024 of L = 64 5.2 / 4.4, of L = 256 38.5 /
+// 31.2; int8: 256 of L = 256 16.7 / 17.2, 1024 of it 57.1 / 37.6; 256 of 3D L = 16
+// 8.5 / 3.3.  Of 164 such batches the choice was the faster one or within 8 % of it
+// but once (four of 3D L = 24, 2.8 / 2.6).  Mixed sizes, ms: 256 lattices, 50 sweeps,
+// 3.5 jointly (3.7 with those below 2^12 sites queued), 8.2 queued; 2048, 100 sweeps,
+// 44.9 jointly, 37.9 queued, which is what the choice takes.
+void choose_joint(const ising_batch* b, std::vector<int>& jobs, std::vector<int>& joint) {
+    struct Member {
+        double chain, work, share, joint, pass, sweeps;  // us, of one pass each way
+        int i, ctas;
+    };
+    std::vector<Member> ms;
+    ms.reserve(jobs.size());
+    double rest = 0.0;
+    int ctas = 0;
+    for (int i : jobs) {
+        const ising_lattice* h = b->lats[i];
+        const PassCost c = pass_cost(h);
+        const double n = (double)b->sweeps[i];
+        // a cluster of four takes its words 3.7 times as fast
+        const bool cluster = h->sites >= kClusterSites;
+        const double work = c.alone / (cluster ? 3.7 : 1.0);
+        ms.push_back(Member{n * (0.9 + work), n * work, n * c.queue, n * c.joint, c.pass, n, i,
+                            cluster ? kOpenCluster : 1});
+        rest += ms.back().share;
+        ctas += ms.back().ctas;
+    }
+    std::stable_sort(ms.begin(), ms.end(),
+                     [](const Member& x, const Member& y) { return x.chain > y.chain; });
+    double best = 0.0, work = 0.0, sweeps = 0.0, pass = 0.0;
+    size_t best_k = 0;
+    for (size_t k = 0; k <= ms.size(); ++k) {  // the first k jointly
+        double queue = 0.0;
+        if (k < ms.size()) {
+            const double shared = (ctas < 35 ? ctas : 35) / 25.0;
+            queue = std::max(ms[k].chain + shared * ms[k].work, rest);
+        }
+        const double total = queue + pass * sweeps + work;
+        if (k == 0 || total < best) {
+            best = total;
+            best_k = k;
+        }
+        if (k == ms.size()) break;
+        sweeps = std::max(sweeps, ms[k].sweeps);
+        pass = std::max(pass, ms[k].pass);
+        work += ms[k].joint;
+        rest -= ms[k].share;
+        ctas -= ms[k].ctas;
+    }
+    jobs.clear();
+    for (size_t k = 0; k < ms.size(); ++k) (k < best_k ? joint : jobs).push_back(ms[k].i);
 }
 
 // Items of a lattice in a joint pass, and how many a warp takes at a time.
@@ -681,12 +768,25 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
             b->in_table[i] = 0;
         } else {
             const bool large = b->lats[i]->sites >= o.big_sites;
-            (b->joint && large                 ? b->joint_jobs[r]
+            (b->joint && !b->by_cost && large  ? b->joint_jobs[r]
              : o.cluster_size > 1 && large ? big[r]
                                            : small[r])
                 .push_back(i);
         }
     }
+    int cluster = o.cluster_size;
+    if (b->by_cost) {
+        for (int r = 0; r < 2; ++r) {
+            std::vector<int> queued;
+            queued.swap(small[r]);
+            choose_joint(b, queued, b->joint_jobs[r]);
+            for (int i : queued)
+                (b->lats[i]->sites >= kClusterSites ? big[r] : small[r]).push_back(i);
+        }
+        cluster = big[0].empty() && big[1].empty() ? 1 : kOpenCluster;
+    }
+    if (cluster != b->cluster) b->grid[0] = b->grid[1] = 0;
+    b->cluster = cluster;
     auto by_work = [&](int x, int y) {
         return b->lats[x]->sites * b->sweeps[x] > b->lats[y]->sites * b->sweeps[y];
     };
@@ -728,8 +828,8 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
             continue;
         }
         int clusters = 0;
-        ISING_BCHECK(resident_clusters(r, o.block_threads, o.cluster_size, &clusters));
-        b->grid[r] = clusters * o.cluster_size;
+        ISING_BCHECK(resident_clusters(r, o.block_threads, b->cluster, &clusters));
+        b->grid[r] = clusters * b->cluster;
         b->q[r].grid = b->grid[r];
     }
     const int rc = joint_tables(b);
@@ -757,8 +857,9 @@ int ising_batch_create(ising_batch** out, ising_lattice* const* lats, int n,
     if (opts) o = *opts;
     const bool joint = o.cluster_size == 0;
     if (o.block_threads == 0) o.block_threads = 256;
-    if (joint) o.cluster_size = 1;  // what is left runs a CTA each
-    if (o.big_sites == 0) o.big_sites = joint ? kJointSites : 1 << 18;
+    const bool by_cost = joint && o.big_sites == 0;
+    if (joint) o.cluster_size = 1;
+    if (o.big_sites == 0) o.big_sites = kClusterSites;
     if (o.huge_sites == 0) o.huge_sites = (int64_t)1 << 22;
     if (o.block_threads != 128 && o.block_threads != 256) return ISING_EINVAL;
     if (o.cluster_size < 1 || o.cluster_size > 8) return ISING_EINVAL;
@@ -776,6 +877,7 @@ int ising_batch_create(ising_batch** out, ising_lattice* const* lats, int n,
     if (!b) return ISING_ENOMEM;
     b->opts = o;
     b->joint = joint;
+    b->by_cost = by_cost;
     b->dp = dp;
     b->stream = static_cast<cudaStream_t>(stream);
     cudaError_t e = pool_alloc(reinterpret_cast<void**>(&b->d_counters), 4 * sizeof(int), *dp,

@@ -109,3 +109,40 @@ def test_chosen_kernel_runs(eng, dims, L):
     assert kernels_of(eng, lat, 4) == strip
     eng.clear_int8_configs()
     assert kernels_of(eng, lat, 4) == whole
+
+
+def batch_launches(eng, specs, **opts):
+    """Launches of a batch of (dims, L, sweeps, copies[, rule]): joint passes, the
+    persistent kernel, and the lattices counted as large and as small."""
+    lats, sweeps = [], []
+    for dims, L, n, copies, *rule in specs:
+        for k in range(copies):
+            lats.append(eng.Lattice(dims, L, 0.3, k, layout=BITPACK, rule=rule[0] if rule else 0))
+            sweeps.append(n)
+    batch = eng.Batch(lats, sweeps, use_graph=False, **opts)
+    eng.load_library().fake_clear_launches()
+    batch.launch()
+    info = batch.info()
+    batch.close()
+    return (launches(eng, "joint_pass_kernel"), launches(eng, "batch_kernel"), info["n_big"],
+            info["n_small"])
+
+
+def test_batch_routes(eng):
+    """Which lattices of a batch take joint passes when the caller names no cluster
+    size: those that would keep a queue of CTAs waiting, not small ones beside
+    them that run longer, and none where the queue fills the GPU or waits for a
+    small one all the same."""
+    assert batch_launches(eng, [(2, 64, 5000, 4)]) == (0, 1, 0, 4)
+    assert batch_launches(eng, [(2, 512, 30, 16)]) == (60, 0, 16, 0)
+    assert batch_launches(eng, [(2, 1024, 100, 4), (2, 64, 300, 4)]) == (200, 1, 4, 4)
+    assert batch_launches(eng, [(2, 512, 30, 16), (2, 64, 5000, 4)]) == (0, 1, 16, 4)
+    assert batch_launches(eng, [(2, 256, 10, 1024)]) == (0, 1, 0, 1024)
+    assert batch_launches(eng, [(2, 1024, 10, 256)]) == (0, 1, 256, 0)  # clusters of four
+    # each update rule for itself
+    assert batch_launches(eng, [(2, 512, 30, 16), (2, 64, 500, 4, 1)]) == (60, 1, 16, 4)
+    # a size to go by, or a cluster size
+    assert batch_launches(eng, [(2, 64, 5, 4)], big_sites=1) == (10, 0, 4, 0)
+    assert batch_launches(eng, [(2, 64, 5, 4), (2, 32, 7, 3)], big_sites=4096) == (10, 1, 4, 3)
+    assert batch_launches(eng, [(2, 512, 30, 16)], cluster_size=2) == (0, 1, 16, 0)
+    assert batch_launches(eng, [(2, 512, 0, 16)])[0] == 0
