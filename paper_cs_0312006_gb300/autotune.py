@@ -1,9 +1,10 @@
 """Autotuner for the batched launch and the int8 per-lattice pass.
 
-Searches the launch shape of the persistent batched kernel -- threads per CTA,
-CTAs per cluster for large lattices, the size threshold of the cluster queue,
-and the spin layout policy -- on a scaled-down sample of the workload, and
-keeps the fastest; and, per lattice shape, the int8 colour pass (register
+Searches the launch shape of a batch -- the engine's own choice between joint
+passes and a queue, or the persistent kernel alone with its threads per CTA, CTAs
+per cluster for large lattices and the size threshold of the cluster queue -- and
+the spin layout policy on a scaled-down sample of the workload, and keeps the
+fastest; and, per lattice shape, the int8 colour pass (register
 strips, or tiles staged by bulk copies with their rows per tile -- one or two
 rows per thread at a time -- and resident CTAs per SM), registered with the
 engine so that ISING_KERNEL_AUTO runs the winner.  Every candidate must produce bit-identical spins and E/M
@@ -25,7 +26,7 @@ from . import batched
 
 CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_cs_0312006_gb300", "autotune.json")
 
-CANDIDATES = [
+CANDIDATES = [dict(block_threads=0, cluster_size=0, big_sites=0)] + [
     dict(block_threads=bt, cluster_size=cs, big_sites=bs)
     for bt in (128, 256)
     for cs in (1, 2, 4, 8)
@@ -60,7 +61,7 @@ def tune(specs, sample_sweeps: int = 40, sample_lattices: int = 512, seed: int =
          use_cache: bool = True, verbose: bool = False) -> dict:
     """Pick launch options for ``specs``; returns {"opts": ..., "layout": ...,
     "results": [...]}."""
-    key = f"{_device_name()}|{signature(specs)}"
+    key = f"batch|{_device_name()}|{signature(specs)}|{len(CANDIDATES)}"
     if use_cache and os.path.exists(CACHE):
         try:
             with open(CACHE) as f:

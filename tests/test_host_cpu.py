@@ -146,3 +146,16 @@ def test_batch_routes(eng):
     assert batch_launches(eng, [(2, 64, 5, 4), (2, 32, 7, 3)], big_sites=4096) == (10, 1, 4, 3)
     assert batch_launches(eng, [(2, 512, 30, 16)], cluster_size=2) == (0, 1, 16, 0)
     assert batch_launches(eng, [(2, 512, 0, 16)])[0] == 0
+
+
+def test_tuner_can_choose_the_default(monkeypatch):
+    """A batch run with no options is among what the batch tuner compares."""
+    from paper_cs_0312006_gb300 import autotune, workloads
+
+    def run_batched(specs, opts, launches, layout):
+        return (1.0 if opts.get("cluster_size") or opts.get("big_sites") else 0.5), []
+
+    monkeypatch.setattr(autotune.batched, "run_batched", run_batched)
+    monkeypatch.setattr(autotune, "_device_name", lambda: "none")
+    best = autotune.tune(workloads.batched_mix(8, 10), use_cache=False)["opts"]
+    assert not best["cluster_size"] and not best["big_sites"] and not best["block_threads"]
