@@ -760,7 +760,7 @@ def run_gpu(args, world, rank, local):
 
 def batched_form(args) -> dict:
     """The batched form on its full workload (2048 lattices x 500 sweeps):
-    one persistent launch against one ising_sweep per lattice (one stream and
+    one launch of a batch against one ising_sweep per lattice (one stream and
     eight streams); every lattice bit-identical across the forms."""
     import torch
     from paper_cs_0312006_gb300 import autotune, batched, engine, workloads
@@ -898,8 +898,8 @@ def small_form(args) -> dict:
 
 def run_batched_workload(args):
     """2048 independent lattices (70% 2D L in [16,1024], 30% 3D L in [8,128],
-    log-uniform), 500 sweeps each: one persistent CUDA-graph launch (launch
-    shape from the autotuner) against one ising_sweep call per lattice."""
+    log-uniform), 500 sweeps each: one launch of a batch (its options from
+    the autotuner) against one ising_sweep call per lattice."""
     import torch
     from paper_cs_0312006_gb300 import _build, autotune, batched, engine, workloads
     _build.build()

@@ -1,6 +1,6 @@
-"""Batched workload driver: many independent lattices advanced by one
-persistent CUDA-graph launch (``Batch``) versus the plain form, one
-``ising_sweep`` call per lattice issued back to back on one stream.
+"""Batched workload driver: many independent lattices advanced together by one
+launch of a ``Batch`` versus the plain form, one ``ising_sweep`` call per lattice
+issued back to back on one stream.
 
 Both forms run identical arithmetic, so every lattice must end bit-identical;
 ``compare_forms`` checks that for every lattice and reports aggregate site

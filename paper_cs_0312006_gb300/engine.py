@@ -376,7 +376,10 @@ class Lattice:
 
 
 class Batch:
-    """Many lattices advanced by one persistent launch (``ising_batch_*``).
+    """Many lattices advanced together (``ising_batch_*``): by default in joint
+    passes, two launches a sweep, or from the queue of one persistent launch,
+    whichever the engine reckons shorter for each; with a ``cluster_size`` all from
+    the queue, with ``big_sites`` alone jointly from that size on.
 
     ``sweeps`` and ``measure_every`` are per lattice (sequences) or scalars.
     While a launch is in flight the lattices must not be used directly; call
@@ -450,8 +453,8 @@ class Batch:
 
 
 def batch_run(lattices, sweeps, measure_every: int = 1, stream=None) -> None:
-    """``ising_batch_run``: advance every lattice by its sweeps in one
-    persistent launch on ``stream`` and wait; records go to the handles."""
+    """``ising_batch_run``: advance every lattice by its sweeps as one batch
+    with default options on ``stream`` and wait; records go to the handles."""
     lib = load_library()
     n = len(lattices)
     sw = np.asarray(np.broadcast_to(np.asarray(sweeps, dtype=np.int64), (n,)),
