@@ -646,15 +646,16 @@ constexpr int kThresholds = RULE == kRuleHeatBath ? 2 * DIMS + 1 : DIMS;
 //
 // The draws of the Philox groups g0 .. g0 + 7 against all N thresholds: bit b of
 // A[n] is set iff draw b (word b & 3 of group g0 + (b >> 2)) lies below
-// threshold n.  Four calls at a time; without `both`, bits 16..31 stay clear.
+// threshold n.  Four calls at a time; of the second four only as many as `second`
+// says (0, 1 or 4), the other bits stay clear.
 template <int N>
-__device__ __forceinline__ void word_tests(uint32_t g0, const PassArgs& a, uint32_t c2, bool both,
+__device__ __forceinline__ void word_tests(uint32_t g0, const PassArgs& a, uint32_t c2, int second,
                                            uint32_t (&A)[N]) {
 #pragma unroll
     for (int n = 0; n < N; ++n) A[n] = 0u;
     static_for<2>([&](auto half) {
         constexpr int h = decltype(half)::value;
-        if (h == 1 && !both) return;
+        if (h == 1 && second < 4) return;
         PhiloxRuns<1> ps;
         const uint32_t base[1] = {g0 + 4u * h};
         ps.first_round(base, a.t, c2, kTagSweep, a.key0, a.key1);
@@ -668,6 +669,15 @@ __device__ __forceinline__ void word_tests(uint32_t g0, const PassArgs& a, uint3
             for (int n = 0; n < N; ++n) mark_below<(1u << (16 * h + b))>(A[n], w, a.thr[n]);
         });
     });
+    if (second == 1) {
+        const Philox4 u = philox4x32_10(g0 + 4u, a.t, c2, kTagSweep, a.key0, a.key1);
+        static_for<4>([&](auto bit) {
+            constexpr int j = decltype(bit)::value;
+            const uint32_t w = j == 0 ? u.w0 : j == 1 ? u.w1 : j == 2 ? u.w2 : u.w3;
+#pragma unroll
+            for (int n = 0; n < N; ++n) mark_below<(1u << (16 + j))>(A[n], w, a.thr[n]);
+        });
+    }
 }
 
 // Each site's answer for the threshold of its own number of disagreeing
@@ -714,11 +724,11 @@ constexpr uint32_t kWarpWords = DRAW == kDrawRagged ? 31u : 32u;
 // place: 3D L = 202 11.0 -> 8.6 us per pass; a joint pass of 256 mixed lattices
 // 47 -> 39 us.
 template <int DIMS, int RULE, int DRAW>
-__device__ __forceinline__ void packed_draws(uint32_t hbase, bool both, const PassArgs& a,
+__device__ __forceinline__ void packed_draws(uint32_t hbase, int second, const PassArgs& a,
                                              uint32_t c2,
                                              uint32_t (&A)[kThresholds<DIMS, RULE>]) {
     constexpr int N = kThresholds<DIMS, RULE>;
-    word_tests<N>(hbase >> 2, a, c2, both, A);
+    word_tests<N>(hbase >> 2, a, c2, second, A);
     if constexpr (DRAW == kDrawRagged) {
 #pragma unroll
         for (int n = 0; n < N; ++n) {
@@ -767,7 +777,7 @@ __device__ __forceinline__ uint32_t x_neighbours(const PackedWord& w) {
 // ragged draws the whole warp takes part.
 template <int DIMS, bool MEASURE, int RULE, int DRAW>
 __device__ __forceinline__ void packed_update(const PassArgs& a, const PackedWord& w,
-                                              uint32_t (&A)[kThresholds<DIMS, RULE>], bool both,
+                                              uint32_t (&A)[kThresholds<DIMS, RULE>], int second,
                                               int& e_acc, int& m_acc,
                                               const uint32_t* later = nullptr, int n_later = 0) {
     const uint32_t s = w.s, sh = x_neighbours(w);
@@ -797,7 +807,7 @@ __device__ __forceinline__ void packed_update(const PassArgs& a, const PackedWor
                     A[n] = later[((m - 1) * kThresholds<DIMS, RULE> + n) * (int)blockDim.x];
                 continue;
             }
-            packed_draws<DIMS, RULE, DRAW>(w.hbase, both, a, (uint32_t)a.c + 2u * (uint32_t)m, A);
+            packed_draws<DIMS, RULE, DRAW>(w.hbase, second, a, (uint32_t)a.c + 2u * (uint32_t)m, A);
         }
         flip = cur ^ s;
     }
@@ -889,8 +899,13 @@ __device__ __forceinline__ PackedWord packed_load(const PassArgs& a, const Packe
     return w;
 }
 
-// Rows of at most 13 sites need no draw past a word's first half.
-__device__ __forceinline__ bool packed_both(const PassArgs& a) { return a.W > 13; }
+// How many of a word's second four calls any of its sites needs: rows of one word
+// that start at most 3 draws into a group (2 where W is even, 0 where W % 4 == 0).
+// (64 of 3D L = 30 in a CTA each: 14.1 us a pass with eight calls, 9.8 with five.)
+__device__ __forceinline__ int packed_second(const PassArgs& a) {
+    const int last = a.W + (a.W % 4 == 0 ? 0 : a.W % 2 == 0 ? 2 : 3);
+    return last <= 16 ? 0 : last <= 20 ? 1 : 4;
+}
 
 // One step of a warp, loads first: their latency hides behind the draws.
 template <int DIMS, bool MEASURE, int RULE, int DRAW>
@@ -900,8 +915,8 @@ __device__ __forceinline__ void packed_words(const PassArgs& a, const PackedGeom
         packed_load<DIMS>(a, g, packed_place<DRAW>(g, (uint32_t)a.W, first));
     uint32_t A[kThresholds<DIMS, RULE>];
     __syncwarp();
-    packed_draws<DIMS, RULE, DRAW>(w.hbase, packed_both(a), a, (uint32_t)a.c, A);
-    packed_update<DIMS, MEASURE, RULE, DRAW>(a, w, A, packed_both(a), e_acc, m_acc);
+    packed_draws<DIMS, RULE, DRAW>(w.hbase, packed_second(a), a, (uint32_t)a.c, A);
+    packed_update<DIMS, MEASURE, RULE, DRAW>(a, w, A, packed_second(a), e_acc, m_acc);
 }
 
 }  // namespace ising

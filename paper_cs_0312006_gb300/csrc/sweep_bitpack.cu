@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
     constexpr uint32_t step = kWarpWords<draw>;
     const uint32_t items = geom.items, L = (uint32_t)a.L, W = (uint32_t)a.W;
     const uint32_t stride = ((gridDim.x * blockDim.x) >> 5) * step;
-    const bool both = WORDS == kWordsFull || packed_both(a);
+    const int second = WORDS == kWordsFull ? 4 : packed_second(a);
     auto place = [&](uint32_t first) {
         if constexpr (WORDS != kWordsFull) {
             return packed_place<draw>(geom, W, first);
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
     if (first < items) {
         uint32_t A[kThresholds<DIMS, RULE>];
         PackedPlace pl = place(first);
-        packed_draws<DIMS, RULE, draw>(pl.hbase, both, a, (uint32_t)a.c, A);
+        packed_draws<DIMS, RULE, draw>(pl.hbase, second, a, (uint32_t)a.c, A);
 #pragma unroll
         for (uint32_t& v : A) pin_here(v);
         constexpr int N = kThresholds<DIMS, RULE>;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
 #pragma unroll 1
             for (int m = 0; m < n_later; ++m) {
                 uint32_t B[N];
-                packed_draws<DIMS, RULE, draw>(pl.hbase, both, a,
+                packed_draws<DIMS, RULE, draw>(pl.hbase, second, a,
                                                (uint32_t)a.c + 2u * (uint32_t)(m + 1), B);
 #pragma unroll
                 for (int n = 0; n < N; ++n) later[(m * N + n) * 256] = B[n];
@@ -131,13 +131,13 @@ __global__ void __launch_bounds__(256, 3) pass_packed(PassArgs a, PackedGeom geo
         PackedWord w = load(pl);
         for (;;) {
             __syncwarp();
-            packed_update<DIMS, MEASURE, RULE, draw>(a, w, A, both, e_acc, m_acc, later, n_later);
+            packed_update<DIMS, MEASURE, RULE, draw>(a, w, A, second, e_acc, m_acc, later, n_later);
             first += stride;
             n_later = 0;
             if (first >= items) break;
             pl = place(first);
             w = load(pl);
-            packed_draws<DIMS, RULE, draw>(pl.hbase, both, a, (uint32_t)a.c, A);
+            packed_draws<DIMS, RULE, draw>(pl.hbase, second, a, (uint32_t)a.c, A);
         }
     } else {
         grid_dependency_wait();
