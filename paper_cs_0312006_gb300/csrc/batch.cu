@@ -166,41 +166,31 @@ __device__ __forceinline__ PassArgs job_args(const BatchJob& j, int c, uint32_t 
     return a;
 }
 
-// The int8 layout's pass of a job: not inlined, so that it does not add to the
-// registers of the packed one (ISING_AUTO's layout).
-template <int DIMS, bool MEASURE, int RULE>
-__device__ __noinline__ void job_pass_int8(const BatchJob& j, const PassArgs& a, uint32_t rank,
-                                           uint32_t nthr, int& e_acc, int& m_acc) {
-    const WordGeom g((uint32_t)j.W, (uint32_t)j.L, j.rows);
-    const uint32_t vecs = (j.half + 15u) >> 4;
-    if (j.W >= 64 && vecs >= nthr) {
-        for (uint32_t v = rank; v < vecs; v += nthr)
-            int8_vec<DIMS, MEASURE, RULE>(a, g, v, e_acc, m_acc);
-    } else if (j.W % 4 == 0 && RULE != kRuleMultiHit) {
-        // short rows of whole words: one uniform path for every word
-        const uint32_t words = j.half >> 2;
-        for (uint32_t w = rank; w < words; w += nthr)
-            int8_word_rows<DIMS, MEASURE, RULE>(a, g, w, e_acc, m_acc);
-    } else {  // short rows or few vectors: four sites per item spread further
-        const uint32_t words = (j.half + 3u) >> 2;
-        for (uint32_t w = rank; w < words; w += nthr)
-            int8_word<DIMS, MEASURE, RULE>(a, g, w, e_acc, m_acc);
-    }
-}
+// How a job's passes walk its colour arrays: the packed words of rows that start on
+// a Philox group or anywhere (packed_words), or, in int8, 16-site vectors, words of
+// rows of whole words, or words of any rows.
+constexpr int kBodyAligned = 0, kBodyRagged = 1, kBodyVectors = 2, kBodyRows = 3, kBodyWords = 4;
 
-template <int DIMS, int LAYOUT, bool MEASURE, int RULE>
-__device__ __forceinline__ void job_pass(const BatchJob& j, const PackedGeom& geom, int c,
-                                         uint32_t t, uint32_t rank, uint32_t nthr, int& e_acc,
-                                         int& m_acc) {
+// A thread's items of one colour pass.
+template <int DIMS, int BODY, bool MEASURE, int RULE, typename Geom>
+__device__ __forceinline__ void job_pass(const BatchJob& j, const Geom& geom, int c, uint32_t t,
+                                         uint32_t rank, uint32_t nthr, int& e_acc, int& m_acc) {
     const PassArgs a = job_args(j, c, t);
-    if (LAYOUT == ISING_INT8) {
-        job_pass_int8<DIMS, MEASURE, RULE>(j, a, rank, nthr, e_acc, m_acc);
+    if constexpr (BODY == kBodyAligned || BODY == kBodyRagged) {
+        constexpr int DRAW = BODY == kBodyAligned ? kDrawAligned : kDrawRagged;
+        constexpr uint32_t step = kWarpWords<DRAW>;
+        for (uint32_t w = (rank >> 5) * step; w < geom.items; w += (nthr >> 5) * step)
+            packed_words<DIMS, MEASURE, RULE, DRAW>(a, geom, w, e_acc, m_acc);
+    } else if constexpr (BODY == kBodyVectors) {
+        for (uint32_t v = rank; 16u * v < geom.half; v += nthr)
+            int8_vec<DIMS, MEASURE, RULE>(a, geom, v, e_acc, m_acc);
     } else {
-        // (one body for aligned and ragged rows: at half the code the kernels
-        // spill less and stay in the instruction cache)
-        constexpr uint32_t step = kWarpWords<kDrawRagged>;
-        for (uint32_t first = (rank >> 5) * step; first < geom.items; first += (nthr >> 5) * step)
-            packed_words<DIMS, MEASURE, RULE, kDrawRagged>(a, geom, first, e_acc, m_acc);
+        for (uint32_t w = rank; 4u * w < geom.half; w += nthr) {
+            if constexpr (BODY == kBodyRows)
+                int8_word_rows<DIMS, MEASURE, RULE>(a, geom, w, e_acc, m_acc);
+            else
+                int8_word<DIMS, MEASURE, RULE>(a, geom, w, e_acc, m_acc);
+        }
     }
 }
 
@@ -218,19 +208,27 @@ __device__ __forceinline__ void joint_chunk(const BatchJob& j, const PackedGeom&
     }
 }
 
-template <int DIMS, int LAYOUT, int MODE, int RULE>
-__device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader) {
+// All sweeps of a job.  Not inlined: the bodies of a kernel would otherwise share
+// one allocation of its 80 registers.  That, and the geometry's divisors worked out
+// once per job, took a pass of 64 lattices of 2D L = 32 from 1.7 to 0.77 us in int8 and
+// from 1.1 to 0.97 bit-packed, of 1024 of 2D L = 64 from 5.8 to 3.7 and 4.4 to 4.0.
+template <int DIMS, int BODY, int MODE, int RULE>
+__device__ __noinline__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader) {
     // (the passes of a cluster job are separated by the cluster barrier, whose
     // release/acquire at cluster scope makes the other CTAs' writes of the
     // previous pass visible to plain loads: 3 % faster on the 2048-lattice mix
     // than reading through L2 only)
-    const BatchJob j = *jp;
-    // in shared memory: the kernel runs at its register cap
-    __shared__ PackedGeom geom;
-    if (LAYOUT == ISING_BITPACK) {
-        if (threadIdx.x == 0) geom = PackedGeom((uint32_t)j.W, (uint32_t)j.L, j.rows);
-        __syncthreads();
+    using Geom = std::conditional_t<BODY <= kBodyRagged, PackedGeom, WordGeom>;
+    __shared__ BatchJob s_held;
+    __shared__ Geom geom;
+    if (threadIdx.x == 0) {
+        s_held = *jp;
+        geom = Geom((uint32_t)s_held.W, (uint32_t)s_held.L, s_held.rows);
     }
+    __syncthreads();
+    // the words' bodies hold the job in registers; the others, at the kernel's cap,
+    // read it pass by pass
+    std::conditional_t<(BODY >= kBodyRows), const BatchJob, const BatchJob&> j = s_held;
     int rec = 0;
     for (int s = 0; s < j.nsweeps; ++s) {
         const uint32_t t = j.t0 + (uint32_t)s;
@@ -238,9 +236,9 @@ __device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader)
         int e = 0, m = 0;
         for (int c = 0; c < 2; ++c) {
             if (measure)
-                job_pass<DIMS, LAYOUT, true, RULE>(j, geom, c, t, rank, nthr, e, m);
+                job_pass<DIMS, BODY, true, RULE>(j, geom, c, t, rank, nthr, e, m);
             else
-                job_pass<DIMS, LAYOUT, false, RULE>(j, geom, c, t, rank, nthr, e, m);
+                job_pass<DIMS, BODY, false, RULE>(j, geom, c, t, rank, nthr, e, m);
             group_sync<MODE>();  // this pass's writes before the next pass reads them
         }
         if (measure) {
@@ -255,20 +253,29 @@ __device__ void run_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader)
     }
 }
 
+template <int DIMS, int MODE, int RULE>
+__device__ void dispatch_body(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader) {
+    const int W = jp->W;
+    if (jp->layout == ISING_BITPACK) {
+        if (W % 4 == 0)
+            run_job<DIMS, kBodyAligned, MODE, RULE>(jp, rank, nthr, leader);
+        else
+            run_job<DIMS, kBodyRagged, MODE, RULE>(jp, rank, nthr, leader);
+    } else if ((W >= 64 || (W >= 16 && W % 4 != 0)) && (jp->half + 15u) >> 4 >= nthr) {
+        run_job<DIMS, kBodyVectors, MODE, RULE>(jp, rank, nthr, leader);
+    } else if (W % 4 == 0) {  // short rows of whole words: one uniform path for every word
+        run_job<DIMS, kBodyRows, MODE, RULE>(jp, rank, nthr, leader);
+    } else {  // short rows or few vectors: four sites per item spread further
+        run_job<DIMS, kBodyWords, MODE, RULE>(jp, rank, nthr, leader);
+    }
+}
+
 template <int MODE, int RULE>
 __device__ void dispatch_job(BatchJob* jp, uint32_t rank, uint32_t nthr, bool leader) {
-    const int dims = jp->dims, layout = jp->layout;
-    if (dims == 2) {
-        if (layout == ISING_BITPACK)
-            run_job<2, ISING_BITPACK, MODE, RULE>(jp, rank, nthr, leader);
-        else
-            run_job<2, ISING_INT8, MODE, RULE>(jp, rank, nthr, leader);
-    } else {
-        if (layout == ISING_BITPACK)
-            run_job<3, ISING_BITPACK, MODE, RULE>(jp, rank, nthr, leader);
-        else
-            run_job<3, ISING_INT8, MODE, RULE>(jp, rank, nthr, leader);
-    }
+    if (jp->dims == 2)
+        dispatch_body<2, MODE, RULE>(jp, rank, nthr, leader);
+    else
+        dispatch_body<3, MODE, RULE>(jp, rank, nthr, leader);
 }
 
 // counters[0] / counters[1]: next index into the large / small queue.  Every
@@ -532,28 +539,43 @@ void free_batch(ising_batch* b) {
 }
 
 // What a pass of a lattice costs, in us by its items (32-site words, 16-site
-// vectors) over a rate: run by a CTA that has an SM to itself (besides 0.9 us a
+// vectors) over a rate: run by a CTA that has an SM to itself (besides 0.6 us a
 // pass), as a share of a GPU full of such CTAs or clusters, and as a share of a
 // joint pass (besides its launch, `pass` us: the host's two launches a sweep, or
-// one wave of word-by-word rows).  The rates are those of batches of 1 to 1024
-// equal lattices, 2D L = 64 - 1024 and 3D L = 16 - 96, by the body that takes the
-// rows.
+// the time of one wave).  The rates are those of batches of 1 to 1024 equal
+// lattices, 2D L = 22 - 1024 and 3D L = 16 - 96, by the body that takes the rows.
 struct PassCost {
     double alone, queue, joint, pass;
 };
 PassCost pass_cost(const ising_lattice* h) {
-    double cta, queue, joint, pass = 2.9, items = (double)(h->half_sites + 15) / 16;
+    struct Rates {
+        double alone, queue, joint;
+    } r;
+    const bool flat = h->dims == 2, whole = h->W % 4 == 0;  // rows of whole draw groups
+    double pass = 2.9, items = (double)((h->half_sites + 15) / 16);
     if (h->layout == ISING_BITPACK) {
         items = (double)h->rows * (double)((h->W + 31) / 32);
-        cta = 200, queue = 35e3, joint = 28e3;
-    } else if (h->W >= 64) {
-        cta = 310, queue = 55e3, joint = 36e3;
-    } else if (h->W >= 16) {
-        cta = 155, queue = 29e3, joint = 24e3;
+        if (h->W <= 20)  // a word a row, some of its calls left out
+            r = whole ? Rates{330, 50e3, 39e3} : Rates{240, 42e3, 39e3};
+        else
+            r = whole ? Rates{230, 38e3, 28e3} : Rates{175, 32e3, 28e3};
+    } else if (h->W < 16) {  // joint passes take these word by word
+        r = whole ? Rates{180, 29e3, 9e3} : Rates{55, 11.5e3, 9e3};
+        pass = 7.0;
+    } else if (whole) {
+        if (h->W >= 64)
+            r = Rates{300, 57e3, 36e3};
+        else
+            r = flat ? Rates{250, 40e3, 32e3} : Rates{150, 29e3, 24e3};
+        if (!flat) pass = 4.0;
     } else {
-        cta = 170, queue = 23e3, joint = 9e3, pass = 7.0;
+        if (items < 256)  // too few vectors for a CTA: word by word in the queue
+            r = Rates{55, 11.5e3, flat ? 30e3 : 21e3};
+        else
+            r = flat ? Rates{200, 40e3, 30e3} : Rates{140, 31e3, 21e3};
+        pass = flat ? 3.4 : 4.0;
     }
-    return PassCost{items / cta, items / queue, items / joint, pass};
+    return PassCost{items / r.alone, items / r.queue, items / r.joint, pass};
 }
 
 // Which of `jobs` (one update rule's) take joint passes, when the caller names
@@ -564,14 +586,14 @@ PassCost pass_cost(const ising_lattice* h) {
 // passes' launches and work.  So a few small lattices stay with a CTA each, a
 // batch that fills the GPU with CTAs or clusters too, and what would leave it idle
 // goes jointly.  Us a pass, joint / queue (a CTA each, below 2^18 sites, clusters of
-// four above), bit-packed: 4 of 2D L = 64 2.8 / 1.1, 16 of L = 128 3.3 / 3.1, of L =
-// 192 3.4 / 5.5, of L = 512 5.2 / 10.5; 64 of L = 256 5.2 / 13.5; 256 of L = 256
-// 12.5 / 13.6, of L = 1024 146 / 116; 1024 of L = 64 5.2 / 4.4, of L = 256 38.5 /
-// 31.2; int8: 256 of L = 256 16.7 / 17.2, 1024 of it 57.1 / 37.6; 256 of 3D L = 16
-// 8.5 / 3.3.  Of 164 such batches the choice was the faster one or within 8 % of it
-// but once (four of 3D L = 24, 2.8 / 2.6).  Mixed sizes, ms: 256 lattices, 50 sweeps,
-// 3.5 jointly (3.7 with those below 2^12 sites queued), 8.2 queued; 2048, 100 sweeps,
-// 44.9 jointly, 37.9 queued, which is what the choice takes.
+// four above), bit-packed: 4 of 2D L = 64 3.1 / 1.2, 16 of L = 128 3.4 / 2.3, of L =
+// 256 3.4 / 8.3, of L = 512 5.3 / 13.0; 64 of L = 256 5.2 / 12.0; 256 of L = 256 13.1 /
+// 12.1, of L = 1024 149 / 130; 1024 of L = 64 5.4 / 4.0, of L = 256 39.3 / 27.6; int8:
+// 256 of L = 256 15.1 / 16.2, 1024 of it 56.3 / 37.1, 64 of L = 90 3.8 / 8.2; 256 of
+// 3D L = 16 8.6 / 2.1.  Of 312 such batches the choice was the faster one or within
+// 10 % of it in all but four (1.2 times in the worst: one of 2D L = 130, 3.4 / 2.8).
+// Mixed sizes, ms: 256 lattices, 50 sweeps, 3.6 jointly, 9.7 queued; 2048, 100
+// sweeps, 45 jointly, 38 queued, which is what the choice takes.
 void choose_joint(const ising_batch* b, std::vector<int>& jobs, std::vector<int>& joint) {
     struct Member {
         double chain, work, share, joint, pass, sweeps;  // us, of one pass each way
@@ -585,10 +607,10 @@ void choose_joint(const ising_batch* b, std::vector<int>& jobs, std::vector<int>
         const ising_lattice* h = b->lats[i];
         const PassCost c = pass_cost(h);
         const double n = (double)b->sweeps[i];
-        // a cluster of four takes its words 3.7 times as fast
+        // a cluster of four takes its words 3.3 times as fast
         const bool cluster = h->sites >= kClusterSites;
-        const double work = c.alone / (cluster ? 3.7 : 1.0);
-        ms.push_back(Member{n * (0.9 + work), n * work, n * c.queue, n * c.joint, c.pass, n, i,
+        const double work = c.alone / (cluster ? 3.3 : 1.0);
+        ms.push_back(Member{n * (0.6 + work), n * work, n * c.queue, n * c.joint, c.pass, n, i,
                             cluster ? kOpenCluster : 1});
         rest += ms.back().share;
         ctas += ms.back().ctas;
@@ -785,7 +807,7 @@ int assign_members(ising_batch* b, ising_lattice* const* lats, int n, const int6
         }
         cluster = big[0].empty() && big[1].empty() ? 1 : kOpenCluster;
     }
-    if (cluster != b->cluster) b->grid[0] = b->grid[1] = 0;
+    if (cluster != b->cluster) b->grid[0] = b->grid[1] = 0;  // resident CTAs of the other
     b->cluster = cluster;
     auto by_work = [&](int x, int y) {
         return b->lats[x]->sites * b->sweeps[x] > b->lats[y]->sites * b->sweeps[y];

@@ -901,7 +901,7 @@ __device__ __forceinline__ PackedWord packed_load(const PassArgs& a, const Packe
 
 // How many of a word's second four calls any of its sites needs: rows of one word
 // that start at most 3 draws into a group (2 where W is even, 0 where W % 4 == 0).
-// (64 of 3D L = 30 in a CTA each: 14.1 us a pass with eight calls, 9.8 with five.)
+// (64 of 3D L = 30 in a CTA each: 14.1 us a pass with eight calls, 10.0 with five.)
 __device__ __forceinline__ int packed_second(const PassArgs& a) {
     const int last = a.W + (a.W % 4 == 0 ? 0 : a.W % 2 == 0 ? 2 : 3);
     return last <= 16 ? 0 : last <= 20 ? 1 : 4;
