@@ -76,16 +76,16 @@ __device__ __forceinline__ Philox4 philox4x32_10_split(uint32_t c0, uint32_t c1,
     return Philox4{c0, c1, c2, c3};
 }
 
-// LEN * RUNS calls whose counter word 0 runs over RUNS sets of LEN
-// consecutive values (base[r] .. base[r] + LEN - 1, no 32-bit wrap), the other
+// 4 * RUNS calls whose counter word 0 runs over RUNS sets of four
+// consecutive values (base[r] .. base[r] + 3, no 32-bit wrap), the other
 // counter words and the key shared, advanced one round at a time so that a
 // caller can place other work between the rounds.  In the first round the
 // product of base + i is the product of base plus i times the multiplier (a
 // 64-bit add instead of a multiply).  result(w) equals philox4x32_10 of call
-// w's counter (base[w / LEN] + w % LEN, ctr1, ctr2, ctr3) under the same key.
-template <int RUNS, int LEN = 4>
+// w's counter (base[w / 4] + w % 4, ctr1, ctr2, ctr3) under the same key.
+template <int RUNS>
 struct PhiloxRuns {
-    static constexpr int N = LEN * RUNS;
+    static constexpr int N = 4 * RUNS;
     uint32_t c0[N], c1[N], c2[N], c3[N];
     uint32_t k0, k1;
 
@@ -97,8 +97,8 @@ struct PhiloxRuns {
         for (int r = 0; r < RUNS; ++r) {
             const uint64_t pa0 = (uint64_t)base[r] * kPhiloxMulA;
 #pragma unroll
-            for (int i = 0; i < LEN; ++i) {
-                const int w = LEN * r + i;
+            for (int i = 0; i < 4; ++i) {
+                const int w = 4 * r + i;
                 const uint64_t pa = pa0 + (uint64_t)i * kPhiloxMulA;
                 c0[w] = (uint32_t)(pb >> 32) ^ ctr1 ^ key0;
                 c1[w] = (uint32_t)pb;

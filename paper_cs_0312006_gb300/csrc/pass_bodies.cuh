@@ -681,8 +681,7 @@ __device__ __forceinline__ void word_tests(uint32_t g0, const PassArgs& a, uint3
 }
 
 // Each site's answer for the threshold of its own number of disagreeing
-// neighbours, from the answers A[n] for every threshold (site_threshold's
-// choice, 32 sites at once).
+// neighbours, from the answers A[n] for every threshold, 32 sites at once.
 template <int DIMS>
 __device__ __forceinline__ uint32_t choose_answer(const Counts& k, const uint32_t (&A)[DIMS]) {
     if constexpr (DIMS == 2) return (k.eq0 & A[1]) | (k.eq1 & A[0]);

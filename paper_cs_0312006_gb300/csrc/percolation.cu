@@ -911,9 +911,9 @@ cudaError_t launch_blocked(const perc_medium* m, const BlockedPlan& p, int launc
 }
 
 // Blocked growth from the seeded C and F[0] (which hold the same) to the
-// steady state; the cluster ends in both.  The host looks at the pass count
-// after a few launches at a time: passes run beyond the last that added a site
-// mean the steady state is reached.
+// steady state; the cluster ends in C (the launches go in even groups, or in
+// place).  The host looks at the pass count after each group: passes run beyond
+// the last that added a site mean the steady state is reached.
 int invade_blocked(perc_medium* m, int64_t* steps_out) {
     const BlockedPlan p = blocked_plan(m->g);
     const size_t stamp_bytes = sizeof(int) * 2 * (size_t)p.tg.nx * p.tg.ny;
@@ -1030,13 +1030,11 @@ int perc_invade(perc_medium* m, int source, int64_t site, perc_result* out) {
     if (m->mode == PERC_PASSES_AUTO && m->g.dims == 2) {
         const int rc = invade_blocked(m, &steps);
         if (rc != ISING_OK) return rc;
-    } else
-    // the graph: on GB300 it measured 4.6 us per pass at L = 16384
-    // (chained launches, eight CTAs per SM) against 8.5 us for the persistent
-    // launch (2 - 4 CTAs per SM; 12 us with one, 14 us with all that fit): the
-    // pass's own work needs the wide grid, and the grid barrier costs more than
-    // a chained graph node
-    if (m->mode == PERC_PASSES_PERSISTENT && m->coop_grid > 0) {
+    } else if (m->mode == PERC_PASSES_PERSISTENT && m->coop_grid > 0) {
+        // on request: at L = 16384 it measured 8.5 us per pass (2 - 4 CTAs per SM;
+        // 12 us with one, 14 us with all that fit) against the graph's 4.6 (chained
+        // launches, eight CTAs per SM): the pass's own work needs the wide grid, and
+        // the grid barrier costs more than a chained graph node
         unsigned char* cb = static_cast<unsigned char*>(m->coop);
         unsigned long long* cnt = reinterpret_cast<unsigned long long*>(cb);
         GridBar* gb = reinterpret_cast<GridBar*>(cb + kBandSlots * 8);
@@ -1063,48 +1061,48 @@ int perc_invade(perc_medium* m, int source, int64_t site, perc_result* out) {
         if (host_out.err) return ISING_ETIMEOUT;
         steps = (int64_t)host_out.steps;
     } else {
-    if (!m->passes) {
-        // eight CTAs per SM walk the band (grid-stride): at L = 16384 on GB300
-        // 4.6 us per pass, against 4.8 us with four, 6.4 us with two and 6.1 us
-        // with sixteen (most of whose CTAs find no band words and leave)
-        const unsigned cap8 = (unsigned)m->sm_count * 8u;
-        const unsigned pass_grid = grid < cap8 ? grid : cap8;
-        // capture [zero the counts, kPassesPerGraph banded passes] once; the
-        // buffers and slots it uses belong to the medium, so replays continue
-        cudaStream_t cap = nullptr;
-        PERC_CHECK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-        cudaGraph_t graph = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            cudaError_t le = cudaMemsetAsync(m->counts, 0, kPassesPerGraph * 8, cap);
-            for (int k = 0; k < kPassesPerGraph && le == cudaSuccess; ++k) {
-                // chained: a pass is placed on the SMs while the previous one drains
-                le = launch_chained(perc_band_kernel, pass_grid, 256u, 0, cap,
-                                    static_cast<const uint32_t*>(m->pore), m->C,
-                                    static_cast<const uint32_t*>(m->F[k & 1]),
-                                    m->F[(k & 1) ^ 1], m->g, m->bands, k, m->counts + k);
+        if (!m->passes) {
+            // eight CTAs per SM walk the band (grid-stride): at L = 16384 on GB300
+            // 4.6 us per pass, against 4.8 us with four, 6.4 us with two and 6.1 us
+            // with sixteen (most of whose CTAs find no band words and leave)
+            const unsigned cap8 = (unsigned)m->sm_count * 8u;
+            const unsigned pass_grid = grid < cap8 ? grid : cap8;
+            // capture [zero the counts, kPassesPerGraph banded passes] once; the
+            // buffers and slots it uses belong to the medium, so replays continue
+            cudaStream_t cap = nullptr;
+            PERC_CHECK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+            cudaGraph_t graph = nullptr;
+            cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+            if (e == cudaSuccess) {
+                cudaError_t le = cudaMemsetAsync(m->counts, 0, kPassesPerGraph * 8, cap);
+                for (int k = 0; k < kPassesPerGraph && le == cudaSuccess; ++k) {
+                    // chained: a pass is placed on the SMs while the previous one drains
+                    le = launch_chained(perc_band_kernel, pass_grid, 256u, 0, cap,
+                                        static_cast<const uint32_t*>(m->pore), m->C,
+                                        static_cast<const uint32_t*>(m->F[k & 1]),
+                                        m->F[(k & 1) ^ 1], m->g, m->bands, k, m->counts + k);
+                }
+                e = cudaStreamEndCapture(cap, &graph);
+                if (e == cudaSuccess) e = le;
             }
-            e = cudaStreamEndCapture(cap, &graph);
-            if (e == cudaSuccess) e = le;
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&m->passes, graph, 0);
+            if (graph) cudaGraphDestroy(graph);
+            cudaStreamDestroy(cap);
+            if (e != cudaSuccess) return cuda_fail(e);
         }
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&m->passes, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        cudaStreamDestroy(cap);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    // replay until a pass adds nothing (each replay that continues added at
-    // least kPassesPerGraph sites, so this ends)
-    unsigned long long host[kPassesPerGraph];
-    while (true) {
-        PERC_CHECK(cudaGraphLaunch(m->passes, m->stream));
-        PERC_CHECK(cudaMemcpyAsync(host, m->counts, sizeof(host), cudaMemcpyDeviceToHost,
-                                   m->stream));
-        PERC_CHECK(cudaStreamSynchronize(m->stream));
-        int k = 0;
-        while (k < kPassesPerGraph && host[k] != 0ull) ++k;
-        steps += k;
-        if (k < kPassesPerGraph) break;
-    }
+        // replay until a pass adds nothing (each replay that continues added at
+        // least kPassesPerGraph sites, so this ends)
+        unsigned long long host[kPassesPerGraph];
+        while (true) {
+            PERC_CHECK(cudaGraphLaunch(m->passes, m->stream));
+            PERC_CHECK(cudaMemcpyAsync(host, m->counts, sizeof(host), cudaMemcpyDeviceToHost,
+                                       m->stream));
+            PERC_CHECK(cudaStreamSynchronize(m->stream));
+            int k = 0;
+            while (k < kPassesPerGraph && host[k] != 0ull) ++k;
+            steps += k;
+            if (k < kPassesPerGraph) break;
+        }
     }
     PERC_CHECK(cudaMemsetAsync(m->meas, 0, 3 * 8, m->stream));
     perc_measure_kernel<<<grid, 256, 0, m->stream>>>(m->C, m->g, m->meas);
